@@ -109,7 +109,7 @@ struct InstRec {
     uint32_t nf, minfin, drain;   // formations done; next finishing formation; drain start
     uint16_t wmask;               // non-empty tier buckets
     uint8_t nrun, pc, phase;      // running requests; iteration-ended flag; nf mod T
-    uint8_t mrole, mpeer, pad;    // migration role and peer
+    uint8_t mrole, mpeer, mpend;  // migration role and peer; phase of a log record held back in mslot, or 0
 };
 static_assert(sizeof(InstRec) == 52, "InstRec is 13 words");
 
@@ -191,6 +191,7 @@ struct Ctx {
     MT_FIELD(uint8_t, phase);
     MT_FIELD(uint8_t, mrole);
     MT_FIELD(uint8_t, mpeer);
+    MT_FIELD(uint8_t, mpend);
     uint32_t *head, *tail, *hinfo;
     int *h;
     uint16_t *cnt;
@@ -208,12 +209,13 @@ struct Ctx {
     unsigned long long magT;
     int N, K, T, TH, Bmax, S, cap, lane, drains;
     uint32_t Q, t;
+    bool hold;                        // inside a window: log records are held back until it closes
 };
 
 // Counters.  Lane 0's copy carries the replica's totals; the other lanes'
 // copies collect what they add while advancing their own instances and are
-// folded into lane 0's when the warp leaves the replica (`finished` after
-// every window).
+// folded into lane 0's when the warp leaves the replica.  `finished` is the
+// replica's total on every lane; a status below 0 on any lane ends the run.
 struct Cnt {
     uint32_t finished, log_events, migrations, preemptions, starts, aborts, steps, iterations;
     uint32_t scale_out, scale_in;  // lane 0 only
@@ -337,6 +339,59 @@ __device__ __forceinline__ void log_ev(const Ctx &x, Cnt &cn, int kind, uint32_t
         reinterpret_cast<uint4 *>(x.log)[k] = w;
     }
 }
+// The record that ends the migration out of source s (phase 1: copy stage or
+// finish, phase 4: preemption in batch formation).  In a window the pairs of
+// migrating instances advance independently of one another, so the record is
+// held back in the source's slot copy, which nothing needs any more, and
+// flush_held writes the window's records in the order of time, phase and
+// instance.  A migration starts only at a tick, so a source has at most one.
+__device__ __forceinline__ void log_end(const Ctx &x, Cnt &cn, int kind, uint32_t r, int s, int d, int blocks, int ph) {
+    if (x.hold) {
+        x.mslot[s] = make_uint4(x.t, r, (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24),
+                                (uint32_t)kind);
+        x.mpend[s] = (uint8_t)ph;
+    } else {
+        log_ev(x, cn, kind, r, s, d, blocks);
+    }
+}
+// Closes a window with migrations: writes the records held back, and returns
+// whether some instance is still in a migration.  Collective.
+template <int C>
+__device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
+    uint32_t left = 0;
+    bool mig = false;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        const int i = x.lane * C + j;
+        if (i < x.N && x.mpend[i] != 0) left |= 1u << j;
+        if (i < x.N && x.mrole[i] != MIG_NONE) mig = true;
+    }
+    mig = __any_sync(kFull, mig);
+    while (__any_sync(kFull, left != 0)) {
+        uint32_t bt = kNone;
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+            if ((left >> j) & 1u) bt = min(bt, x.mslot[x.lane * C + j].x);
+        const uint32_t t = __reduce_min_sync(kFull, bt);
+        uint32_t bk = kNone;
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            const int i = x.lane * C + j;
+            if (((left >> j) & 1u) && x.mslot[i].x == t) bk = min(bk, ((uint32_t)x.mpend[i] << 16) | (uint32_t)i);
+        }
+        const int s = (int)(__reduce_min_sync(kFull, bk) & 0xFFFFu);
+        if (x.lane == s / C) {
+            left &= ~(1u << (s % C));
+            x.mpend[s] = 0;
+        }
+        if (x.lane == 0) {
+            const uint32_t k = cn.log_events++;
+            if (k < (uint32_t)x.cap) reinterpret_cast<uint4 *>(x.log)[k] = x.mslot[s];
+        }
+    }
+    __syncwarp();
+    return mig;
+}
 // The result record's last word holds n_preemptions (low half) and
 // n_migrations (high half), both modulo 2^16.  A migration adds 1 << 16: a
 // wrap carries out of the word, so nothing waits on the add.  A preemption
@@ -357,12 +412,12 @@ __device__ __forceinline__ void clear_mig(const Ctx &x, int s, int d) {
     x.mcopied[s] = 0;
 }
 // Abandon the staged copy out of source s: the destination releases what was copied.
-__device__ __forceinline__ void abort_mig(const Ctx &x, Cnt &cn, int s) {
+__device__ __forceinline__ void abort_mig(const Ctx &x, Cnt &cn, int s, int ph) {
     const int d = x.mpeer[s];
     const int cp = x.mcopied[s];
     x.free_[d] += cp;
     x.resv[d] -= cp;
-    log_ev(x, cn, SIM_EV_ABORT, x.mreq[s], s, d, cp);
+    log_end(x, cn, SIM_EV_ABORT, x.mreq[s], s, d, cp, ph);
     cn.aborts++;
     clear_mig(x, s, d);
 }
@@ -421,7 +476,7 @@ __device__ __forceinline__ void commit_book(const Ctx &x, Cnt &cn, int s, const 
     bump_mig(x, sl.x);
     cn.migrations++;
     cn.events++;
-    log_ev(x, cn, SIM_EV_COMMIT, sl.x, s, d, blocks);
+    log_end(x, cn, SIM_EV_COMMIT, sl.x, s, d, blocks, 1);
     clear_mig(x, s, d);
 }
 
@@ -462,7 +517,7 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
             if (x.lane == 0) {
                 cnt_dec(x, i, (int)(w & 0xFFu));
                 x.hist[i * x.TH + (w >> 16)]--;
-                if (x.mrole[i] == MIG_SRC && x.mreq[i] == rid) abort_mig(x, cn, i);
+                if (x.mrole[i] == MIG_SRC && x.mreq[i] == rid) abort_mig(x, cn, i, 1);
             }
         }
     }
@@ -474,30 +529,31 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
     __syncwarp();
     if (k0 && p0 != q0) p[p0] = a0;  // only the records that move are written
     if (k1 && p1 != q1) p[p1] = a1;
+    const uint32_t nfin = __popc(m0) + __popc(m1);
+    cn.finished += nfin;
     if (x.lane == 0) {
-        const uint32_t nfin = __popc(m0) + __popc(m1);
         x.free_[i] += freed;
         x.nrun[i] = (uint8_t)(__popc(e0) + __popc(e1));
         x.minfin[i] = fm;
-        cn.finished += nfin;
         cn.events += nfin;
     }
     __syncwarp();
 }
 
-// One copy stage at the end of an iteration of migration source s, whole
+// One copy stage at the end of an iteration of migration source s (nothing
+// to do if s is none, or if a finish has just abandoned its migration), whole
 // warp: up to S of the request's blocks are reserved on the destination
 // (abandoning the migration if they do not fit), and the request commits
 // there once all of them are copied (Sec. 3.5, Fig. 4).
 __device__ __forceinline__ void coop_stage(const Ctx &x, Cnt &cn, int s) {
     int commit = 0;
-    if (x.lane == 0) {
+    if (x.lane == 0 && x.mrole[s] == MIG_SRC) {
         const int d = x.mpeer[s];
         const int blocks = sl_blocks(x, s, x.mslot[s]);
         const int cp = x.mcopied[s];
         const int cc = min(x.S, blocks - cp);
         if (x.free_[d] < cc) {
-            abort_mig(x, cn, s);
+            abort_mig(x, cn, s, 1);
         } else {
             x.free_[d] -= cc;
             x.resv[d] += cc;
@@ -551,7 +607,7 @@ __device__ __forceinline__ unsigned int preempt_book(const Ctx &x, Cnt &cn, int 
     const unsigned int word = bump_pre(x, r);
     cn.preemptions++;
     cn.events++;
-    if (x.mrole[i] == MIG_SRC && x.mreq[i] == r) abort_mig(x, cn, i);
+    if (x.mrole[i] == MIG_SRC && x.mreq[i] == r) abort_mig(x, cn, i, 4);
     return word;  // for pre_fix, which the caller runs later so that nothing waits here
 }
 
@@ -886,9 +942,10 @@ __device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Para
     __syncwarp();
 }
 
-// Phase 3: periodic rebalancing between low- and high-freeness instances (Sec. 3.5).
+// Phase 3: periodic rebalancing between low- and high-freeness instances
+// (Sec. 3.5).  Returns whether a staged copy started.
 template <int C, bool EXT>
-__device__ __forceinline__ void migration_tick(const Ctx &x, Cnt &cn, int theta_num, int theta_den) {
+__device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_num, int theta_den) {
     refresh_keys<C>(x);
     uint32_t el = 0, dr = 0;  // eligible (not migrating); draining
 #pragma unroll
@@ -897,6 +954,7 @@ __device__ __forceinline__ void migration_tick(const Ctx &x, Cnt &cn, int theta_
         if (i < x.N && x.mrole[i] == MIG_NONE) el |= 1u << j;
         if (EXT && i < x.N && x.drains && x.drain[i] <= x.t) dr |= 1u << j;
     }
+    bool started = false;
     for (;;) {
         const int nel = __reduce_add_sync(kFull, __popc(el));
         if (nel < 2) break;
@@ -977,12 +1035,14 @@ __device__ __forceinline__ void migration_tick(const Ctx &x, Cnt &cn, int theta_
                     log_ev(x, cn, SIM_EV_START, rid, s, d, blocks);
                 }
                 moved = 1;
+                started = true;
             }
         }
         if (x.lane == s / C) el &= ~(1u << (s % C));
         if (moved && x.lane == d / C) el &= ~(1u << (d % C));
         __syncwarp();
     }
+    return started;
 }
 
 // Distinct event times of a window (C > 1): a per-warp open-addressing set.
@@ -1006,7 +1066,7 @@ __device__ __forceinline__ void bind_blob(Ctx &x, const Layout &L, unsigned char
     unsigned char *ib = blob + L.inst;
     x.busy.base = x.free_.base = x.resv.base = x.hol.base = x.hr.base = x.key.base = ib;
     x.mreq.base = x.mcopied.base = x.nf.base = x.minfin.base = x.drain.base = ib;
-    x.wmask.base = x.nrun.base = x.pc.base = x.phase.base = x.mrole.base = x.mpeer.base = ib;
+    x.wmask.base = x.nrun.base = x.pc.base = x.phase.base = x.mrole.base = x.mpeer.base = x.mpend.base = ib;
     x.cnt = reinterpret_cast<uint16_t *>(blob + L.cnt);
     x.head = reinterpret_cast<uint32_t *>(blob + L.head);
     x.tail = reinterpret_cast<uint32_t *>(blob + L.tail);
@@ -1034,9 +1094,9 @@ __device__ __forceinline__ void complete_all(const Ctx &x, Cnt &cn, uint32_t mas
             h &= h - 1;
             int fp = 0;
             if (x.lane == 0) fp = inst_complete_head(x, i);
+            const bool src = x.mrole[i] == MIG_SRC;
             if (__shfl_sync(kFull, fp, 0)) coop_finish(x, cn, i);
-            __syncwarp();
-            if (x.mrole[i] == MIG_SRC) coop_stage(x, cn, i);
+            if (src) coop_stage(x, cn, i);
         }
     }
 }
@@ -1070,6 +1130,53 @@ __device__ __forceinline__ uint32_t pick_c(const uint32_t (&a)[C], int j) {
     for (int k = 1; k < C; ++k)
         if (j == k) v = a[k];
     return v;
+}
+
+// The events of a window [tb, t1) that can be taken in the next round, bit j =
+// own instance lane*C + j, at time et[j].  A window is short enough that every
+// instance ends at most one iteration, and instances interact only as the two
+// ends of a migration: the source's event (finish, copy stage, commit or
+// abort) reads and changes the destination, the destination's event changes
+// nothing at the source.  So the instances outside migrations and the earlier
+// event of every pair are taken together, each at its own time (`first`), and
+// the later events of the pairs in a second round (`later`: there are some).
+// A pair whose two iterations end at the same time (`same`) is stepped as the
+// oracle orders one time: both ends, then both formations.  `wake_lo`,
+// `wake_hi`: idle destinations of a source in `first`, which may be able to
+// form a batch once the source's event is done, before the source forms its
+// own (lower index) or after it.
+template <int C>
+struct Window {
+    uint32_t first, same, wake_lo, wake_hi;
+    bool later;
+};
+template <int C>
+__device__ __forceinline__ Window<C> classify(const Ctx &x, uint32_t t1, uint32_t (&et)[C]) {
+    Window<C> w{0, 0, 0, 0, false};
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        const int i = x.lane * C + j;
+        if (i >= x.N) continue;
+        const int role = x.mrole[i];
+        if (et[j] < t1) {
+            if (role == MIG_NONE) {
+                w.first |= 1u << j;
+            } else {
+                const uint32_t pb = x.busy[x.mpeer[i]];
+                if (pb > et[j]) w.first |= 1u << j;
+                else if (pb < et[j]) w.later = true;
+                else w.same |= 1u << j;
+            }
+        } else if (role == MIG_DST && et[j] == kNone) {
+            const int s = x.mpeer[i];
+            const uint32_t pb = x.busy[s];
+            if (pb < t1) {
+                (i < s ? w.wake_lo : w.wake_hi) |= 1u << j;
+                et[j] = pb;
+            }
+        }
+    }
+    return w;
 }
 
 // Which main loop a variant runs.  The variants that keep running-request
@@ -1168,7 +1275,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
         cn.migrations = rs.migrations;
         cn.preemptions = l0 ? rs.preemptions : 0u;
         cn.starts = rs.starts;
-        cn.aborts = rs.aborts;
+        cn.aborts = l0 ? rs.aborts : 0u;
         cn.scale_out = rs.scale_out;
         cn.scale_in = rs.scale_in;
         cn.steps = 0;
@@ -1176,6 +1283,12 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
         cn.member_iterations = l0 ? rs.member_iterations : 0ull;
         cn.events = l0 ? rs.events : 0ull;
         cn.status = SIM_REPLICA_RUNNING;
+        x.hold = false;
+        // whether some instance may be in a migration (kept current: set by a tick
+        // that starts one, taken back when a window closes without any)
+        bool mig = false;
+        for (int i = lane; i < x.N; i += 32) mig = mig || x.mrole[i] != MIG_NONE;
+        mig = __any_sync(kFull, mig);
         uint32_t cursor = rs.cursor;
         uint32_t next_tick = rs.next_tick;
         ArrBuf ab;
@@ -1185,103 +1298,96 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
             const uint32_t max_steps = p.max_steps;
             const uint32_t all = own_mask<C>(x);
             const bool ticks = EXT ? p.ticks != 0 : p.enable_mig != 0;
-            // Every pass of the loop below is one of three modes, which share one
+            // Every pass of the loop below is one of four modes, which share one
             // copy of each phase (iteration ends; finishes and copy stages;
             // dispatch and tick; batch formation), so the hot loop stays small:
             //   0: a window [tb, t1) in which every instance ends at most one
-            //      iteration: each lane ends and re-forms its own instances that
-            //      are in no migration ("solo"), each at its own time;
-            //   1: one step, at the next time tc < t1, of the window's instances
-            //      in a migration (both ends of every migration), in time order;
+            //      iteration: each lane ends and re-forms its own instances, each
+            //      at its own time, the later events of migrating pairs in a
+            //      second pass (classify);
+            //   1: one step, at the next time tc < t1, of the window's pairs whose
+            //      two iterations end at the same time;
             //   2: one step at the next global event (arrival, tick), or near the
-            //      step limit, over all instances.
-            bool in_cm = false;              // mode-1 steps of the current window remain
-            uint32_t t1 = 0, cm = 0;         // window end; own instances stepped in mode 1
-            uint32_t ucount = 0, u = kNone;  // distinct event times of the window; own solo time (C = 1)
-            uint32_t tlast = 0;              // latest event time processed in the window
+            //      step limit, over all instances;
+            //   3: nothing left of mode 1: the window closes.
+            bool any_b = false, in_cm = false;  // second events / mode-1 steps of the window remain
+            uint32_t t1 = 0, cm = 0;            // window end; own instances stepped in mode 1
+            uint32_t ucount = 0;                // distinct event times of the window
             for (;;) {
                 int mode;
                 uint32_t et[C];      // event time of each own instance in this pass
                 uint32_t heads = 0;  // own instances whose iteration ends in this pass
+                uint32_t wake_lo = 0, wake_hi = 0;  // own idle instances to form in a window pass
+                bool any_wake = false;
                 uint32_t tstep = 0;  // step time (modes 1 and 2)
                 bool tick = false;
-                if (in_cm) {
+                if (in_cm && !any_b) {
                     uint32_t cb = kNone;
 #pragma unroll
                     for (int j = 0; j < C; ++j)
                         if ((cm >> j) & 1u) cb = min(cb, x.busy[lane * C + j]);
-                    const uint32_t tc = __reduce_min_sync(kFull, cb);
-                    if (tc >= t1) {  // the window is complete
-                        in_cm = false;
-                        cn.steps += ucount;
-                        tmax = max(tmax, tlast);
-                        cn.finished = __shfl_sync(kFull, cn.finished, 0);  // finishes are all counted on lane 0
-                        cn.status = __reduce_min_sync(kFull, cn.status);
-                        if (cn.status < 0) break;
-                        continue;
-                    }
-                    mode = 1;
-                    tstep = tc;
-                    tlast = max(tlast, tc);
+                    tstep = __reduce_min_sync(kFull, cb);
+                    mode = tstep < t1 ? 1 : 3;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
-                        et[j] = tc;
-                        if (((cm >> j) & 1u) && x.busy[lane * C + j] == tc) heads |= 1u << j;
+                        et[j] = tstep;
+                        if (mode == 1 && ((cm >> j) & 1u) && x.busy[lane * C + j] == tstep) heads |= 1u << j;
                     }
                 } else {
-                    if (cn.finished == x.Q) { cn.status = SIM_REPLICA_DONE; break; }
-                    if (cn.steps == max_steps) break;
-                    uint32_t bz[C];
+                    if (!any_b) {
+                        if (cn.finished == x.Q) { cn.status = SIM_REPLICA_DONE; break; }
+                        if (cn.steps == max_steps) break;
+                    }
                     uint32_t mb = kNone;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
                         const int i = lane * C + j;
-                        bz[j] = i < x.N ? x.busy[i] : kNone;
-                        mb = min(mb, bz[j]);
+                        et[j] = i < x.N ? x.busy[i] : kNone;
+                        mb = min(mb, et[j]);
                     }
-                    const uint32_t tb = __reduce_min_sync(kFull, mb);
-                    const uint32_t tg = ticks ? min(next_arr, next_tick) : next_arr;
-                    if (tb < tg && max_steps - cn.steps > (uint32_t)x.N) {
+                    uint32_t tb = 0, tg = kNone;
+                    if (!any_b) {
+                        tb = __reduce_min_sync(kFull, mb);
+                        tg = ticks ? min(next_arr, next_tick) : next_arr;
+                    }
+                    if (any_b || (tb < tg && max_steps - cn.steps > (uint32_t)x.N)) {
                         mode = 0;
+                        if (!any_b) {
                         t1 = (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
-                        // instances with an iteration end in the window: stepped with
-                        // the others of a migration in time order (cm), or alone
-                        // (solo).  A destination whose source's next event comes
-                        // strictly later (or after the window) is alone: only the
-                        // source's events (stages, commit, abort) touch the other
-                        // end, and those then follow the destination's own event,
-                        // as in the oracle's time order.
-                        cm = 0;
-                        uint32_t solo = 0;
-#pragma unroll
-                        for (int j = 0; j < C; ++j) {
-                            const int i = lane * C + j;
-                            et[j] = bz[j];
-                            if (bz[j] < t1) {
-                                const int role = x.mrole[i];
-                                if (role == MIG_NONE || (role == MIG_DST && x.busy[x.mpeer[i]] > bz[j])) solo |= 1u << j;
-                                else cm |= 1u << j;
-                            }
-                        }
-                        heads = solo;
-                        tlast = 0;
+                        // distinct event times of the window, and the latest
                         if (C == 1) {
-                            // distinct event times: one group per value of the solo times
-                            u = solo ? bz[0] : kNone;
+                            const uint32_t u = et[0] < t1 ? et[0] : kNone;
                             const uint32_t grp = __match_any_sync(kFull, u);
                             ucount = __popc(__ballot_sync(kFull, u != kNone && (__ffs(grp) - 1) == lane));
-                            if (solo) tlast = bz[0];
+                            if (u != kNone) tmax = max(tmax, u);
                         } else {
                             for (uint32_t q = (uint32_t)lane; q < kHashSlots; q += 32) tset[q] = kNone;
                             __syncwarp();
                             uint32_t fresh = 0;
 #pragma unroll
                             for (int j = 0; j < C; ++j) {
-                                if (!((solo >> j) & 1u)) continue;
-                                tlast = max(tlast, bz[j]);
-                                fresh += tset_insert(x, bz[j]);
+                                if (et[j] >= t1) continue;
+                                tmax = max(tmax, et[j]);
+                                fresh += tset_insert(x, et[j]);
                             }
                             ucount = __reduce_add_sync(kFull, fresh);
+                        }
+                        }
+                        if (!mig) {
+#pragma unroll
+                            for (int j = 0; j < C; ++j) heads |= (et[j] < t1 ? 1u : 0u) << j;
+                        } else {
+                            const Window<C> w = classify<C>(x, t1, et);
+                            heads = w.first;
+                            wake_lo = w.wake_lo;
+                            wake_hi = w.wake_hi;
+                            cm = w.same;
+                            const uint32_t any = __reduce_or_sync(kFull, (w.later ? 1u : 0u) | (cm != 0 ? 2u : 0u) |
+                                                                             ((wake_lo | wake_hi) != 0 ? 4u : 0u));
+                            any_wake = any & 4u;
+                            any_b = any & 1u;
+                            in_cm = any & 2u;
+                            x.hold = true;
                         }
                     } else {
                         mode = 2;
@@ -1293,34 +1399,32 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                         ++cn.steps;
 #pragma unroll
                         for (int j = 0; j < C; ++j) {
+                            if (et[j] == tstep) heads |= 1u << j;
                             et[j] = tstep;
-                            if (bz[j] == tstep) heads |= 1u << j;
                         }
                     }
                 }
                 // ---- 1. iteration ends: each lane ends its own instances' iterations ----
-                uint32_t fz = 0;  // own instances with a finishing request
+                uint32_t fz = 0;  // own instances with a finishing request (bits 0..C-1), sources (bits C..)
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
                     if (!((heads >> j) & 1u)) continue;
-                    x.t = et[j];
-                    if (inst_complete_head(x, lane * C + j)) fz |= 1u << j;
+                    const int i = lane * C + j;
+                    if (inst_complete_head(x, i)) fz |= 1u << j;
+                    if (mig && x.mrole[i] == MIG_SRC) fz |= 1u << (C + j);
                 }
                 __syncwarp();
                 // ---- finishes and copy stages, instance by instance in ascending
-                // order, by the whole warp (in mode 0 only finishes, which touch
-                // their own instance alone, so their order does not matter) ----
-                const uint32_t visit = mode == 0 ? fz : heads;
-                for (uint32_t fl = __ballot_sync(kFull, visit != 0); fl; fl &= fl - 1) {
+                // order, by the whole warp ----
+                for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
                     const int l = __ffs(fl) - 1;
-                    const uint32_t vl = C == 1 ? 1u : __shfl_sync(kFull, visit, l);
                     const uint32_t fzl = __shfl_sync(kFull, fz, l);
-                    for (uint32_t h = vl; h; h &= h - 1) {
+                    for (uint32_t h = (fzl | (fzl >> C)) & ((1u << C) - 1u); h; h &= h - 1) {
                         const int j = __ffs(h) - 1;
                         const int i = l * C + j;
                         x.t = __shfl_sync(kFull, pick_c<C>(et, j), l);
                         if ((fzl >> j) & 1u) coop_finish(x, cn, i);
-                        if (mode != 0 && x.mrole[i] == MIG_SRC) coop_stage(x, cn, i);
+                        if ((fzl >> (C + j)) & 1u) coop_stage(x, cn, i);
                     }
                 }
                 if (mode == 2) {
@@ -1330,16 +1434,16 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                         const uint32_t nt = next_tick + p.interval;
                         next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                         if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
-                        if (p.enable_mig) migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den);
+                        if (p.enable_mig) mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
                     }
                 }
-                // ---- 4. batch formation: in mode 0 every lane forms its own solo
+                // ---- 4. batch formation: in mode 0 every lane forms its own
                 // instances at their own times; otherwise the idle instances with
                 // work are formed on lane 0 in ascending order (their preemptions
                 // may abort migrations, whose log records are lane 0's) ----
                 uint32_t want = 0;
                 if (mode == 0) {
-                    want = heads;
+                    want = any_wake ? wake_lo : heads;
                 } else {
                     const uint32_t mask = mode == 1 ? cm : all;
 #pragma unroll
@@ -1348,7 +1452,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                         if (((mask >> j) & 1u) && x.busy[i] == kNone && (x.nrun[i] | x.wmask[i]) != 0) want |= 1u << j;
                     }
                 }
-                for (uint32_t fl = mode == 0 ? 1u : __ballot_sync(kFull, want != 0); fl; fl &= fl - 1) {
+                // (mode 0 with destinations to wake: three rounds, the lower wakes, the
+                // instances whose iterations ended, the higher wakes)
+                for (uint32_t fl = mode != 0 ? __ballot_sync(kFull, want != 0) : any_wake ? 7u : 1u; fl; fl &= fl - 1) {
                     const int l = __ffs(fl) - 1;
                     const uint32_t hl = mode == 0 ? want : (C == 1 ? 1u : __shfl_sync(kFull, want, l));
                     const int owner = mode == 0 ? lane : l;
@@ -1359,47 +1465,19 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                             inst_form(x, cn, owner * C + j, p.base, p.a, p.b);
                         }
                     }
+                    if (mode == 0) want = l == 0 ? heads : wake_hi;
                     __syncwarp();
                 }
                 // ---- step accounting ----
-                if (mode == 0) {
-                    if (__any_sync(kFull, cm != 0)) {
-                        // the window's instances in a migration next (both ends of
-                        // every migration, with or without an event of their own)
-#pragma unroll
-                        for (int j = 0; j < C; ++j) {
-                            const int i = lane * C + j;
-                            if (i < x.N && x.mrole[i] != MIG_NONE) cm |= 1u << j;
-                        }
-                        in_cm = true;
-                        continue;
-                    }
+                if (mode == 0 || mode == 3) {
+                    if (mode == 0 && (any_b || in_cm)) continue;
+                    // the window closes
+                    in_cm = false;
+                    x.hold = false;
+                    if (mig) mig = flush_held<C>(x, cn);
                     cn.steps += ucount;
-                    tmax = max(tmax, tlast);
-                    cn.finished = __shfl_sync(kFull, cn.finished, 0);
-                    cn.status = __reduce_min_sync(kFull, cn.status);
-                    if (cn.status < 0) break;
-                } else if (mode == 1) {
-                    if (C == 1) {
-                        ucount += __any_sync(kFull, u == tstep) ? 0u : 1u;
-                    } else {
-                        uint32_t f2 = 0;
-                        if (lane == 0) f2 = tset_insert(x, tstep);
-                        ucount += __shfl_sync(kFull, f2, 0);
-                    }
-                    cn.status = __reduce_min_sync(kFull, cn.status);  // also a solo lane's error of this window
-                    if (cn.status < 0) {
-                        in_cm = false;
-                        cn.steps += ucount;
-                        tmax = max(tmax, tlast);
-                        cn.finished = __shfl_sync(kFull, cn.finished, 0);
-                        break;
-                    }
-                } else {
-                    cn.finished = __shfl_sync(kFull, cn.finished, 0);
-                    cn.status = __shfl_sync(kFull, cn.status, 0);
-                    if (cn.status < 0) break;
                 }
+                if (__any_sync(kFull, cn.status < 0)) break;
             }
             __syncwarp();
         } else {
@@ -1423,99 +1501,107 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                     // ---- window [tb, t1): at most one iteration end per instance ----
                     const uint32_t t1 =
                         (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
-                    // instances with an iteration end in the window: stepped with the
-                    // others of a migration in time order (cm), or alone (solo).  A
-                    // destination whose source's next event comes strictly later is
-                    // alone: only the source's events (stages, commit, abort) touch
-                    // the other end, and those then follow the destination's own event.
-                    uint32_t cm = 0, solo = 0;
-#pragma unroll
-                    for (int j = 0; j < C; ++j) {
-                        const int i = lane * C + j;
-                        if (bz[j] < t1) {
-                            const int role = x.mrole[i];
-                            if (role == MIG_NONE || (role == MIG_DST && x.busy[x.mpeer[i]] > bz[j])) solo |= 1u << j;
-                            else cm |= 1u << j;
-                        }
-                    }
-                    if (C > 1) {
-                        for (uint32_t q = (uint32_t)lane; q < kHashSlots; q += 32) tset[q] = kNone;
-                        __syncwarp();
-                    }
-                    uint32_t fresh = 0;  // distinct event times this lane contributes (C > 1)
-                    uint32_t tlast = 0;  // latest event time processed in the window
-                    uint32_t fz = 0;     // this lane's instances with a finishing request
-#pragma unroll
-                    for (int j = 0; j < C; ++j) {
-                        if (!((solo >> j) & 1u)) continue;
-                        const int i = lane * C + j;
-                        x.t = bz[j];
-                        tlast = max(tlast, bz[j]);
-                        if (C > 1) fresh += tset_insert(x, bz[j]);
-                        if (inst_complete_head(x, i)) fz |= 1u << j;
-                    }
-                    // finishes, one instance at a time by the whole warp (they touch
-                    // only their own instance, so their order does not matter) ...
-                    for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
-                        const int l = __ffs(fl) - 1;
-                        for (uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, fz, l); h; h &= h - 1) {
-                            const int j = __ffs(h) - 1;
-                            x.t = __shfl_sync(kFull, bz[j], l);
-                            coop_finish(x, cn, l * C + j);
-                        }
-                    }
-                    // ... then every lane forms its instances' next batches together
-#pragma unroll
-                    for (int j = 0; j < C; ++j) {
-                        if (!((solo >> j) & 1u)) continue;
-                        x.t = bz[j];
-                        inst_form(x, cn, lane * C + j, p.base, p.a, p.b);
-                    }
-                    __syncwarp();
-                    uint32_t ucount, u = kNone;
+                    // distinct event times of the window, and the latest
+                    uint32_t ucount;
                     if (C == 1) {
-                        u = solo ? bz[0] : kNone;
+                        const uint32_t u = bz[0] < t1 ? bz[0] : kNone;
                         const uint32_t grp = __match_any_sync(kFull, u);
                         ucount = __popc(__ballot_sync(kFull, u != kNone && (__ffs(grp) - 1) == lane));
+                        if (u != kNone) tmax = max(tmax, u);
                     } else {
-                        ucount = __reduce_add_sync(kFull, fresh);
-                    }
-                    // instances in a migration (both ends, with or without an event
-                    // of their own in the window): steps in time order on lane 0
-                    if (__any_sync(kFull, cm != 0)) {
+                        for (uint32_t q = (uint32_t)lane; q < kHashSlots; q += 32) tset[q] = kNone;
+                        __syncwarp();
+                        uint32_t fresh = 0;
 #pragma unroll
                         for (int j = 0; j < C; ++j) {
-                            const int i = lane * C + j;
-                            if (i < x.N && x.mrole[i] != MIG_NONE) cm |= 1u << j;
+                            if (bz[j] >= t1) continue;
+                            tmax = max(tmax, bz[j]);
+                            fresh += tset_insert(x, bz[j]);
                         }
-                        for (;;) {
+                        ucount = __reduce_add_sync(kFull, fresh);
+                    }
+                    // The iterations of the own instances in `sel` end; finishes and copy
+                    // stages follow, one instance at a time by the whole warp (each
+                    // touches only its own pair, so their order does not matter).
+                    auto ends = [&](uint32_t sel, bool stages) {
+                        uint32_t fz = 0;  // own instances with a finishing request (bits 0..C-1), sources (bits C..)
+#pragma unroll
+                        for (int j = 0; j < C; ++j) {
+                            if (!((sel >> j) & 1u)) continue;
+                            const int i = lane * C + j;
+                            if (inst_complete_head(x, i)) fz |= 1u << j;
+                            if (stages && x.mrole[i] == MIG_SRC) fz |= 1u << (C + j);
+                        }
+                        __syncwarp();
+                        for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
+                            const int l = __ffs(fl) - 1;
+                            const uint32_t fzl = C == 1 && !stages ? 1u : __shfl_sync(kFull, fz, l);
+                            for (uint32_t h = (fzl | (stages ? fzl >> C : 0u)) & ((1u << C) - 1u); h; h &= h - 1) {
+                                const int j = __ffs(h) - 1;
+                                x.t = __shfl_sync(kFull, pick_c<C>(bz, j), l);
+                                if (!stages || ((fzl >> j) & 1u)) coop_finish(x, cn, l * C + j);
+                                if (stages && ((fzl >> (C + j)) & 1u)) coop_stage(x, cn, l * C + j);
+                            }
+                        }
+                    };
+                    // Every lane forms its own instances' next batches.
+                    auto forms = [&](uint32_t sel) {
+#pragma unroll
+                        for (int j = 0; j < C; ++j) {
+                            if (!((sel >> j) & 1u)) continue;
+                            x.t = bz[j];
+                            inst_form(x, cn, lane * C + j, p.base, p.a, p.b);
+                        }
+                        __syncwarp();
+                    };
+                    if (!mig) {
+                        uint32_t sel = 0;
+#pragma unroll
+                        for (int j = 0; j < C; ++j) sel |= (bz[j] < t1 ? 1u : 0u) << j;
+                        ends(sel, false);
+                        forms(sel);
+                    } else {
+                        x.hold = true;
+                        uint32_t same, any;
+                        do {
+                            const Window<C> w = classify<C>(x, t1, bz);
+                            any = __reduce_or_sync(kFull, (w.later ? 1u : 0u) | (w.same != 0 ? 2u : 0u) |
+                                                              ((w.wake_lo | w.wake_hi) != 0 ? 4u : 0u));
+                            same = w.same;
+                            ends(w.first, true);
+                            // idle destinations to wake form before or after the others, by index
+                            uint32_t sel = (any & 4u) ? w.wake_lo : w.first;
+#pragma unroll 1
+                            for (int sub = (any & 4u) ? 3 : 1;;) {
+                                forms(sel);
+                                if (--sub == 0) break;
+                                sel = sub == 2 ? w.first : w.wake_hi;
+                            }
+                            if (any & 1u) {
+#pragma unroll
+                                for (int j = 0; j < C; ++j)
+                                    bz[j] = lane * C + j < x.N ? x.busy[lane * C + j] : kNone;
+                            }
+                        } while (any & 1u);
+                        // pairs whose two iterations end at the same time: whole steps
+                        // in time order
+                        while (any & 2u) {
                             uint32_t cb = kNone;
 #pragma unroll
                             for (int j = 0; j < C; ++j)
-                                if ((cm >> j) & 1u) cb = min(cb, x.busy[lane * C + j]);
+                                if ((same >> j) & 1u) cb = min(cb, x.busy[lane * C + j]);
                             const uint32_t tc = __reduce_min_sync(kFull, cb);
                             if (tc >= t1) break;
                             x.t = tc;
-                            tlast = max(tlast, tc);
-                            complete_all<C>(x, cn, cm);
-                            form_all<C>(x, cn, cm, p);
-                            if (C == 1) {
-                                ucount += __any_sync(kFull, u == tc) ? 0u : 1u;
-                            } else {
-                                uint32_t f2 = 0;
-                                if (lane == 0) f2 = tset_insert(x, tc);
-                                ucount += __shfl_sync(kFull, f2, 0);
-                            }
-                            cn.status = __shfl_sync(kFull, cn.status, 0);
-                            if (cn.status < 0) break;
+                            complete_all<C>(x, cn, same);
+                            form_all<C>(x, cn, same, p);
+                            if (__any_sync(kFull, cn.status < 0)) break;
                         }
+                        x.hold = false;
+                        mig = flush_held<C>(x, cn);
                     }
                     cn.steps += ucount;
-                    tmax = max(tmax, tlast);  // x.t is set again before any further use
-                    cn.finished = __shfl_sync(kFull, cn.finished, 0);  // finishes are all counted on lane 0
-                    const int ws = __reduce_min_sync(kFull, cn.status);
-                    cn.status = ws;
-                    if (cn.status < 0) break;
+                    if (__any_sync(kFull, cn.status < 0)) break;
                     continue;
                 }
                 // ---- one step at the next event time (global events, or near the step limit) ----
@@ -1525,26 +1611,25 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                 x.t = tick ? next_tick : tc;
                 tmax = max(tmax, x.t);
                 ++cn.steps;
-                const uint32_t f1 = cn.finished;
                 if (tb == x.t) complete_all<C>(x, cn, all);  // 1. iteration ends
-                cn.finished = __shfl_sync(kFull, cn.finished, 0);
                 if (next_arr == x.t) dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
                 if (tick) {  // 3. auto-scaling signal and migration tick
                     const uint32_t nt = next_tick + p.interval;
                     next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                     if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
-                    if (p.enable_mig) migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den);
+                    if (p.enable_mig) mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
                 }
                 form_all<C>(x, cn, all, p);  // 4. batch formation
-                (void)f1;
-                cn.status = __shfl_sync(kFull, cn.status, 0);
-                if (cn.status < 0) break;
+                if (__any_sync(kFull, cn.status < 0)) break;
             }
             __syncwarp();
         }
-        // fold the other lanes' counters into lane 0's
+        // fold the other lanes' counters into lane 0's (status: DONE or RUNNING on
+        // every lane, or an error on some)
+        cn.status = __reduce_min_sync(kFull, cn.status);
         const uint32_t tfin = __reduce_max_sync(kFull, tmax);
         const uint32_t a_pre = __reduce_add_sync(kFull, l0 ? 0u : cn.preemptions);
+        const uint32_t a_ab = __reduce_add_sync(kFull, l0 ? 0u : cn.aborts);
         const uint32_t a_it = __reduce_add_sync(kFull, cn.iterations);
         uint64_t a_mi = cn.member_iterations, a_ev = cn.events;
 #pragma unroll
@@ -1571,7 +1656,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
             o2.migrations = cn.migrations;
             o2.preemptions = cn.preemptions + a_pre;
             o2.starts = cn.starts;
-            o2.aborts = cn.aborts;
+            o2.aborts = cn.aborts + a_ab;
             o2.scale_out = cn.scale_out;
             o2.scale_in = cn.scale_in;
             o2.status = cn.status;
