@@ -60,6 +60,10 @@
 #include <string>
 #include <vector>
 
+// A condition that rarely holds: its code is laid out away from the hot loop,
+// which several warps at different points share through the instruction cache.
+#define MT_RARE(c) (__builtin_expect(!!(c), 0))
+
 namespace mt {
 
 constexpr uint32_t kNone = 0xFFFFFFFFu;  // idle instance / no pending event / nil link
@@ -70,7 +74,9 @@ constexpr int kMagicShift = 40;          // floor(n / T) = (n * ceil(2^40 / T)) 
 constexpr int kWarpsPerBlock = 2;
 constexpr int kMaxBlockTokens = 64;      // T limit of the per-instance growth histogram
 constexpr uint32_t kMagicBytes = 528;    // ceil(2^64 / d) for d = 0..64, rounded up to 16 bytes
-constexpr uint32_t kHashSlots = 512;     // per-warp set of event times (C > 1 variants)
+// Bytes (2^n) of the per-warp scratch that counts a window's distinct event
+// times (distinct_times): small where many warps share an SM's shared memory.
+constexpr int kSetBitsShared = 12, kSetBits = 11;
 
 enum : int { MIG_NONE = 0, MIG_SRC = 1, MIG_DST = 2 };
 
@@ -130,8 +136,15 @@ struct Layout {
     uint32_t h;                                                          // [K] x 4 B
     uint32_t hist;                                                       // [N*TH] x 1 B
     uint32_t mslot;                                                      // [N] x 16 B
+    uint32_t tot;                                                        // [TOT_COUNT] x 4 B
     uint32_t bytes;
 };
+
+// A replica's rarely changing counters, kept with its instance state so that
+// they hold no registers: log records, migrations, preemptions, migration
+// starts and aborts, scale-out and scale-in signals.  Formations on several
+// lanes may add to TOT_PRE and TOT_ABORT at once; lane 0 alone adds to the others.
+enum : int { TOT_LOG = 0, TOT_MIG, TOT_PRE, TOT_START, TOT_ABORT, TOT_OUT, TOT_IN, TOT_COUNT };
 
 // Per-replica scalars persisted between sim_run calls.
 struct RepState {
@@ -154,7 +167,7 @@ struct Params {
     int drains;                   // a drain schedule is loaded
     unsigned long long lcm_lo, lcm_hi;  // lcm(1, ..., Bmax) as two 64-bit halves
     Layout L;
-    uint32_t hash_bytes;          // per-warp event-time set (C > 1 variants), else 0
+    int set_bits;                 // per-warp scratch of distinct_times, log2 of its bytes
     const long long *offsets;
     const uint32_t *drain_src;    // [R][N] drain start times, or NULL
     const uint32_t *arrival;
@@ -162,6 +175,7 @@ struct Params {
     const uint8_t *tier;
     uint4 *node;                  // queue node per request: next, info of next, prev, own info
     sim_request_result_t *res;
+    long long res_off;            // bytes from a request's queue node to its result record
     unsigned char *blobs;
     uint4 *slots;                 // [R][N][Bmax]
     RepState *rep;
@@ -198,28 +212,40 @@ struct Ctx {
     uint8_t *hist;
     uint4 *mslot;                     // record of the request a migration source is copying out
     uint4 *slots;
-    uint32_t *tset;                   // event-time set (C > 1)
+    uint32_t *tset;                   // scratch of distinct_times
     const unsigned long long *magic;  // [65]: ceil(2^64 / d) for d >= 2
+    uint32_t *tot;                    // TOT_* counters
+    uint4 *node;                      // the replica's queue nodes
+    int r;                            // the replica
+    unsigned long long magT;
+    int N, K, T, TH, Bmax, S, lane, drains, set_bits;
+    uint32_t Q, t;
+    bool hold;                        // inside a window: log records are held back until it closes
+
+    // Copies of kernel parameters (they hold no registers), and from them the
+    // first trace record of the replica, its result records and its log.
     const uint32_t *arrival;
     const uint16_t *plen, *olen;
     const uint8_t *tier;
-    uint4 *node;
-    sim_request_result_t *res;
-    sim_migration_event_t *log;
-    unsigned long long magT;
-    int N, K, T, TH, Bmax, S, cap, lane, drains;
-    uint32_t Q, t;
-    bool hold;                        // inside a window: log records are held back until it closes
+    const uint4 *node0;
+    sim_migration_event_t *log0;
+    long long res_off;
+    int cap;
+    __device__ __forceinline__ long long first() const { return node - node0; }
+    __device__ __forceinline__ sim_request_result_t *res(uint32_t q) const {
+        return reinterpret_cast<sim_request_result_t *>(reinterpret_cast<unsigned char *>(node + q) + res_off);
+    }
+    __device__ __forceinline__ uint4 *log(uint32_t k) const {
+        return reinterpret_cast<uint4 *>(log0) + (size_t)r * cap + k;
+    }
 };
 
-// Counters.  Lane 0's copy carries the replica's totals; the other lanes'
-// copies collect what they add while advancing their own instances and are
-// folded into lane 0's when the warp leaves the replica.  `finished` is the
-// replica's total on every lane; a status below 0 on any lane ends the run.
+// Counters of this launch.  `iterations` and `member_iterations` are summed over
+// the lanes when the warp leaves the replica; `finished` is the replica's total
+// on every lane; a status below 0 on any lane ends the run.
 struct Cnt {
-    uint32_t finished, log_events, migrations, preemptions, starts, aborts, steps, iterations;
-    uint32_t scale_out, scale_in;  // lane 0 only
-    uint64_t member_iterations, events;
+    uint32_t finished, steps, iterations;
+    uint64_t member_iterations;
     int status;
 };
 
@@ -329,15 +355,10 @@ __device__ __forceinline__ void refresh_hol(const Ctx &x, int i) {
     x.hol[i] = wm ? blocks_for(x, x.hinfo[i * x.K + (__ffs(wm) - 1)] & 0xFFFFu) : 0;
 }
 __device__ __forceinline__ void log_ev(const Ctx &x, Cnt &cn, int kind, uint32_t r, int s, int d, int blocks) {
-    const uint32_t k = cn.log_events++;
-    if (k < (uint32_t)x.cap) {
-        uint4 w;
-        w.x = x.t;
-        w.y = r;
-        w.z = (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24);
-        w.w = (uint32_t)kind;
-        reinterpret_cast<uint4 *>(x.log)[k] = w;
-    }
+    const uint32_t k = x.tot[TOT_LOG]++;
+    if (k < (uint32_t)x.cap)
+        *x.log(k) = make_uint4(x.t, r, (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24),
+                               (uint32_t)kind);
 }
 // The record that ends the migration out of source s (phase 1: copy stage or
 // finish, phase 4: preemption in batch formation).  In a window the pairs of
@@ -367,6 +388,7 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
         if (i < x.N && x.mrole[i] != MIG_NONE) mig = true;
     }
     mig = __any_sync(kFull, mig);
+#pragma unroll 1
     while (__any_sync(kFull, left != 0)) {
         uint32_t bt = kNone;
 #pragma unroll
@@ -385,8 +407,8 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
             x.mpend[s] = 0;
         }
         if (x.lane == 0) {
-            const uint32_t k = cn.log_events++;
-            if (k < (uint32_t)x.cap) reinterpret_cast<uint4 *>(x.log)[k] = x.mslot[s];
+            const uint32_t k = x.tot[TOT_LOG]++;
+            if (k < (uint32_t)x.cap) *x.log(k) = x.mslot[s];
         }
     }
     __syncwarp();
@@ -398,7 +420,7 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
 // adds 1 to the low half and gets the old word back; when the low half
 // wrapped, the carry into n_migrations is taken back (pre_fix).
 __device__ __forceinline__ unsigned int *count_word(const Ctx &x, uint32_t r) {
-    return reinterpret_cast<unsigned int *>(reinterpret_cast<unsigned char *>(x.res + r) + 12);
+    return reinterpret_cast<unsigned int *>(reinterpret_cast<unsigned char *>(x.res(r)) + 12);
 }
 __device__ __forceinline__ void bump_mig(const Ctx &x, uint32_t r) { atomicAdd(count_word(x, r), 1u << 16); }
 __device__ __forceinline__ unsigned int bump_pre(const Ctx &x, uint32_t r) { return atomicAdd(count_word(x, r), 1u); }
@@ -418,7 +440,7 @@ __device__ __forceinline__ void abort_mig(const Ctx &x, Cnt &cn, int s, int ph) 
     x.free_[d] += cp;
     x.resv[d] -= cp;
     log_end(x, cn, SIM_EV_ABORT, x.mreq[s], s, d, cp, ph);
-    cn.aborts++;
+    atomicAdd(&x.tot[TOT_ABORT], 1u);
     clear_mig(x, s, d);
 }
 
@@ -474,8 +496,7 @@ __device__ __forceinline__ void commit_book(const Ctx &x, Cnt &cn, int s, const 
     slot_join(x, d, nd, sl.x, sl_c(sl) + adv, sl_left(sl) - adv, tr);
     x.nrun[d] = (uint8_t)(nd + 1);
     bump_mig(x, sl.x);
-    cn.migrations++;
-    cn.events++;
+    x.tot[TOT_MIG]++;
     log_end(x, cn, SIM_EV_COMMIT, sl.x, s, d, blocks, 1);
     clear_mig(x, s, d);
 }
@@ -502,24 +523,21 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
     const uint4 a0 = v0 ? p[q0] : make_uint4(0, 0, 0, 0);
     const uint4 a1 = v1 ? p[q1] : make_uint4(0, 0, 0, 0);
     const bool f0 = v0 && sl_fin(a0) == nf, f1 = v1 && sl_fin(a1) == nf;
-    if (f0) { x.res[a0.x].finish_us = x.t; x.res[a0.x].final_instance = (uint16_t)i; }
-    if (f1) { x.res[a1.x].finish_us = x.t; x.res[a1.x].final_instance = (uint16_t)i; }
+    if (f0) { x.res(a0.x)->finish_us = x.t; x.res(a0.x)->final_instance = (uint16_t)i; }
+    if (f1) { x.res(a1.x)->finish_us = x.t; x.res(a1.x)->final_instance = (uint16_t)i; }
     const int freed = __reduce_add_sync(kFull, (f0 ? sl_blocks(x, i, a0) : 0) + (f1 ? sl_blocks(x, i, a1) : 0));
     const uint32_t m0 = __ballot_sync(kFull, f0), m1 = __ballot_sync(kFull, f1);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        uint32_t lanes = j ? m1 : m0;
-        while (lanes) {
-            const int l = __ffs(lanes) - 1;
-            lanes &= lanes - 1;
-            const uint32_t rid = __shfl_sync(kFull, j ? a1.x : a0.x, l);
-            const uint32_t w = __shfl_sync(kFull, j ? a1.w : a0.w, l);
-            if (x.lane == 0) {
-                cnt_dec(x, i, (int)(w & 0xFFu));
-                x.hist[i * x.TH + (w >> 16)]--;
-                if (x.mrole[i] == MIG_SRC && x.mreq[i] == rid) abort_mig(x, cn, i, 1);
-            }
+    // each finishing request is booked by the lane that holds it, in turn
+#pragma unroll 1
+    for (uint64_t m = ((uint64_t)m1 << 32) | m0; m; m &= m - 1) {
+        const int l = __ffsll((long long)m) - 1;
+        if (x.lane == (l & 31)) {
+            const uint32_t rid = l & 32 ? a1.x : a0.x, w = l & 32 ? a1.w : a0.w;
+            cnt_dec(x, i, (int)(w & 0xFFu));
+            x.hist[i * x.TH + (w >> 16)]--;
+            if (MT_RARE(x.mrole[i] == MIG_SRC && x.mreq[i] == rid)) abort_mig(x, cn, i, 1);
         }
+        __syncwarp();
     }
     const bool k0 = v0 && !f0, k1 = v1 && !f1;
     const uint32_t e0 = __ballot_sync(kFull, k0), e1 = __ballot_sync(kFull, k1);
@@ -535,7 +553,6 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
         x.free_[i] += freed;
         x.nrun[i] = (uint8_t)(__popc(e0) + __popc(e1));
         x.minfin[i] = fm;
-        cn.events += nfin;
     }
     __syncwarp();
 }
@@ -552,7 +569,7 @@ __device__ __forceinline__ void coop_stage(const Ctx &x, Cnt &cn, int s) {
         const int blocks = sl_blocks(x, s, x.mslot[s]);
         const int cp = x.mcopied[s];
         const int cc = min(x.S, blocks - cp);
-        if (x.free_[d] < cc) {
+        if (MT_RARE(x.free_[d] < cc)) {
             abort_mig(x, cn, s, 1);
         } else {
             x.free_[d] -= cc;
@@ -576,7 +593,7 @@ __device__ __forceinline__ void coop_stage(const Ctx &x, Cnt &cn, int s) {
         const uint32_t h0 = __ballot_sync(kFull, v0 && a0.x == rid);
         const uint32_t h1 = __ballot_sync(kFull, v1 && a1.x == rid);
         const int pos = h0 ? __ffs(h0) - 1 : (h1 ? 32 + __ffs(h1) - 1 : -1);
-        if (pos < 0) {
+        if (MT_RARE(pos < 0)) {
             if (x.lane == 0) cn.status = SIM_ERR_INTERNAL;
         } else {
             const uint4 sl = p[pos];
@@ -605,8 +622,7 @@ __device__ __forceinline__ unsigned int preempt_book(const Ctx &x, Cnt &cn, int 
     if ((old & ((1u << tr) - 1u)) == 0) x.hol[i] = blocks_for(x, sl_c(sl) + adv);  // now head of line
     x.hist[i * x.TH + sl_rho(sl)]--;
     const unsigned int word = bump_pre(x, r);
-    cn.preemptions++;
-    cn.events++;
+    atomicAdd(&x.tot[TOT_PRE], 1u);
     if (x.mrole[i] == MIG_SRC && x.mreq[i] == r) abort_mig(x, cn, i, 4);
     return word;  // for pre_fix, which the caller runs later so that nothing waits here
 }
@@ -626,7 +642,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
     int need = x.hol[i];
     if (n > 0) {
         const int deficit = x.hist[i * x.TH + (ph == 0 ? 0u : (uint32_t)x.T - ph)];
-        if (deficit <= fr) {
+        if (!MT_RARE(deficit > fr)) {
             fr -= deficit;  // every request that needs a block gets it
         } else {
             x.free_[i] = fr;
@@ -654,6 +670,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
             int fb = fr;
             uint32_t pr = kNone;  // the last preempted request and its counter word before the add
             unsigned int pold = 0;
+#pragma unroll 1
             for (int q = 0; q < n; ++q) {
                 if (!((alive & needs) >> q & 1ull)) continue;
                 for (;;) {
@@ -663,6 +680,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
                         v = v1;  // nobody preempted yet: the victim found by the scan
                     } else {
                         uint32_t vt = 0, vr = 0;
+#pragma unroll 1
                         for (uint64_t m = alive; m; m &= m - 1) {
                             const int s2 = __ffsll((long long)m) - 1;
                             const uint32_t ts = sl_tier(p[s2]), rs = p[s2].x;
@@ -682,6 +700,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
             x.free_[i] = fb;
             int w = 0;
             uint32_t fm = kNone;  // the survivors' next finishing formation
+#pragma unroll 1
             for (int q = 0; q < n; ++q) {
                 if ((alive >> q) & 1ull) {
                     const uint4 sl = p[q];
@@ -702,6 +721,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
     // (ii) admission; the waiting mask and the HoL demand follow in registers
     const int n_decode = n;
     int prefill = 0;
+#pragma unroll 1
     while (n < x.Bmax) {
         if (!wm) break;
         if (need > fr) break;
@@ -709,7 +729,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
         const int b = i * x.K + k;
         const uint32_t info = x.hinfo[b];
         const uint32_t r = x.head[b];
-        if (r >= x.Q) { cn.status = SIM_ERR_INTERNAL; break; }
+        if (MT_RARE(r >= x.Q)) { cn.status = SIM_ERR_INTERNAL; break; }
         const uint4 nd = x.node[r];  // the head leaves its bucket; nd.x is the new head
         x.head[b] = nd.x;
         const uint32_t c = info & 0xFFFFu;
@@ -736,13 +756,14 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
     // (iii) the iteration starts
     if (n > 0) {
         const long long end = (long long)x.t + base + (long long)a_us * prefill + (long long)b_us * n_decode;
-        if (end > 0xFFFFFFFELL) {
+        if (MT_RARE(end > 0xFFFFFFFELL)) {
             cn.status = SIM_ERR_OVERFLOW;
             return;
         }
         x.busy[i] = (uint32_t)end;
         const uint4 *sp = slot_ptr(x, i, 0);
-        for (int q = n_decode; q < n; ++q) atomicMin(&x.res[sp[q].x].first_token_us, (uint32_t)end);
+#pragma unroll 1
+        for (int q = n_decode; q < n; ++q) atomicMin(&x.res(sp[q].x)->first_token_us, (uint32_t)end);
         x.nf[i] = nf + 1u;
         x.phase[i] = ph + 1u == (uint32_t)x.T ? (uint8_t)0 : (uint8_t)(ph + 1u);
         x.pc[i] = 0;
@@ -777,8 +798,7 @@ __device__ __forceinline__ void dispatch_to(const Ctx &x, Cnt &cn, int best, uin
         x.cnt[b] = (uint16_t)(c0 + 1u);
         if (c0 == 0) x.hr[best] = hr += hk;                    // tier k now present (Eq. 4)
         if ((old & ((2u << k) - 1u)) == 0) x.hol[best] = hol = blocks_for(x, P);  // becomes head of line
-        x.res[r].dispatch_instance = (uint16_t)best;
-        cn.events++;
+        x.res(r)->dispatch_instance = (uint16_t)best;
         if (store_key) x.key[best] = make_key(x, fr - hol - hr, nr);
     }
 }
@@ -794,23 +814,24 @@ __device__ __forceinline__ void dispatch_one(const Ctx &x, Cnt &cn, uint32_t r, 
 
 // The next 32 trace records, one per lane: index pb + lane.
 struct ArrBuf {
-    uint32_t pb, time, tier, P, O;
+    uint32_t pb, time, tier, po;  // po: prompt length | output length << 16
 };
 
 __device__ __forceinline__ void arr_refill(const Ctx &x, ArrBuf &ab, uint32_t cursor) {
     ab.pb = cursor;
     const uint32_t idx = cursor + (uint32_t)x.lane;
     const bool in = idx < x.Q;
-    ab.time = in ? x.arrival[idx] : kNone;
-    ab.tier = in ? (uint32_t)x.tier[idx] : 0u;
-    ab.P = in ? (uint32_t)x.plen[idx] : 0u;
-    ab.O = in ? (uint32_t)x.olen[idx] : 0u;
+    const long long at = x.first() + idx;
+    ab.time = in ? x.arrival[at] : kNone;
+    ab.tier = in ? (uint32_t)x.tier[at] : 0u;
+    ab.po = in ? (uint32_t)x.plen[at] | ((uint32_t)x.olen[at] << 16) : 0u;
 }
 
 // Phase 2: arrivals at t, tier 0 first, FCFS (trace order) within a tier.
-// EXT: draining instances may exist.
+// EXT: draining instances may exist.  Returns the destination of a lone
+// arrival, or -1 after several.
 template <int C, bool EXT>
-__device__ __forceinline__ void dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &cursor, uint32_t &next_arr,
+__device__ __forceinline__ int dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &cursor, uint32_t &next_arr,
                                                ArrBuf &ab) {
     uint32_t all = own_mask<C>(x);
     if (EXT && x.drains) {
@@ -823,18 +844,19 @@ __device__ __forceinline__ void dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &
             if (((all >> j) & 1u) && x.drain[x.lane * C + j] > x.t) live |= 1u << j;
         if (__any_sync(kFull, live != 0)) all = live;
     }
+    int dest = -1;
     const uint32_t off = cursor - ab.pb;
     uint32_t eq = __ballot_sync(kFull, (uint32_t)x.lane >= off && ab.time == x.t);
-    if ((eq >> 31) && off > 0) {
+    if (MT_RARE((eq >> 31) && off > 0)) {
         // the run of arrivals at t may continue past the buffer: realign it on the cursor
         arr_refill(x, ab, cursor);
         eq = __ballot_sync(kFull, ab.time == x.t);
     }
-    if (eq != kFull && (eq & (eq - 1u)) == 0u) {
+    if (!MT_RARE(eq == kFull || (eq & (eq - 1u)) != 0u)) {
         // one arrival at t (the usual case): no tier ordering to do
         const int l = __ffs(eq) - 1;
         const uint32_t k1 = __shfl_sync(kFull, ab.tier, l);
-        const uint32_t po = __shfl_sync(kFull, ab.P | (ab.O << 16), l);
+        const uint32_t po = __shfl_sync(kFull, ab.po, l);
         // the freest instance from keys computed in registers (nothing reads
         // the key array before the next refresh)
         int bv = INT_MIN, bi = -1;
@@ -850,20 +872,23 @@ __device__ __forceinline__ void dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &
         const int best = __reduce_min_sync(kFull, (bi >= 0 && bv == m) ? bi : INT_MAX);
         dispatch_to(x, cn, best, ab.pb + (uint32_t)l, (int)k1, po & 0xFFFFu, po >> 16, false);
         __syncwarp();
+        dest = best;
         cursor += 1u;
     } else if (eq != kFull) {
         refresh_keys<C>(x);
         const bool mine = (eq >> x.lane) & 1u;
         uint32_t tm = __reduce_or_sync(kFull, mine ? (1u << ab.tier) : 0u);
+#pragma unroll 1
         while (tm) {
             const int k = __ffs(tm) - 1;
             tm &= tm - 1;
             uint32_t bits = __ballot_sync(kFull, mine && ab.tier == (uint32_t)k);
+#pragma unroll 1
             while (bits) {
                 const int l = __ffs(bits) - 1;
                 bits &= bits - 1;
-                dispatch_one<C>(x, cn, ab.pb + (uint32_t)l, k, __shfl_sync(kFull, ab.P, l),
-                                __shfl_sync(kFull, ab.O, l), all);
+                const uint32_t po = __shfl_sync(kFull, ab.po, l);
+                dispatch_one<C>(x, cn, ab.pb + (uint32_t)l, k, po & 0xFFFFu, po >> 16, all);
             }
         }
         cursor += (uint32_t)__popc(eq);
@@ -871,22 +896,27 @@ __device__ __forceinline__ void dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &
         // 32 or more arrivals share this time (the buffer starts at the cursor):
         // count them, then go tier by tier from the trace.
         refresh_keys<C>(x);
+        const long long at = x.first();
         uint32_t m = 32;
+#pragma unroll 1
         for (;;) {
             const uint32_t j2 = cursor + m + (uint32_t)x.lane;
             const bool in2 = j2 < x.Q;
-            const uint32_t e2 = __ballot_sync(kFull, in2 && x.arrival[j2] == x.t);
+            const uint32_t e2 = __ballot_sync(kFull, in2 && x.arrival[at + j2] == x.t);
             m += (uint32_t)__popc(e2);
             if (e2 != kFull) break;
         }
+#pragma unroll 1
         for (int k = 0; k < x.K; ++k) {
+#pragma unroll 1
             for (uint32_t base = 0; base < m; base += 32) {
                 const uint32_t j2 = cursor + base + (uint32_t)x.lane;
                 const bool mine = base + (uint32_t)x.lane < m;
-                const uint32_t tr = mine ? x.tier[j2] : 0u;
-                const uint32_t P = mine ? x.plen[j2] : 0u;
-                const uint32_t O = mine ? x.olen[j2] : 0u;
+                const uint32_t tr = mine ? x.tier[at + j2] : 0u;
+                const uint32_t P = mine ? x.plen[at + j2] : 0u;
+                const uint32_t O = mine ? x.olen[at + j2] : 0u;
                 uint32_t bits = __ballot_sync(kFull, mine && tr == (uint32_t)k);
+#pragma unroll 1
                 while (bits) {
                     const int l = __ffs(bits) - 1;
                     bits &= bits - 1;
@@ -897,8 +927,9 @@ __device__ __forceinline__ void dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &
         }
         cursor += m;
     }
-    if (cursor - ab.pb >= 32u) arr_refill(x, ab, cursor);
+    if (MT_RARE(cursor - ab.pb >= 32u)) arr_refill(x, ab, cursor);
     next_arr = __shfl_sync(kFull, ab.time, (int)(cursor - ab.pb));
+    return dest;
 }
 
 // Auto-scaling signal at a tick (Sec. 3.6): the mean normal-priority freeness
@@ -932,10 +963,10 @@ __device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Para
     if (x.lane == 0 && n > 0) {
         const __int128 lhs = sum * p.scale_den;
         if (lhs < (__int128)p.scale_out_num * n * L) {
-            cn.scale_out++;
+            x.tot[TOT_OUT]++;
             log_ev(x, cn, SIM_EV_SCALE_OUT, kNone, 255, 255, 0);
         } else if (lhs > (__int128)p.scale_in_num * n * L) {
-            cn.scale_in++;
+            x.tot[TOT_IN]++;
             log_ev(x, cn, SIM_EV_SCALE_IN, kNone, 255, 255, 0);
         }
     }
@@ -995,8 +1026,7 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
                     cnt_inc(x, d, k);
                     if ((old & ((2u << k) - 1u)) == 0) x.hol[d] = blocks_for(x, info & 0xFFFFu);
                     bump_mig(x, r);
-                    cn.migrations++;
-                    cn.events++;
+                    x.tot[TOT_MIG]++;
                     log_ev(x, cn, SIM_EV_QUEUED, r, s, d, 0);
                 }
             }
@@ -1031,7 +1061,7 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
                     x.mslot[s] = rec;
                     x.mrole[d] = MIG_DST;
                     x.mpeer[d] = (uint8_t)s;
-                    cn.starts++;
+                    x.tot[TOT_START]++;
                     log_ev(x, cn, SIM_EV_START, rid, s, d, blocks);
                 }
                 moved = 1;
@@ -1045,19 +1075,61 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
     return started;
 }
 
-// Distinct event times of a window (C > 1): a per-warp open-addressing set.
-__device__ __forceinline__ uint32_t tset_insert(const Ctx &x, uint32_t t) {
-    uint32_t h = (t * 0x9E3779B1u) >> 23;  // 9 bits: kHashSlots = 512
-    for (uint32_t probe = 0; probe < kHashSlots; ++probe) {
-        const uint32_t old = atomicCAS(&x.tset[h], kNone, t);
-        if (old == kNone) return 1u;
-        if (old == t) return 0u;
-        h = (h + 1u) & (kHashSlots - 1u);
+// The number of distinct times et[j] < t1 over the warp, for a window
+// [tb, t1).  Collective.  Every instance writes its index into a byte that its
+// time selects and reads it back: one index per byte wins and counts, nothing
+// needs clearing.  When the scratch has a byte for every microsecond of the
+// window the others have the winner's time; in a longer window the byte is
+// hashed, the winner's time is compared, and the instances that met another
+// time try again without the winners (at least one per byte leaves each round).
+template <int C>
+__device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, uint32_t t1, const uint32_t (&et)[C]) {
+    uint8_t *set = reinterpret_cast<uint8_t *>(x.tset);
+    uint32_t fresh = 0;
+    if (!MT_RARE(t1 - tb > 1u << x.set_bits)) {
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+            if (et[j] < t1) set[et[j] - tb] = (uint8_t)(x.lane * C + j);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < C; ++j)
+            if (et[j] < t1) fresh += set[et[j] - tb] == (uint8_t)(x.lane * C + j) ? 1u : 0u;
+    } else {
+        uint32_t todo = 0, at[C], win[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            todo |= (et[j] < t1 ? 1u : 0u) << j;
+            at[j] = ((et[j] - tb) * 0x9E3779B1u) >> (32 - x.set_bits);
+        }
+#pragma unroll 1
+        while (__any_sync(kFull, todo != 0)) {
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                if ((todo >> j) & 1u) set[at[j]] = (uint8_t)(x.lane * C + j);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                win[j] = ((todo >> j) & 1u) ? set[at[j]] : 0u;
+                if (((todo >> j) & 1u) && win[j] == (uint32_t)(x.lane * C + j)) {
+                    ++fresh;
+                    todo &= ~(1u << j);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+#pragma unroll
+                for (int k = 0; k < C; ++k) {  // instance win[j] is number k of its lane
+                    const uint32_t tw = __shfl_sync(kFull, et[k], (int)(win[j] / C));
+                    if (win[j] % C == (uint32_t)k && tw == et[j]) todo &= ~(1u << j);
+                }
+        }
     }
-    return 0u;
+    if (C == 1) return __popc(__ballot_sync(kFull, fresh != 0));
+    return __reduce_add_sync(kFull, fresh);
 }
 
 __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *src, uint32_t bytes, int lane) {
+#pragma unroll 1
     for (uint32_t o = (uint32_t)lane * 16u; o < bytes; o += 512u)
         *reinterpret_cast<uint4 *>(dst + o) = *reinterpret_cast<const uint4 *>(src + o);
 }
@@ -1074,6 +1146,7 @@ __device__ __forceinline__ void bind_blob(Ctx &x, const Layout &L, unsigned char
     x.h = reinterpret_cast<int *>(blob + L.h);
     x.hist = blob + L.hist;
     x.mslot = reinterpret_cast<uint4 *>(blob + L.mslot);
+    x.tot = reinterpret_cast<uint32_t *>(blob + L.tot);
 }
 
 // Phase 1 at x.t for the instances in `mask` (bit j = instance lane*C + j)
@@ -1202,15 +1275,16 @@ constexpr bool kUnifiedLoop = !SMS && C <= 2;
 // order.  EXT: the variant that also handles draining instances and
 // the auto-scaling signal (the other variant compiles that code out).
 template <int C, bool SMS, bool EXT>
-// Variants that keep the running-request records in HBM (C <= 2) run
-// workloads with many replicas and must stay at 128 registers so that 8
-// blocks of two warps fit on an SM.  The bound asks for 7: the compiler
-// still allocates 128 registers and the launch still holds 8 blocks per SM,
-// but its code for that bound measured faster than for a bound of 8 (1-4 %,
-// same-box A/B on the 16,384- and 3,840-replica workloads); a bound of 10
-// (96 registers, 9-10 blocks) was 10-16 % slower.  The others keep 4: their
-// shared memory or register needs limit residency anyway.
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4) k_run(Params p) {
+// Resident warps against registers, same-box A/B.  Two instances per lane,
+// records in HBM: a bound of 10 blocks compiles to 96 registers (no spills),
+// and shared memory then holds 9 blocks of two warps: 113.6 ms on 8,192
+// replicas x 64 instances x 4,000 requests, against 131.0 ms with 8 blocks at
+// 124 registers.  (10 resident blocks, with 1 KB less of scratch per warp:
+// 110.4 ms; 12 blocks would need 80
+// registers, which spills.)  One instance per lane: 8 blocks (110 registers)
+// 20.8 ms on 3,840 x 32 x 1,000, 10 blocks 21.8 ms, 12 blocks (80 registers)
+// 21.9 ms.  The others are bound by one replica's chain.
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2 ? 10 : 8) k_run(Params p) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long *magic = reinterpret_cast<unsigned long long *>(smem);
     for (int d = threadIdx.x; d <= 64; d += blockDim.x)
@@ -1218,7 +1292,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t slot_bytes = SMS ? (uint32_t)p.N * (uint32_t)p.Bmax * 16u : 0u;
-    const uint32_t per_warp = p.L.bytes + slot_bytes + p.hash_bytes;
+    const uint32_t per_warp = p.L.bytes + slot_bytes + (1u << p.set_bits);
     unsigned char *blob = smem + kMagicBytes + (size_t)(threadIdx.x >> 5) * per_warp;
     uint4 *sslots = reinterpret_cast<uint4 *>(blob + p.L.bytes);
     uint32_t *tset = reinterpret_cast<uint32_t *>(blob + p.L.bytes + slot_bytes);
@@ -1230,8 +1304,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
         }
         r = __shfl_sync(kFull, r, 0);
         if (r >= p.R) break;
-        const RepState rs = p.rep[r];
-        if (rs.status != SIM_REPLICA_RUNNING) continue;
+        if (p.rep[r].status != SIM_REPLICA_RUNNING) continue;
         unsigned char *gblob = p.blobs + (size_t)r * p.L.bytes;
         copy16(blob, gblob, p.L.bytes, lane);
         Ctx x;
@@ -1245,16 +1318,20 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
             x.slots = g_slots;
         }
         x.tset = tset;
+        x.set_bits = p.set_bits;
         __syncwarp();
         const long long o = p.offsets[r];
         x.Q = (uint32_t)(p.offsets[r + 1] - o);
-        x.arrival = p.arrival + o;
-        x.plen = p.plen + o;
-        x.olen = p.olen + o;
-        x.tier = p.tier + o;
         x.node = p.node + o;
-        x.res = p.res + o;
-        x.log = p.log + (size_t)r * p.cap;
+        x.r = r;
+        x.arrival = p.arrival;
+        x.plen = p.plen;
+        x.olen = p.olen;
+        x.tier = p.tier;
+        x.node0 = p.node;
+        x.log0 = p.log;
+        x.res_off = p.res_off;
+        x.cap = p.cap;
         x.magic = magic;
         x.magT = p.magT;
         x.N = p.N;
@@ -1263,34 +1340,24 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
         x.TH = p.TH;
         x.Bmax = p.Bmax;
         x.S = p.S;
-        x.cap = p.cap;
         x.lane = lane;
         x.drains = EXT ? p.drains : 0;
-        x.t = rs.t;
-        uint32_t tmax = rs.t;  // latest event time this lane has processed (the replica's: max over lanes)
-        Cnt cn;  // lane 0: the replica's totals; other lanes: what they add in windows
-        const bool l0 = lane == 0;
-        cn.finished = rs.finished;
-        cn.log_events = rs.log_events;
-        cn.migrations = rs.migrations;
-        cn.preemptions = l0 ? rs.preemptions : 0u;
-        cn.starts = rs.starts;
-        cn.aborts = l0 ? rs.aborts : 0u;
-        cn.scale_out = rs.scale_out;
-        cn.scale_in = rs.scale_in;
+        x.t = p.rep[r].t;
+        uint32_t tmax = x.t;  // latest event time this lane has processed (the replica's: max over lanes)
+        Cnt cn;
+        cn.finished = p.rep[r].finished;
         cn.steps = 0;
         cn.iterations = 0;
-        cn.member_iterations = l0 ? rs.member_iterations : 0ull;
-        cn.events = l0 ? rs.events : 0ull;
+        cn.member_iterations = 0;
         cn.status = SIM_REPLICA_RUNNING;
+        uint32_t cursor = p.rep[r].cursor;
+        uint32_t next_tick = p.rep[r].next_tick;
         x.hold = false;
         // whether some instance may be in a migration (kept current: set by a tick
         // that starts one, taken back when a window closes without any)
         bool mig = false;
         for (int i = lane; i < x.N; i += 32) mig = mig || x.mrole[i] != MIG_NONE;
         mig = __any_sync(kFull, mig);
-        uint32_t cursor = rs.cursor;
-        uint32_t next_tick = rs.next_tick;
         ArrBuf ab;
         arr_refill(x, ab, cursor);
         uint32_t next_arr = __shfl_sync(kFull, ab.time, 0);
@@ -1318,10 +1385,10 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                 uint32_t et[C];      // event time of each own instance in this pass
                 uint32_t heads = 0;  // own instances whose iteration ends in this pass
                 uint32_t wake_lo = 0, wake_hi = 0;  // own idle instances to form in a window pass
-                bool any_wake = false;
+                bool any_wake = false, ends = true;
                 uint32_t tstep = 0;  // step time (modes 1 and 2)
                 bool tick = false;
-                if (in_cm && !any_b) {
+                if (MT_RARE(in_cm && !any_b)) {
                     uint32_t cb = kNone;
 #pragma unroll
                     for (int j = 0; j < C; ++j)
@@ -1353,25 +1420,12 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                     if (any_b || (tb < tg && max_steps - cn.steps > (uint32_t)x.N)) {
                         mode = 0;
                         if (!any_b) {
-                        t1 = (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
-                        // distinct event times of the window, and the latest
-                        if (C == 1) {
-                            const uint32_t u = et[0] < t1 ? et[0] : kNone;
-                            const uint32_t grp = __match_any_sync(kFull, u);
-                            ucount = __popc(__ballot_sync(kFull, u != kNone && (__ffs(grp) - 1) == lane));
-                            if (u != kNone) tmax = max(tmax, u);
-                        } else {
-                            for (uint32_t q = (uint32_t)lane; q < kHashSlots; q += 32) tset[q] = kNone;
-                            __syncwarp();
-                            uint32_t fresh = 0;
+                            t1 = (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
+                            // distinct event times of the window, and the latest
+                            ucount = distinct_times<C>(x, tb, t1, et);
 #pragma unroll
-                            for (int j = 0; j < C; ++j) {
-                                if (et[j] >= t1) continue;
-                                tmax = max(tmax, et[j]);
-                                fresh += tset_insert(x, et[j]);
-                            }
-                            ucount = __reduce_add_sync(kFull, fresh);
-                        }
+                            for (int j = 0; j < C; ++j)
+                                if (et[j] < t1) tmax = max(tmax, et[j]);
                         }
                         if (!mig) {
 #pragma unroll
@@ -1395,6 +1449,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                         if (tc == kNone) { cn.status = SIM_ERR_DEADLOCK; break; }
                         tick = ticks && next_tick <= tc;
                         tstep = tick ? next_tick : tc;
+                        ends = tb == tstep;
                         tmax = max(tmax, tstep);
                         ++cn.steps;
 #pragma unroll
@@ -1427,10 +1482,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                         if ((fzl >> (C + j)) & 1u) coop_stage(x, cn, i);
                     }
                 }
+                int dest = -1;
                 if (mode == 2) {
                     x.t = tstep;
-                    if (next_arr == tstep) dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
-                    if (tick) {  // 3. auto-scaling signal and migration tick
+                    if (next_arr == tstep) dest = dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
+                    if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                         const uint32_t nt = next_tick + p.interval;
                         next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                         if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
@@ -1441,10 +1497,13 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                 // instances at their own times; otherwise the idle instances with
                 // work are formed on lane 0 in ascending order (their preemptions
                 // may abort migrations, whose log records are lane 0's) ----
+                // After a lone arrival only its destination can have become able to form
+                // (an instance that stayed idle had nothing that fits, and nothing
+                // else changed).
                 uint32_t want = 0;
                 if (mode == 0) {
                     want = any_wake ? wake_lo : heads;
-                } else {
+                } else if (dest < 0 || ends || tick || x.busy[dest] == kNone) {
                     const uint32_t mask = mode == 1 ? cm : all;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
@@ -1477,7 +1536,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                     if (mig) mig = flush_held<C>(x, cn);
                     cn.steps += ucount;
                 }
-                if (__any_sync(kFull, cn.status < 0)) break;
+                if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
             }
             __syncwarp();
         } else {
@@ -1502,24 +1561,10 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                     const uint32_t t1 =
                         (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
                     // distinct event times of the window, and the latest
-                    uint32_t ucount;
-                    if (C == 1) {
-                        const uint32_t u = bz[0] < t1 ? bz[0] : kNone;
-                        const uint32_t grp = __match_any_sync(kFull, u);
-                        ucount = __popc(__ballot_sync(kFull, u != kNone && (__ffs(grp) - 1) == lane));
-                        if (u != kNone) tmax = max(tmax, u);
-                    } else {
-                        for (uint32_t q = (uint32_t)lane; q < kHashSlots; q += 32) tset[q] = kNone;
-                        __syncwarp();
-                        uint32_t fresh = 0;
+                    const uint32_t ucount = distinct_times<C>(x, tb, t1, bz);
 #pragma unroll
-                        for (int j = 0; j < C; ++j) {
-                            if (bz[j] >= t1) continue;
-                            tmax = max(tmax, bz[j]);
-                            fresh += tset_insert(x, bz[j]);
-                        }
-                        ucount = __reduce_add_sync(kFull, fresh);
-                    }
+                    for (int j = 0; j < C; ++j)
+                        if (bz[j] < t1) tmax = max(tmax, bz[j]);
                     // The iterations of the own instances in `sel` end; finishes and copy
                     // stages follow, one instance at a time by the whole warp (each
                     // touches only its own pair, so their order does not matter).
@@ -1546,11 +1591,18 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                     };
                     // Every lane forms its own instances' next batches.
                     auto forms = [&](uint32_t sel) {
-#pragma unroll
-                        for (int j = 0; j < C; ++j) {
-                            if (!((sel >> j) & 1u)) continue;
-                            x.t = bz[j];
-                            inst_form(x, cn, lane * C + j, p.base, p.a, p.b);
+                        if (C == 1) {
+                            if (sel) {
+                                x.t = bz[0];
+                                inst_form(x, cn, lane, p.base, p.a, p.b);
+                            }
+                        } else {
+#pragma unroll 1
+                            for (uint32_t h = sel; h; h &= h - 1) {
+                                const int j = __ffs(h) - 1;
+                                x.t = pick_c<C>(bz, j);
+                                inst_form(x, cn, lane * C + j, p.base, p.a, p.b);
+                            }
                         }
                         __syncwarp();
                     };
@@ -1595,13 +1647,13 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                             x.t = tc;
                             complete_all<C>(x, cn, same);
                             form_all<C>(x, cn, same, p);
-                            if (__any_sync(kFull, cn.status < 0)) break;
+                            if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
                         }
                         x.hold = false;
                         mig = flush_held<C>(x, cn);
                     }
                     cn.steps += ucount;
-                    if (__any_sync(kFull, cn.status < 0)) break;
+                    if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
                     continue;
                 }
                 // ---- one step at the next event time (global events, or near the step limit) ----
@@ -1612,15 +1664,19 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
                 tmax = max(tmax, x.t);
                 ++cn.steps;
                 if (tb == x.t) complete_all<C>(x, cn, all);  // 1. iteration ends
-                if (next_arr == x.t) dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
-                if (tick) {  // 3. auto-scaling signal and migration tick
+                int dest = -1;
+                if (next_arr == x.t) dest = dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
+                if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                     const uint32_t nt = next_tick + p.interval;
                     next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                     if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
                     if (p.enable_mig) mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
                 }
-                form_all<C>(x, cn, all, p);  // 4. batch formation
-                if (__any_sync(kFull, cn.status < 0)) break;
+                // 4. batch formation.  After a lone arrival only its destination can
+                // have become able to form (an instance that stayed idle had nothing
+                // that fits, and nothing else changed).
+                if (tb == x.t || tick || dest < 0 || x.busy[dest] == kNone) form_all<C>(x, cn, all, p);
+                if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
             }
             __syncwarp();
         }
@@ -1628,39 +1684,32 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, (!SMS && C <= 2) ? 7 : 4)
         // every lane, or an error on some)
         cn.status = __reduce_min_sync(kFull, cn.status);
         const uint32_t tfin = __reduce_max_sync(kFull, tmax);
-        const uint32_t a_pre = __reduce_add_sync(kFull, l0 ? 0u : cn.preemptions);
-        const uint32_t a_ab = __reduce_add_sync(kFull, l0 ? 0u : cn.aborts);
         const uint32_t a_it = __reduce_add_sync(kFull, cn.iterations);
-        uint64_t a_mi = cn.member_iterations, a_ev = cn.events;
+        uint64_t a_mi = cn.member_iterations;
 #pragma unroll
-        for (int sh = 16; sh > 0; sh >>= 1) {
-            a_mi += __shfl_xor_sync(kFull, a_mi, sh);
-            a_ev += __shfl_xor_sync(kFull, a_ev, sh);
-        }
+        for (int sh = 16; sh > 0; sh >>= 1) a_mi += __shfl_xor_sync(kFull, a_mi, sh);
         copy16(gblob, blob, p.L.bytes, lane);
         if (SMS)
             copy16(reinterpret_cast<unsigned char *>(g_slots), reinterpret_cast<const unsigned char *>(sslots),
                    slot_bytes, lane);
-        if (l0) {
-            RepState o2;
+        if (lane == 0) {
+            RepState o2 = p.rep[r];  // this warp's until the launch ends
             o2.t = tfin;
             o2.cursor = cursor;
             o2.finished = cn.finished;
-            o2.log_events = cn.log_events;
+            o2.log_events = x.tot[TOT_LOG];
             o2.next_tick = next_tick;
-            o2.pad0 = 0;
-            o2.steps = rs.steps + cn.steps;
-            o2.iterations = rs.iterations + a_it;
-            o2.member_iterations = a_mi;
-            o2.events = a_ev;
-            o2.migrations = cn.migrations;
-            o2.preemptions = cn.preemptions + a_pre;
-            o2.starts = cn.starts;
-            o2.aborts = cn.aborts + a_ab;
-            o2.scale_out = cn.scale_out;
-            o2.scale_in = cn.scale_in;
+            o2.steps += cn.steps;
+            o2.iterations += a_it;
+            o2.member_iterations += a_mi;
+            o2.migrations = x.tot[TOT_MIG];
+            o2.preemptions = x.tot[TOT_PRE];
+            o2.starts = x.tot[TOT_START];
+            o2.aborts = x.tot[TOT_ABORT];
+            o2.scale_out = x.tot[TOT_OUT];
+            o2.scale_in = x.tot[TOT_IN];
+            o2.events = (uint64_t)cursor + cn.finished + o2.migrations + o2.preemptions;
             o2.status = cn.status;
-            o2.pad1 = 0;
             p.rep[r] = o2;
         }
         __syncwarp();
@@ -1689,6 +1738,7 @@ __global__ void k_init_state(Params p, const int *rep_table, const int *tbl_k, c
             reinterpret_cast<InstRec *>(b + L.inst)[i] = v;
         }
         for (int q = lane; q < N * p.TH; q += 32) b[L.hist + q] = 0;
+        if (lane < TOT_COUNT) reinterpret_cast<uint32_t *>(b + L.tot)[lane] = 0;
         for (int i = lane; i < NK; i += 32) {
             reinterpret_cast<uint16_t *>(b + L.cnt)[i] = 0;
             reinterpret_cast<uint32_t *>(b + L.head)[i] = kNone;
@@ -1852,25 +1902,27 @@ inline Layout make_layout(int N, int K, int T) {
     L.cnt = take(2u * N * K, 16);
     L.hist = take((uint32_t)N * hist_stride(T), 16);
     L.mslot = take(16u * N, 16);
+    L.tot = take(4u * TOT_COUNT, 16);
     L.bytes = (o + 15u) & ~15u;
     return L;
 }
 
-// Bytes of the per-warp event-time set; only variants with several instances per lane use it.
-inline uint32_t hash_bytes_for(int N) { return lanes_c(N) > 1 ? kHashSlots * 4u : 0u; }
+// Size of the per-warp scratch of distinct_times, log2 of its bytes.
+inline int set_bits_for(int N, bool sms) { return sms || lanes_c(N) > 2 ? kSetBitsShared : kSetBits; }
 
 // Chooses the kernel variant and grid for a problem; cudaSuccess or the error.
 // Running-request records go to shared memory while a replica's take at most this many bytes.
 constexpr uint32_t kSmemSlotLimit = 24u * 1024u;
+inline bool slots_in_shared(int N, int Bmax) { return (uint32_t)N * (uint32_t)Bmax * 16u <= kSmemSlotLimit; }
 
 inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &out) {
     const uint32_t slot_bytes = (uint32_t)N * (uint32_t)Bmax * 16u;
-    const bool sms = slot_bytes <= kSmemSlotLimit;
+    const bool sms = slots_in_shared(N, Bmax);
     out.c = lanes_c(N);
     out.sms = sms;
     out.fn = sms ? pick<true, false>(lanes_c(N)) : pick<false, false>(lanes_c(N));
     out.fn_ext = sms ? pick<true, true>(lanes_c(N)) : pick<false, true>(lanes_c(N));
-    out.smem = kMagicBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + hash_bytes_for(N));
+    out.smem = kMagicBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << set_bits_for(N, sms)));
     int dev = 0, sms_count = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
@@ -2021,7 +2073,7 @@ void fill_scalars(mt::Params &p, const sim_cluster_t &cl, const sim_policy_t &po
     p.lcm_lo = (unsigned long long)l;
     p.lcm_hi = (unsigned long long)(l >> 64);
     p.L = L;
-    p.hash_bytes = mt::hash_bytes_for(cl.num_instances);
+    p.set_bits = mt::set_bits_for(cl.num_instances, mt::slots_in_shared(cl.num_instances, cl.max_batch));
 }
 
 mt::Params make_params(const sim_t *s, long long max_steps) {
@@ -2037,6 +2089,7 @@ mt::Params make_params(const sim_t *s, long long max_steps) {
     p.tier = s->d_tier;
     p.node = s->d_node;
     p.res = s->d_res;
+    p.res_off = (const char *)s->d_res - (const char *)s->d_node;
     p.blobs = s->d_blobs;
     p.slots = s->d_slots;
     p.rep = s->d_rep;
@@ -2594,6 +2647,7 @@ extern "C" int sim_run_static(const sim_cluster_t *cl, const sim_tier_table_t *t
     p.tier = tier;
     p.node = (uint4 *)(base + o_node);
     p.res = per_request;
+    p.res_off = (const char *)p.res - (const char *)p.node;
     p.blobs = base + o_blobs;
     p.slots = (uint4 *)(base + o_slots);
     p.rep = (mt::RepState *)(base + o_rep);
