@@ -1252,6 +1252,64 @@ __device__ __forceinline__ Window<C> classify(const Ctx &x, uint32_t t1, uint32_
     return w;
 }
 
+// Advances the instances (one per lane, in no migration) through windows in
+// which every iteration that ends is a quiet one, with the instances' state in
+// registers: nothing finishes, the running requests get the blocks they need,
+// and no waiting request can join, so the next iteration takes the same time
+// with the same members.  Stops at the first window with another event, at tg
+// or near the step limit, and returns the earliest iteration end then.
+// Collective.  A window takes a reduction, two votes and three shared accesses
+// instead of the phases below: one lightly loaded 4-instance cluster (2,000
+// requests), most of whose windows are quiet, went from 59.9 to 45.4 ms.
+__device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &busy, uint32_t tb, uint32_t tg,
+                                              uint32_t max_steps, uint32_t &tmax, const Params &p) {
+    const int i = x.lane < x.N ? x.lane : 0;
+    const uint32_t n = x.nrun[i], minfin = x.minfin[i], dur = (uint32_t)p.base + (uint32_t)p.b * n;
+    const bool waits = x.wmask[i] != 0 && (int)n < x.Bmax;
+    const int need = x.hol[i];
+    const uint8_t *hist = x.hist + i * x.TH;
+    uint32_t nf = x.nf[i], ph = x.phase[i], done = 0;
+    int fr = x.free_[i], grow = 0;
+    bool quiet = false;
+    // whether the end of the running iteration is quiet, and the blocks its successor takes
+    auto look = [&]() {
+        grow = hist[ph == 0 ? 0u : (uint32_t)x.T - ph];
+        quiet = nf != minfin && grow <= fr && !(waits && need <= fr - grow) && busy < 0xFFFFFFFEu - dur;
+    };
+    look();
+    while (tb < tg && max_steps - cn.steps > (uint32_t)x.N) {
+        const uint32_t t1 = (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
+        const bool ends = busy < t1;
+        if (__any_sync(kFull, ends && !quiet)) break;
+        const uint32_t et[1] = {busy};
+        cn.steps += distinct_times<1>(x, tb, t1, et);
+        if (ends) {
+            ++done;
+            tmax = max(tmax, busy);
+            fr -= grow;
+            ++nf;
+            ph = ph + 1u == (uint32_t)x.T ? 0u : ph + 1u;
+            busy += dur;
+            look();
+        }
+        tb = __reduce_min_sync(kFull, busy);
+    }
+    if (done) {
+        x.busy[i] = busy;
+        x.free_[i] = fr;
+        x.nf[i] = nf;
+        x.phase[i] = (uint8_t)ph;
+        cn.iterations += done;
+        cn.member_iterations += (uint64_t)done * n;
+    }
+    __syncwarp();
+    return tb;
+}
+
+// Which variants run quiet windows in registers.
+template <int C, bool SMS>
+constexpr bool kQuiet = C == 1;
+
 // Which main loop a variant runs.  The variants that keep running-request
 // records in HBM with at most two instances per lane run 16 warps per SM
 // (many replicas); there instruction fetch was the bottleneck, and a loop
@@ -1416,6 +1474,8 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                     if (!any_b) {
                         tb = __reduce_min_sync(kFull, mb);
                         tg = ticks ? min(next_arr, next_tick) : next_arr;
+                        if (kQuiet<C, SMS> && !mig && tb < tg)
+                            tb = run_quiet(x, cn, et[0], tb, tg, max_steps, tmax, p);
                     }
                     if (any_b || (tb < tg && max_steps - cn.steps > (uint32_t)x.N)) {
                         mode = 0;
@@ -1553,9 +1613,10 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                     bz[j] = i < x.N ? x.busy[i] : kNone;
                     mb = min(mb, bz[j]);
                 }
-                const uint32_t tb = __reduce_min_sync(kFull, mb);
+                uint32_t tb = __reduce_min_sync(kFull, mb);
                 const bool ticks = EXT ? p.ticks != 0 : p.enable_mig != 0;
                 const uint32_t tg = ticks ? min(next_arr, next_tick) : next_arr;
+                if (kQuiet<C, SMS> && !mig && tb < tg) tb = run_quiet(x, cn, bz[0], tb, tg, max_steps, tmax, p);
                 if (tb < tg && max_steps - cn.steps > (uint32_t)x.N) {
                     // ---- window [tb, t1): at most one iteration end per instance ----
                     const uint32_t t1 =
