@@ -249,6 +249,63 @@ struct Cnt {
     int status;
 };
 
+// The block's dynamic shared memory: a copy of the parameters (for the
+// out-of-line functions below, which cannot reach the kernel's own), the
+// table of ceil(2^64 / d), then each warp's replica state.
+constexpr uint32_t kParamBytes = (sizeof(Params) + 15u) & ~15u;
+constexpr uint32_t kHeadBytes = kParamBytes + kMagicBytes;
+
+__device__ __forceinline__ void bind_blob(Ctx &x, const Layout &L, unsigned char *blob) {
+    unsigned char *ib = blob + L.inst;
+    x.busy.base = x.free_.base = x.resv.base = x.hol.base = x.hr.base = x.key.base = ib;
+    x.mreq.base = x.mcopied.base = x.nf.base = x.minfin.base = x.drain.base = ib;
+    x.wmask.base = x.nrun.base = x.pc.base = x.phase.base = x.mrole.base = x.mpeer.base = x.mpend.base = ib;
+    x.cnt = reinterpret_cast<uint16_t *>(blob + L.cnt);
+    x.head = reinterpret_cast<uint32_t *>(blob + L.head);
+    x.tail = reinterpret_cast<uint32_t *>(blob + L.tail);
+    x.hinfo = reinterpret_cast<uint32_t *>(blob + L.hinfo);
+    x.h = reinterpret_cast<int *>(blob + L.h);
+    x.hist = blob + L.hist;
+    x.mslot = reinterpret_cast<uint4 *>(blob + L.mslot);
+    x.tot = reinterpret_cast<uint32_t *>(blob + L.tot);
+}
+
+// The view of replica r that this warp is simulating, at time t.
+template <bool SMS>
+__device__ __forceinline__ void bind_ctx(Ctx &x, const Params &p, unsigned char *smem, uint4 *node, uint32_t Q, int r,
+                                         uint32_t t) {
+    const uint32_t slot_bytes = SMS ? (uint32_t)p.N * (uint32_t)p.Bmax * 16u : 0u;
+    unsigned char *blob =
+        smem + kHeadBytes + (size_t)(threadIdx.x >> 5) * (p.L.bytes + slot_bytes + (1u << p.set_bits));
+    bind_blob(x, p.L, blob);
+    x.slots = SMS ? reinterpret_cast<uint4 *>(blob + p.L.bytes) : p.slots + (size_t)r * p.N * p.Bmax;
+    x.tset = reinterpret_cast<uint32_t *>(blob + p.L.bytes + slot_bytes);
+    x.set_bits = p.set_bits;
+    x.Q = Q;
+    x.node = node;
+    x.r = r;
+    x.arrival = p.arrival;
+    x.plen = p.plen;
+    x.olen = p.olen;
+    x.tier = p.tier;
+    x.node0 = p.node;
+    x.log0 = p.log;
+    x.res_off = p.res_off;
+    x.cap = p.cap;
+    x.magic = reinterpret_cast<const unsigned long long *>(smem + kParamBytes);
+    x.magT = p.magT;
+    x.N = p.N;
+    x.K = p.K;
+    x.T = p.T;
+    x.TH = p.TH;
+    x.Bmax = p.Bmax;
+    x.S = p.S;
+    x.lane = (int)(threadIdx.x & 31);
+    x.drains = p.drains;
+    x.t = t;
+    x.hold = false;
+}
+
 __device__ __forceinline__ int blocks_for(const Ctx &x, uint32_t tokens) {
     return (int)(((unsigned long long)(tokens + (uint32_t)x.T - 1u) * x.magT) >> kMagicShift);
 }
@@ -476,11 +533,12 @@ __device__ __forceinline__ void slot_join(const Ctx &x, int i, int n, uint32_t r
     slot_join_at(x, i, n, r, c, left, tier, x.nf[i], x.phase[i]);
 }
 
-// Lane 0's part of committing a fully copied running request `sl` of source s
-// to its destination (Sec. 3.5, Fig. 4).  The warp has already taken the
+// Books the commit of the fully copied running request of source s at its
+// destination (Sec. 3.5, Fig. 4), on one lane.  The warp has already taken the
 // slot out of s's running list (order kept); fm is the new minimum finishing
 // formation of what is left there.
-__device__ __forceinline__ void commit_book(const Ctx &x, Cnt &cn, int s, const uint4 &sl, uint32_t fm) {
+__device__ __forceinline__ void commit_book(const Ctx &x, Cnt &cn, int s, uint32_t fm) {
+    const uint4 sl = x.mslot[s];  // slot records do not change while they run
     const int d = x.mpeer[s];
     const int blocks = sl_blocks(x, s, sl);
     const uint32_t adv = sl_adv(x, s, sl);
@@ -496,7 +554,7 @@ __device__ __forceinline__ void commit_book(const Ctx &x, Cnt &cn, int s, const 
     slot_join(x, d, nd, sl.x, sl_c(sl) + adv, sl_left(sl) - adv, tr);
     x.nrun[d] = (uint8_t)(nd + 1);
     bump_mig(x, sl.x);
-    x.tot[TOT_MIG]++;
+    atomicAdd(&x.tot[TOT_MIG], 1u);
     log_end(x, cn, SIM_EV_COMMIT, sl.x, s, d, blocks, 1);
     clear_mig(x, s, d);
 }
@@ -558,54 +616,121 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
 }
 
 // One copy stage at the end of an iteration of migration source s (nothing
-// to do if s is none, or if a finish has just abandoned its migration), whole
-// warp: up to S of the request's blocks are reserved on the destination
-// (abandoning the migration if they do not fit), and the request commits
-// there once all of them are copied (Sec. 3.5, Fig. 4).
+// to do if a finish has just abandoned its migration), single thread: up to S
+// of the request's blocks are reserved on the destination (abandoning the
+// migration if they do not fit).  Returns whether all of them are copied and
+// the request can commit there now (Sec. 3.5, Fig. 4): coop_commit must follow.
+__device__ __forceinline__ bool stage_copy(const Ctx &x, Cnt &cn, int s) {
+    if (x.mrole[s] != MIG_SRC) return false;
+    const int d = x.mpeer[s];
+    const int blocks = sl_blocks(x, s, x.mslot[s]);
+    const int cp = x.mcopied[s];
+    const int cc = min(x.S, blocks - cp);
+    if (MT_RARE(x.free_[d] < cc)) {
+        abort_mig(x, cn, s, 1);
+        return false;
+    }
+    x.free_[d] -= cc;
+    x.resv[d] += cc;
+    x.mcopied[s] = cp + cc;
+    return cp + cc == blocks && (int)x.nrun[d] < x.Bmax;
+}
+
+// The running records of instance s, lane l holding slots l and 32 + l.
+struct Slots2 {
+    uint4 a0, a1;
+};
+__device__ __forceinline__ Slots2 load_slots(const Ctx &x, int s) {
+    const int n = x.nrun[s];
+    const uint4 *p = slot_ptr(x, s, 0);
+    const uint4 none = make_uint4(kNone, 0, 0, 0);
+    return Slots2{x.lane < n ? p[x.lane] : none, x.lane + 32 < n ? p[x.lane + 32] : none};
+}
+
+// Commits the fully copied request of source s, whole warp: finds its slot
+// among the records `v`, closes the gap and takes the survivors' minimum; the
+// lane that owns s books.
+__device__ __forceinline__ void coop_commit(const Ctx &x, Cnt &cn, int s, int owner, const Slots2 &v) {
+    const uint32_t rid = x.mreq[s];
+    const int n = x.nrun[s];
+    uint4 *p = slot_ptr(x, s, 0);
+    const int q0 = x.lane, q1 = x.lane + 32;
+    const uint32_t h0 = __ballot_sync(kFull, q0 < n && v.a0.x == rid);
+    const uint32_t h1 = __ballot_sync(kFull, q1 < n && v.a1.x == rid);
+    const int pos = h0 ? __ffs(h0) - 1 : (h1 ? 32 + __ffs(h1) - 1 : -1);
+    if (MT_RARE(pos < 0)) {
+        if (x.lane == 0) cn.status = SIM_ERR_INTERNAL;
+    } else {
+        const uint32_t fm = __reduce_min_sync(
+            kFull, min(q0 < n && q0 != pos ? sl_fin(v.a0) : kNone, q1 < n && q1 != pos ? sl_fin(v.a1) : kNone));
+        if (q0 < n && q0 > pos) p[q0 - 1] = v.a0;
+        if (q1 < n && q1 > pos) p[q1 - 1] = v.a1;
+        if (x.lane == owner) commit_book(x, cn, s, fm);
+    }
+    __syncwarp();
+}
+
+// Copy stage of source s, then its commit if it is due, whole warp (steps at
+// one time, where the oracle orders instances by index).
 __device__ __forceinline__ void coop_stage(const Ctx &x, Cnt &cn, int s) {
     int commit = 0;
-    if (x.lane == 0 && x.mrole[s] == MIG_SRC) {
-        const int d = x.mpeer[s];
-        const int blocks = sl_blocks(x, s, x.mslot[s]);
-        const int cp = x.mcopied[s];
-        const int cc = min(x.S, blocks - cp);
-        if (MT_RARE(x.free_[d] < cc)) {
-            abort_mig(x, cn, s, 1);
-        } else {
-            x.free_[d] -= cc;
-            x.resv[d] += cc;
-            x.mcopied[s] = cp + cc;
-            commit = (cp + cc == blocks) && ((int)x.nrun[d] < x.Bmax);
-        }
+    if (x.lane == 0) commit = stage_copy(x, cn, s) ? 1 : 0;
+    if (__shfl_sync(kFull, commit, 0)) coop_commit(x, cn, s, 0, load_slots(x, s));
+}
+
+// a[j] for a run-time j without dynamic indexing (the array stays in registers)
+template <int C>
+__device__ __forceinline__ uint32_t pick_c(const uint32_t (&a)[C], int j) {
+    uint32_t v = a[0];
+#pragma unroll
+    for (int k = 1; k < C; ++k)
+        if (j == k) v = a[k];
+    return v;
+}
+
+// The copy stages of the own sources in `src`, each at its own time et[j]: the
+// lanes reserve or abandon together, then the requests that are due commit one
+// after another by the whole warp, the next source's records loaded while one
+// commits.  Pairs share no state and the log records are held back, so the
+// order does not matter.  (256 replicas x 128 instances: a copy takes about
+// five stages, 32 pairs per tick; staged one by one they took a third of the
+// time.)  Collective.
+template <int C>
+__device__ __forceinline__ void stage_all(Ctx &x, Cnt &cn, uint32_t src, const uint32_t (&et)[C]) {
+    uint32_t due = 0;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        if (!((src >> j) & 1u)) continue;
+        x.t = et[j];
+        if (stage_copy(x, cn, x.lane * C + j)) due |= 1u << j;
     }
-    commit = __shfl_sync(kFull, commit, 0);
     __syncwarp();
-    if (commit) {
-        // the whole warp finds the request's slot (lane l holds slots l and
-        // 32 + l), closes the gap and takes the survivors' minimum; lane 0 books
-        const uint32_t rid = x.mreq[s];
-        const int n = x.nrun[s];
-        uint4 *p = slot_ptr(x, s, 0);
-        const int q0 = x.lane, q1 = x.lane + 32;
-        const bool v0 = q0 < n, v1 = q1 < n;
-        const uint4 a0 = v0 ? p[q0] : make_uint4(0, 0, 0, 0);
-        const uint4 a1 = v1 ? p[q1] : make_uint4(0, 0, 0, 0);
-        const uint32_t h0 = __ballot_sync(kFull, v0 && a0.x == rid);
-        const uint32_t h1 = __ballot_sync(kFull, v1 && a1.x == rid);
-        const int pos = h0 ? __ffs(h0) - 1 : (h1 ? 32 + __ffs(h1) - 1 : -1);
-        if (MT_RARE(pos < 0)) {
-            if (x.lane == 0) cn.status = SIM_ERR_INTERNAL;
-        } else {
-            const uint4 sl = p[pos];
-            const uint32_t fm = __reduce_min_sync(
-                kFull, min(v0 && q0 != pos ? sl_fin(a0) : kNone, v1 && q1 != pos ? sl_fin(a1) : kNone));
-            __syncwarp();
-            if (v0 && q0 > pos) p[q0 - 1] = a0;
-            if (v1 && q1 > pos) p[q1 - 1] = a1;
-            __syncwarp();
-            if (x.lane == 0) commit_book(x, cn, s, sl, fm);
+    uint32_t lanes = __ballot_sync(kFull, due != 0), h = 0;
+    int l = 0;
+    auto next = [&]() -> int {  // the next source that is due, or -1
+        if (h == 0) {
+            if (lanes == 0) return -1;
+            l = __ffs(lanes) - 1;
+            lanes &= lanes - 1;
+            h = C == 1 ? 1u : __shfl_sync(kFull, due, l);
         }
-        __syncwarp();
+        const int j = __ffs(h) - 1;
+        h &= h - 1;
+        return l * C + j;
+    };
+    int s = next();
+    if (s < 0) return;
+    Slots2 v = load_slots(x, s);
+#pragma unroll 1
+    for (;;) {
+        const int s2 = next();
+        Slots2 v2;
+        if (s2 >= 0) v2 = load_slots(x, s2);
+        if (C > 1 && x.lane == s / C) x.t = pick_c<C>(et, s % C);
+        coop_commit(x, cn, s, s / C, v);
+        if (s2 < 0) break;
+        s = s2;
+        v = v2;
     }
 }
 
@@ -627,11 +752,100 @@ __device__ __forceinline__ unsigned int preempt_book(const Ctx &x, Cnt &cn, int 
     return word;  // for pre_fix, which the caller runs later so that nothing waits here
 }
 
+// The rare paths below are functions of their own, so that their code and
+// registers stay out of the main loop (which instruction fetch and the
+// registers per resident warp bound); they rebuild the replica's view from
+// shared memory instead of taking it in registers.
+
+// KV growth at the formation of instance i when the running requests need more
+// blocks than are free (Sec. 2.2, 3.1).  Single thread.
+__device__ __forceinline__ void grow_slow(const Ctx &x, Cnt &cn, int i) {
+    const int n = x.nrun[i], fr = x.free_[i];
+    const uint32_t ph = x.phase[i], nf = x.nf[i];
+                // In running order, a request that needs a block (at most one)
+                // takes a free one or preempts the lowest-priority newest running
+                // request, possibly itself.  Positions are the list's before this
+                // step; removals are applied afterwards.
+                uint4 *p = slot_ptr(x, i, 0);
+                const uint64_t all = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
+                uint64_t alive = all, needs = 0, granted = 0;
+                // The requests that need a block now are those whose context reaches
+                // a block boundary: rho == -nf (mod T), the ones hist counts.
+                const uint32_t target = ph == 0 ? 0u : (uint32_t)x.T - ph;
+                // the same pass finds the first victim (lowest priority, then newest):
+                // more requests need a block than there are free blocks, so there is one
+                int v1 = -1;
+                uint32_t vt1 = 0, vr1 = 0;
+#pragma unroll 4
+                for (int q = 0; q < n; ++q) {
+                    const uint4 sl = p[q];
+                    needs |= (uint64_t)(sl_rho(sl) == target) << q;
+                    const uint32_t ts = sl_tier(sl);
+                    if (v1 < 0 || ts > vt1 || (ts == vt1 && sl.x > vr1)) { v1 = q; vt1 = ts; vr1 = sl.x; }
+                }
+                int fb = fr;
+                uint32_t pr = kNone;  // the last preempted request and its counter word before the add
+                unsigned int pold = 0;
+#pragma unroll 1
+                for (int q = 0; q < n; ++q) {
+                    if (!((alive & needs) >> q & 1ull)) continue;
+                    for (;;) {
+                        if (fb > 0) { --fb; granted |= 1ull << q; break; }
+                        int v = -1;
+                        if (alive == all) {
+                            v = v1;  // nobody preempted yet: the victim found by the scan
+                        } else {
+                            uint32_t vt = 0, vr = 0;
+#pragma unroll 1
+                            for (uint64_t m = alive; m; m &= m - 1) {
+                                const int s2 = __ffsll((long long)m) - 1;
+                                const uint32_t ts = sl_tier(p[s2]), rs = p[s2].x;
+                                if (v < 0 || ts > vt || (ts == vt && rs > vr)) { v = s2; vt = ts; vr = rs; }
+                            }
+                        }
+                        const int vb = blocks_for(x, sl_c(p[v]) + nf - p[v].y) + (int)((granted >> v) & 1ull);
+                        alive &= ~(1ull << v);
+                        x.free_[i] = fb;
+                        if (pr != kNone) pre_fix(x, pr, pold);
+                        pr = p[v].x;
+                        pold = preempt_book(x, cn, i, p[v], vb);
+                        fb = x.free_[i];
+                        if (v == q) break;
+                    }
+                }
+                x.free_[i] = fb;
+                int w = 0;
+                uint32_t fm = kNone;  // the survivors' next finishing formation
+#pragma unroll 1
+                for (int q = 0; q < n; ++q) {
+                    if ((alive >> q) & 1ull) {
+                        const uint4 sl = p[q];
+                        if (w != q) p[w] = sl;
+                        ++w;
+                        fm = min(fm, sl_fin(sl));
+                    }
+                }
+                x.nrun[i] = (uint8_t)w;
+                x.minfin[i] = fm;
+                if (pr != kNone) pre_fix(x, pr, pold);
+}
+
+template <bool SMS>
+__device__ __noinline__ void grow_call(uint4 *node, uint32_t Q, int r, uint32_t t, int i, bool hold) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    Ctx x;
+    bind_ctx<SMS>(x, *reinterpret_cast<const Params *>(smem), smem, node, Q, r, t);
+    x.hold = hold;
+    Cnt cn;
+    grow_slow(x, cn, i);
+}
+
 // Phase 4: batch formation at idle instance i at x.t (Sec. 2.2, Sec. 3.1):
 // (i) KV growth of the running requests, preempting the lowest-priority newest
 // one when out of blocks; (ii) admission in (tier, FCFS) order while the head
 // of line fits; (iii) the iteration starts.
-__device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base, int a_us, int b_us) {
+template <bool SMS, bool LEAN>
+__device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &p) {
     // the instance's scalars, read together up front (the code below would
     // otherwise reload them after every shared-memory store)
     int n = x.nrun[i];
@@ -645,74 +859,12 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
         if (!MT_RARE(deficit > fr)) {
             fr -= deficit;  // every request that needs a block gets it
         } else {
-            x.free_[i] = fr;
-            // In running order, a request that needs a block (at most one)
-            // takes a free one or preempts the lowest-priority newest running
-            // request, possibly itself.  Positions are the list's before this
-            // step; removals are applied afterwards.
-            uint4 *p = slot_ptr(x, i, 0);
-            const uint64_t all = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
-            uint64_t alive = all, needs = 0, granted = 0;
-            // The requests that need a block now are those whose context reaches
-            // a block boundary: rho == -nf (mod T), the ones hist counts.
-            const uint32_t target = ph == 0 ? 0u : (uint32_t)x.T - ph;
-            // the same pass finds the first victim (lowest priority, then newest):
-            // more requests need a block than there are free blocks, so there is one
-            int v1 = -1;
-            uint32_t vt1 = 0, vr1 = 0;
-#pragma unroll 4
-            for (int q = 0; q < n; ++q) {
-                const uint4 sl = p[q];
-                needs |= (uint64_t)(sl_rho(sl) == target) << q;
-                const uint32_t ts = sl_tier(sl);
-                if (v1 < 0 || ts > vt1 || (ts == vt1 && sl.x > vr1)) { v1 = q; vt1 = ts; vr1 = sl.x; }
+            if (LEAN) {
+                grow_slow(x, cn, i);
+            } else {
+                grow_call<SMS>(x.node, x.Q, x.r, x.t, i, x.hold);
             }
-            int fb = fr;
-            uint32_t pr = kNone;  // the last preempted request and its counter word before the add
-            unsigned int pold = 0;
-#pragma unroll 1
-            for (int q = 0; q < n; ++q) {
-                if (!((alive & needs) >> q & 1ull)) continue;
-                for (;;) {
-                    if (fb > 0) { --fb; granted |= 1ull << q; break; }
-                    int v = -1;
-                    if (alive == all) {
-                        v = v1;  // nobody preempted yet: the victim found by the scan
-                    } else {
-                        uint32_t vt = 0, vr = 0;
-#pragma unroll 1
-                        for (uint64_t m = alive; m; m &= m - 1) {
-                            const int s2 = __ffsll((long long)m) - 1;
-                            const uint32_t ts = sl_tier(p[s2]), rs = p[s2].x;
-                            if (v < 0 || ts > vt || (ts == vt && rs > vr)) { v = s2; vt = ts; vr = rs; }
-                        }
-                    }
-                    const int vb = blocks_for(x, sl_c(p[v]) + nf - p[v].y) + (int)((granted >> v) & 1ull);
-                    alive &= ~(1ull << v);
-                    x.free_[i] = fb;
-                    if (pr != kNone) pre_fix(x, pr, pold);
-                    pr = p[v].x;
-                    pold = preempt_book(x, cn, i, p[v], vb);
-                    fb = x.free_[i];
-                    if (v == q) break;
-                }
-            }
-            x.free_[i] = fb;
-            int w = 0;
-            uint32_t fm = kNone;  // the survivors' next finishing formation
-#pragma unroll 1
-            for (int q = 0; q < n; ++q) {
-                if ((alive >> q) & 1ull) {
-                    const uint4 sl = p[q];
-                    if (w != q) p[w] = sl;
-                    ++w;
-                    fm = min(fm, sl_fin(sl));
-                }
-            }
-            x.nrun[i] = (uint8_t)w;
-            x.minfin[i] = fm;
-            if (pr != kNone) pre_fix(x, pr, pold);
-            n = w;  // preemptions changed the free blocks, queues and head of line
+            n = x.nrun[i];  // preemptions changed the running list, the free blocks, queues and head of line
             fr = x.free_[i];
             wm = x.wmask[i];
             need = x.hol[i];
@@ -755,7 +907,7 @@ __device__ __forceinline__ void inst_form(const Ctx &x, Cnt &cn, int i, int base
     x.free_[i] = fr;
     // (iii) the iteration starts
     if (n > 0) {
-        const long long end = (long long)x.t + base + (long long)a_us * prefill + (long long)b_us * n_decode;
+        const long long end = (long long)x.t + p.base + (long long)p.a * prefill + (long long)p.b * n_decode;
         if (MT_RARE(end > 0xFFFFFFFELL)) {
             cn.status = SIM_ERR_OVERFLOW;
             return;
@@ -827,12 +979,59 @@ __device__ __forceinline__ void arr_refill(const Ctx &x, ArrBuf &ab, uint32_t cu
     ab.po = in ? (uint32_t)x.plen[at] | ((uint32_t)x.olen[at] << 16) : 0u;
 }
 
+// Dispatches all arrivals at t, from trace record `cursor` on, tier by tier to
+// the instances in `all`; returns their number.  Collective.
+template <int C>
+__device__ __forceinline__ uint32_t dispatch_many(const Ctx &x, Cnt &cn, uint32_t cursor, uint32_t all) {
+    refresh_keys<C>(x);
+    const long long at = x.first();
+    uint32_t m = 0;
+#pragma unroll 1
+    for (;;) {
+        const uint32_t j2 = cursor + m + (uint32_t)x.lane;
+        const bool in2 = j2 < x.Q;
+        const uint32_t e2 = __ballot_sync(kFull, in2 && x.arrival[at + j2] == x.t);
+        m += (uint32_t)__popc(e2);
+        if (e2 != kFull) break;
+    }
+#pragma unroll 1
+    for (int k = 0; k < x.K; ++k) {
+#pragma unroll 1
+        for (uint32_t base = 0; base < m; base += 32) {
+            const uint32_t j2 = cursor + base + (uint32_t)x.lane;
+            const bool mine = base + (uint32_t)x.lane < m;
+            const uint32_t tr = mine ? x.tier[at + j2] : 0u;
+            const uint32_t P = mine ? x.plen[at + j2] : 0u;
+            const uint32_t O = mine ? x.olen[at + j2] : 0u;
+            uint32_t bits = __ballot_sync(kFull, mine && tr == (uint32_t)k);
+#pragma unroll 1
+            while (bits) {
+                const int l = __ffs(bits) - 1;
+                bits &= bits - 1;
+                dispatch_one<C>(x, cn, cursor + base + (uint32_t)l, k, __shfl_sync(kFull, P, l),
+                                __shfl_sync(kFull, O, l), all);
+            }
+        }
+    }
+    return m;
+}
+
+template <int C, bool SMS>
+__device__ __noinline__ uint32_t dispatch_call(uint4 *node, uint32_t Q, int r, uint32_t t, uint32_t cursor,
+                                               uint32_t all) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    Ctx x;
+    bind_ctx<SMS>(x, *reinterpret_cast<const Params *>(smem), smem, node, Q, r, t);
+    Cnt cn;
+    return dispatch_many<C>(x, cn, cursor, all);
+}
+
 // Phase 2: arrivals at t, tier 0 first, FCFS (trace order) within a tier.
 // EXT: draining instances may exist.  Returns the destination of a lone
 // arrival, or -1 after several.
-template <int C, bool EXT>
-__device__ __forceinline__ int dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &cursor, uint32_t &next_arr,
-                                               ArrBuf &ab) {
+template <int C, bool SMS, bool EXT, bool LEAN>
+__device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor, uint32_t &next_arr, ArrBuf &ab,
+                                              const Params &p) {
     uint32_t all = own_mask<C>(x);
     if (EXT && x.drains) {
         // Draining instances (infinite virtual usage, Sec. 3.5) get no
@@ -846,13 +1045,9 @@ __device__ __forceinline__ int dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &c
     }
     int dest = -1;
     const uint32_t off = cursor - ab.pb;
-    uint32_t eq = __ballot_sync(kFull, (uint32_t)x.lane >= off && ab.time == x.t);
-    if (MT_RARE((eq >> 31) && off > 0)) {
-        // the run of arrivals at t may continue past the buffer: realign it on the cursor
-        arr_refill(x, ab, cursor);
-        eq = __ballot_sync(kFull, ab.time == x.t);
-    }
-    if (!MT_RARE(eq == kFull || (eq & (eq - 1u)) != 0u)) {
+    const uint32_t eq = __ballot_sync(kFull, (uint32_t)x.lane >= off && ab.time == x.t);
+    // (an arrival in the buffer's last place may have others at t behind it)
+    if (!MT_RARE((eq >> 31) != 0u || (eq & (eq - 1u)) != 0u)) {
         // one arrival at t (the usual case): no tier ordering to do
         const int l = __ffs(eq) - 1;
         const uint32_t k1 = __shfl_sync(kFull, ab.tier, l);
@@ -874,58 +1069,12 @@ __device__ __forceinline__ int dispatch_phase(const Ctx &x, Cnt &cn, uint32_t &c
         __syncwarp();
         dest = best;
         cursor += 1u;
-    } else if (eq != kFull) {
-        refresh_keys<C>(x);
-        const bool mine = (eq >> x.lane) & 1u;
-        uint32_t tm = __reduce_or_sync(kFull, mine ? (1u << ab.tier) : 0u);
-#pragma unroll 1
-        while (tm) {
-            const int k = __ffs(tm) - 1;
-            tm &= tm - 1;
-            uint32_t bits = __ballot_sync(kFull, mine && ab.tier == (uint32_t)k);
-#pragma unroll 1
-            while (bits) {
-                const int l = __ffs(bits) - 1;
-                bits &= bits - 1;
-                const uint32_t po = __shfl_sync(kFull, ab.po, l);
-                dispatch_one<C>(x, cn, ab.pb + (uint32_t)l, k, po & 0xFFFFu, po >> 16, all);
-            }
-        }
-        cursor += (uint32_t)__popc(eq);
     } else {
-        // 32 or more arrivals share this time (the buffer starts at the cursor):
-        // count them, then go tier by tier from the trace.
-        refresh_keys<C>(x);
-        const long long at = x.first();
-        uint32_t m = 32;
-#pragma unroll 1
-        for (;;) {
-            const uint32_t j2 = cursor + m + (uint32_t)x.lane;
-            const bool in2 = j2 < x.Q;
-            const uint32_t e2 = __ballot_sync(kFull, in2 && x.arrival[at + j2] == x.t);
-            m += (uint32_t)__popc(e2);
-            if (e2 != kFull) break;
+        if (LEAN) {
+            cursor += dispatch_many<C>(x, cn, cursor, all);
+        } else {
+            cursor += dispatch_call<C, SMS>(x.node, x.Q, x.r, x.t, cursor, all);
         }
-#pragma unroll 1
-        for (int k = 0; k < x.K; ++k) {
-#pragma unroll 1
-            for (uint32_t base = 0; base < m; base += 32) {
-                const uint32_t j2 = cursor + base + (uint32_t)x.lane;
-                const bool mine = base + (uint32_t)x.lane < m;
-                const uint32_t tr = mine ? x.tier[at + j2] : 0u;
-                const uint32_t P = mine ? x.plen[at + j2] : 0u;
-                const uint32_t O = mine ? x.olen[at + j2] : 0u;
-                uint32_t bits = __ballot_sync(kFull, mine && tr == (uint32_t)k);
-#pragma unroll 1
-                while (bits) {
-                    const int l = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    dispatch_one<C>(x, cn, cursor + base + (uint32_t)l, k, __shfl_sync(kFull, P, l),
-                                    __shfl_sync(kFull, O, l), all);
-                }
-            }
-        }
-        cursor += m;
     }
     if (MT_RARE(cursor - ab.pb >= 32u)) arr_refill(x, ab, cursor);
     next_arr = __shfl_sync(kFull, ab.time, (int)(cursor - ab.pb));
@@ -973,10 +1122,175 @@ __device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Para
     __syncwarp();
 }
 
+// Whether the freeness of d exceeds that of s by at least theta (Sec. 3.5).
+__device__ __forceinline__ bool over_theta(const Ctx &x, int s, int d, int theta_num, int theta_den) {
+    const long long ns = fnum(x, s), ds = max((int)x.nrun[s], 1);
+    const long long nd = fnum(x, d), dd = max((int)x.nrun[d], 1);
+    return (long long)theta_den * (nd * ds - ns * dd) >= (long long)theta_num * dd * ds;
+}
+
+// The newest request of the lowest-priority bucket of s, which has waiting
+// requests, moves to d at once (no KV to copy).  Single thread; k: its place in the log.
+__device__ __forceinline__ void move_queued(const Ctx &x, Cnt &cn, int s, int d, uint32_t k) {
+    const int tr = 31 - __clz((unsigned)x.wmask[s]);
+    uint32_t info = 0;
+    const uint32_t r = pop_back(x, s, tr, info, cn.status);
+    if (MT_RARE(r == kNone)) return;
+    refresh_hol(x, s);
+    cnt_dec(x, s, tr);
+    const uint32_t old = x.wmask[d];
+    push_back(x, d, tr, r, info);
+    cnt_inc(x, d, tr);
+    if ((old & ((2u << tr) - 1u)) == 0) x.hol[d] = blocks_for(x, info & 0xFFFFu);
+    bump_mig(x, r);
+    if (k < (uint32_t)x.cap) *x.log(k) = make_uint4(x.t, r, ((uint32_t)s << 16) | ((uint32_t)d << 24), SIM_EV_QUEUED);
+}
+
+// The running request of s (its records: v) with the lowest priority, then the
+// fewest blocks, then the newest, starts its staged copy to d if its blocks
+// fit there.  Collective; k: its place in the log.
+__device__ __forceinline__ bool start_copy(const Ctx &x, int s, int d, const Slots2 &v, uint32_t k) {
+    const int n = x.nrun[s];
+    const bool v0 = x.lane < n, v1 = x.lane + 32 < n;
+    const int k0 = v0 ? (int)((sl_tier(v.a0) << 16) | (0xFFFFu - (uint32_t)sl_blocks(x, s, v.a0))) : -1;
+    const int k1 = v1 ? (int)((sl_tier(v.a1) << 16) | (0xFFFFu - (uint32_t)sl_blocks(x, s, v.a1))) : -1;
+    const int km = __reduce_max_sync(kFull, max(k0, k1));
+    if (km < 0) return false;  // nothing runs there
+    const int blocks = (int)(0xFFFFu - ((uint32_t)km & 0xFFFFu));
+    if (MT_RARE(x.free_[d] < blocks)) return false;
+    const bool c0 = k0 == km, c1 = k1 == km;
+    const uint32_t rid = __reduce_max_sync(kFull, max(c0 ? v.a0.x : 0u, c1 ? v.a1.x : 0u));
+    const bool b0 = c0 && v.a0.x == rid;
+    if (b0 || (c1 && v.a1.x == rid)) {  // the lane that holds it books
+        x.mrole[s] = MIG_SRC;
+        x.mpeer[s] = (uint8_t)d;
+        x.mreq[s] = rid;
+        x.mcopied[s] = 0;
+        x.mslot[s] = b0 ? v.a0 : v.a1;
+        x.mrole[d] = MIG_DST;
+        x.mpeer[d] = (uint8_t)s;
+        if (k < (uint32_t)x.cap)
+            *x.log(k) = make_uint4(x.t, rid, (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24),
+                                   SIM_EV_START);
+    }
+    return true;
+}
+
+// Phase 3 with theta > 0 and nothing draining: the freeness order is fixed for
+// the tick, so every lane ranks its instances by ascending (sources) and
+// descending freeness (destinations, lowest index first among equals in both)
+// once, and pair r is then (source r, destination r) as long as the threshold
+// holds; theta > 0 keeps the two sides apart.  The threshold and the moves of
+// queued requests are done by one lane per pair, up to 32 at once; running
+// candidates are found pair by pair by the whole warp, the next source's
+// records loaded meanwhile.  A source whose candidate does not fit leaves its
+// destination to the next source.  Returns whether a staged copy started.
+// (A serial search took about 2,500 cycles per pair, two reductions for each
+// side, the threshold and one memory round trip; 256 replicas x 128 instances
+// start 32 copies per tick.)
+template <int C>
+__device__ __forceinline__ bool ranked_tick(const Ctx &x, Cnt &cn, int theta_num, int theta_den) {
+    int *sk = reinterpret_cast<int *>(x.tset);
+    const int np = (x.N + 3) & ~3;
+    uint8_t *lo = reinterpret_cast<uint8_t *>(sk + np), *hi = lo + np;
+    int key[C], lt[C], eqb[C], eqa[C];
+    uint32_t el = 0;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        const int i = x.lane * C + j;
+        key[j] = INT_MIN;  // below every freeness key: not eligible
+        if (i < x.N && x.mrole[i] == MIG_NONE) {
+            key[j] = make_key(x, fnum(x, i), x.nrun[i]);
+            el |= 1u << j;
+        }
+        if (i < np) sk[i] = key[j];
+        lt[j] = eqb[j] = eqa[j] = 0;
+    }
+    const int nel = __reduce_add_sync(kFull, __popc(el));
+    __syncwarp();
+    if (nel < 2) return false;
+#pragma unroll 1
+    for (int m = 0; m < np; m += 4) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(sk + m);
+        const int kk[4] = {(int)w.x, (int)w.y, (int)w.z, (int)w.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                lt[j] += kk[u] < key[j] ? 1 : 0;
+                if (kk[u] == key[j]) {
+                    eqb[j] += m + u < x.lane * C + j ? 1 : 0;
+                    eqa[j] += m + u > x.lane * C + j ? 1 : 0;
+                }
+            }
+    }
+#pragma unroll
+    for (int j = 0; j < C; ++j)
+        if ((el >> j) & 1u) {
+            const int below = lt[j] - (np - nel);  // eligible ones
+            lo[below + eqb[j]] = (uint8_t)(x.lane * C + j);
+            hi[nel - 1 - below - eqa[j]] = (uint8_t)(x.lane * C + j);
+        }
+    __syncwarp();
+    bool started = false;
+    int k = 0, q = 0;  // next source and destination
+#pragma unroll 1
+    for (;;) {
+        int s = 0, d = 0;
+        bool ok = k + x.lane < nel;  // q <= k
+        if (ok) {
+            s = lo[k + x.lane];
+            d = hi[q + x.lane];
+            ok = sk[s] < sk[d] && over_theta(x, s, d, theta_num, theta_den);  // by the first: not moved yet
+        }
+        const uint32_t okm = __ballot_sync(kFull, ok);
+        const int cnt = okm == kFull ? 32 : __ffs(~okm) - 1;
+        if (cnt == 0) break;
+        const bool waits = x.lane < cnt && x.wmask[s] != 0;
+        const uint32_t wm = __ballot_sync(kFull, waits);
+        uint32_t run = (cnt == 32 ? kFull : (1u << cnt) - 1u) & ~wm;
+        const uint32_t base = x.tot[TOT_LOG];
+        int done = cnt;  // pairs of this batch that move
+        if (run) {
+            Slots2 v = load_slots(x, lo[k + __ffs(run) - 1]);
+#pragma unroll 1
+            do {
+                const int e = __ffs(run) - 1;
+                run &= run - 1;
+                Slots2 v2;
+                if (C != 2 && run) v2 = load_slots(x, lo[k + __ffs(run) - 1]);
+                if (!start_copy(x, lo[k + e], hi[q + e], v, base + (uint32_t)e)) {
+                    done = e;
+                    break;
+                }
+                started = true;
+                if (C == 2 && run) v2 = load_slots(x, lo[k + __ffs(run) - 1]);
+                v = v2;
+            } while (run);
+        }
+        if (waits && x.lane < done) move_queued(x, cn, s, d, base + (uint32_t)x.lane);
+        __syncwarp();
+        if (x.lane == 0) {
+            const uint32_t moved = done == 32 ? kFull : (1u << done) - 1u;
+            x.tot[TOT_LOG] = base + (uint32_t)done;
+            x.tot[TOT_MIG] += (uint32_t)__popc(wm & moved);
+            x.tot[TOT_START] += (uint32_t)__popc(~wm & moved);
+        }
+        __syncwarp();
+        if (done == cnt && cnt < 32) break;
+        q += done;
+        k += done < cnt ? done + 1 : cnt;
+    }
+    return started;
+}
+
 // Phase 3: periodic rebalancing between low- and high-freeness instances
 // (Sec. 3.5).  Returns whether a staged copy started.
 template <int C, bool EXT>
 __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_num, int theta_den) {
+    if (!MT_RARE(theta_num == 0) && !(EXT && x.drains)) return ranked_tick<C>(x, cn, theta_num, theta_den);
+    // Pair by pair: draining instances come first and without the threshold,
+    // and with theta = 0 equal freeness pairs up too.
     refresh_keys<C>(x);
     uint32_t el = 0, dr = 0;  // eligible (not migrating); draining
 #pragma unroll
@@ -1003,76 +1317,41 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
         }
         const int d = arg_ext<C>(x, el & ~dr, true, s);
         if (d < 0) break;
-        if (!dl) {
-            const long long ns = fnum(x, s), ds = max((int)x.nrun[s], 1);
-            const long long nd = fnum(x, d), dd = max((int)x.nrun[d], 1);
-            if ((long long)theta_den * (nd * ds - ns * dd) < (long long)theta_num * dd * ds) break;
-        }
+        if (!dl && !over_theta(x, s, d, theta_num, theta_den)) break;
         const bool has_wait = x.wmask[s] != 0;
-        const int n_s = x.nrun[s];
+        const uint32_t at = x.tot[TOT_LOG];
+        const Slots2 v = load_slots(x, s);
         __syncwarp();
-        int moved = 0;
+        bool moved = has_wait;
         if (has_wait) {
             if (x.lane == 0) {
-                // queued candidate: newest request of the lowest-priority bucket, no KV to copy
-                const int k = 31 - __clz((unsigned)x.wmask[s]);
-                uint32_t info = 0;
-                const uint32_t r = pop_back(x, s, k, info, cn.status);
-                if (r != kNone) {
-                    refresh_hol(x, s);
-                    cnt_dec(x, s, k);
-                    const uint32_t old = x.wmask[d];
-                    push_back(x, d, k, r, info);
-                    cnt_inc(x, d, k);
-                    if ((old & ((2u << k) - 1u)) == 0) x.hol[d] = blocks_for(x, info & 0xFFFFu);
-                    bump_mig(x, r);
-                    x.tot[TOT_MIG]++;
-                    log_ev(x, cn, SIM_EV_QUEUED, r, s, d, 0);
-                }
+                move_queued(x, cn, s, d, at);
+                x.tot[TOT_MIG]++;
             }
-            moved = 1;
-        } else if (n_s > 0) {
-            // running candidate: lowest priority, then fewest blocks, then newest
-            const uint4 *p = slot_ptr(x, s, 0);
-            const bool v0 = x.lane < n_s, v1 = x.lane + 32 < n_s;
-            const uint4 a0 = v0 ? p[x.lane] : make_uint4(0, 0, 0, 0);
-            const uint4 a1 = v1 ? p[x.lane + 32] : make_uint4(0, 0, 0, 0);
-            const int k0 = v0 ? (int)((sl_tier(a0) << 16) | (0xFFFFu - (uint32_t)sl_blocks(x, s, a0))) : -1;
-            const int k1 = v1 ? (int)((sl_tier(a1) << 16) | (0xFFFFu - (uint32_t)sl_blocks(x, s, a1))) : -1;
-            const int km = __reduce_max_sync(kFull, max(k0, k1));
-            const uint32_t c0 = (v0 && k0 == km) ? a0.x : 0u, c1 = (v1 && k1 == km) ? a1.x : 0u;
-            const uint32_t rid = __reduce_max_sync(kFull, max(c0, c1));
-            const int blocks = (int)(0xFFFFu - ((uint32_t)km & 0xFFFFu));
-            const uint32_t o0 = __ballot_sync(kFull, v0 && a0.x == rid);
-            const uint32_t o1 = __ballot_sync(kFull, v1 && a1.x == rid);
-            const int ol = o0 ? __ffs(o0) - 1 : __ffs(o1) - 1;
-            const bool hi = o0 == 0;
-            uint4 rec;
-            rec.x = __shfl_sync(kFull, hi ? a1.x : a0.x, ol);
-            rec.y = __shfl_sync(kFull, hi ? a1.y : a0.y, ol);
-            rec.z = __shfl_sync(kFull, hi ? a1.z : a0.z, ol);
-            rec.w = __shfl_sync(kFull, hi ? a1.w : a0.w, ol);
-            if (x.free_[d] >= blocks) {
-                if (x.lane == 0) {
-                    x.mrole[s] = MIG_SRC;
-                    x.mpeer[s] = (uint8_t)d;
-                    x.mreq[s] = rid;
-                    x.mcopied[s] = 0;
-                    x.mslot[s] = rec;
-                    x.mrole[d] = MIG_DST;
-                    x.mpeer[d] = (uint8_t)s;
-                    x.tot[TOT_START]++;
-                    log_ev(x, cn, SIM_EV_START, rid, s, d, blocks);
-                }
-                moved = 1;
-                started = true;
-            }
+        } else if (start_copy(x, s, d, v, at)) {
+            if (x.lane == 0) x.tot[TOT_START]++;
+            moved = started = true;
         }
+        if (moved && x.lane == 0) x.tot[TOT_LOG] = at + 1u;
         if (x.lane == s / C) el &= ~(1u << (s % C));
         if (moved && x.lane == d / C) el &= ~(1u << (d % C));
         __syncwarp();
     }
     return started;
+}
+
+// The tick as a function of its own: bit 0, a staged copy started; bit 1, an
+// inconsistency on this lane.
+template <int C, bool SMS, bool EXT>
+__device__ __noinline__ int tick_call(uint4 *node, uint32_t Q, int r, uint32_t t) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Params &p = *reinterpret_cast<const Params *>(smem);
+    Ctx x;
+    bind_ctx<SMS>(x, p, smem, node, Q, r, t);
+    Cnt cn;
+    cn.status = SIM_REPLICA_RUNNING;
+    const bool started = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den);
+    return (started ? 1 : 0) | (cn.status < 0 ? 2 : 0);
 }
 
 // The number of distinct times et[j] < t1 over the warp, for a window
@@ -1134,21 +1413,6 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *
         *reinterpret_cast<uint4 *>(dst + o) = *reinterpret_cast<const uint4 *>(src + o);
 }
 
-__device__ __forceinline__ void bind_blob(Ctx &x, const Layout &L, unsigned char *blob) {
-    unsigned char *ib = blob + L.inst;
-    x.busy.base = x.free_.base = x.resv.base = x.hol.base = x.hr.base = x.key.base = ib;
-    x.mreq.base = x.mcopied.base = x.nf.base = x.minfin.base = x.drain.base = ib;
-    x.wmask.base = x.nrun.base = x.pc.base = x.phase.base = x.mrole.base = x.mpeer.base = x.mpend.base = ib;
-    x.cnt = reinterpret_cast<uint16_t *>(blob + L.cnt);
-    x.head = reinterpret_cast<uint32_t *>(blob + L.head);
-    x.tail = reinterpret_cast<uint32_t *>(blob + L.tail);
-    x.hinfo = reinterpret_cast<uint32_t *>(blob + L.hinfo);
-    x.h = reinterpret_cast<int *>(blob + L.h);
-    x.hist = blob + L.hist;
-    x.mslot = reinterpret_cast<uint4 *>(blob + L.mslot);
-    x.tot = reinterpret_cast<uint32_t *>(blob + L.tot);
-}
-
 // Phase 1 at x.t for the instances in `mask` (bit j = instance lane*C + j)
 // whose iteration ends now, ascending index.  Collective.
 template <int C>
@@ -1176,8 +1440,8 @@ __device__ __forceinline__ void complete_all(const Ctx &x, Cnt &cn, uint32_t mas
 
 // Phase 4 at x.t for the idle instances in `mask` that have work, ascending
 // index, on lane 0.  Collective.
-template <int C>
-__device__ __forceinline__ void form_all(const Ctx &x, Cnt &cn, uint32_t mask, const Params &p) {
+template <int C, bool SMS, bool LEAN>
+__device__ __forceinline__ void form_all(Ctx &x, Cnt &cn, uint32_t mask, const Params &p) {
     uint32_t want = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
@@ -1190,19 +1454,9 @@ __device__ __forceinline__ void form_all(const Ctx &x, Cnt &cn, uint32_t mask, c
         lanes &= lanes - 1;
         const uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, want, l);
         if (x.lane == 0)
-            for (uint32_t hh = h; hh; hh &= hh - 1) inst_form(x, cn, l * C + __ffs(hh) - 1, p.base, p.a, p.b);
+            for (uint32_t hh = h; hh; hh &= hh - 1) inst_form<SMS, LEAN>(x, cn, l * C + __ffs(hh) - 1, p);
     }
     __syncwarp();
-}
-
-// a[j] for a run-time j without dynamic indexing (the array stays in registers)
-template <int C>
-__device__ __forceinline__ uint32_t pick_c(const uint32_t (&a)[C], int j) {
-    uint32_t v = a[0];
-#pragma unroll
-    for (int k = 1; k < C; ++k)
-        if (j == k) v = a[k];
-    return v;
 }
 
 // The events of a window [tb, t1) that can be taken in the next round, bit j =
@@ -1306,20 +1560,6 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
     return tb;
 }
 
-// Which variants run quiet windows in registers.
-template <int C, bool SMS>
-constexpr bool kQuiet = C == 1;
-
-// Which main loop a variant runs.  The variants that keep running-request
-// records in HBM with at most two instances per lane run 16 warps per SM
-// (many replicas); there instruction fetch was the bottleneck, and a loop
-// in which the window, its migration steps and the global steps share one
-// copy of every phase keeps the hot code small.  The other variants run few
-// warps per SM and are bound by each replica's dependent chain, which the
-// loop with separately inlined phases keeps shorter.
-template <int C, bool SMS>
-constexpr bool kUnifiedLoop = !SMS && C <= 2;
-
 // The persistent simulation kernel: each warp repeatedly takes a replica and
 // advances it by up to p.max_steps event times; C = instances per lane.
 //
@@ -1327,33 +1567,40 @@ constexpr bool kUnifiedLoop = !SMS && C <= 2;
 // instances that are in no migration do not interact, and an iteration lasts
 // at least `base` microseconds.  So in a window [tmin, min(T_g, tmin + base))
 // every instance ends at most one iteration, and each lane advances its own
-// instances (an O(1) iteration end + batch formation); instances in a
-// migration (but a destination whose source's next event comes later), and
-// every step at a global event, are advanced by the warp in the oracle's
-// order.  EXT: the variant that also handles draining instances and
-// the auto-scaling signal (the other variant compiles that code out).
-template <int C, bool SMS, bool EXT>
+// instances (an O(1) iteration end + batch formation), the two ends of a
+// migration in the order of their events (classify); every step at a global
+// event is advanced by the warp in the oracle's order.
+//
+// EXT: the variant that also handles draining instances and the auto-scaling
+// signal (the other variant compiles that code out).  MANY: the loop for more
+// replicas than a few warps per SM (plan_launch).  What bounds the two differs:
+// with few warps each replica's dependent chain, so the loop without MANY has
+// a straight path per kind of pass; with many, instruction fetch and registers
+// (64 instances: 14 % less code took 161 to 131 ms, 18 instead of 16 warps
+// another 14 %), so the MANY loop has one copy of every phase.
+//
 // Resident warps against registers, same-box A/B.  Two instances per lane,
-// records in HBM: a bound of 10 blocks compiles to 96 registers (no spills),
+// records in HBM: a bound of 10 blocks compiles to 96 registers (few spills),
 // and shared memory then holds 9 blocks of two warps: 113.6 ms on 8,192
 // replicas x 64 instances x 4,000 requests, against 131.0 ms with 8 blocks at
 // 124 registers.  (10 resident blocks, with 1 KB less of scratch per warp:
-// 110.4 ms; 12 blocks would need 80
-// registers, which spills.)  One instance per lane: 8 blocks (110 registers)
-// 20.8 ms on 3,840 x 32 x 1,000, 10 blocks 21.8 ms, 12 blocks (80 registers)
-// 21.9 ms.  The others are bound by one replica's chain.
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2 ? 10 : 8) k_run(Params p) {
+// 110.4 ms; 12 blocks would need 80 registers, which spills.)  One instance
+// per lane: 8 blocks (110 registers) 20.8 ms on 3,840 x 32 x 1,000, 10 blocks
+// 21.8 ms, 12 blocks (80 registers) 21.9 ms.
+template <int C, bool SMS, bool EXT, bool MANY>
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 : 8) k_run(Params p) {
+    // At 96 registers there is no room for values kept across calls: the rare
+    // paths stay inline (116 ms instead of 196 on the 64-instance sweep), and
+    // copy stages go source by source.
+    constexpr bool LEAN = MANY && C == 2;
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long *magic = reinterpret_cast<unsigned long long *>(smem);
+    unsigned long long *magic = reinterpret_cast<unsigned long long *>(smem + kParamBytes);
     for (int d = threadIdx.x; d <= 64; d += blockDim.x)
         magic[d] = d < 2 ? 0ull : ~0ull / (unsigned long long)d + 1ull;
+    if (threadIdx.x == 0) *reinterpret_cast<Params *>(smem) = p;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t slot_bytes = SMS ? (uint32_t)p.N * (uint32_t)p.Bmax * 16u : 0u;
-    const uint32_t per_warp = p.L.bytes + slot_bytes + (1u << p.set_bits);
-    unsigned char *blob = smem + kMagicBytes + (size_t)(threadIdx.x >> 5) * per_warp;
-    uint4 *sslots = reinterpret_cast<uint4 *>(blob + p.L.bytes);
-    uint32_t *tset = reinterpret_cast<uint32_t *>(blob + p.L.bytes + slot_bytes);
     for (;;) {
         int r = 0;
         if (lane == 0) {
@@ -1364,43 +1611,22 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
         if (r >= p.R) break;
         if (p.rep[r].status != SIM_REPLICA_RUNNING) continue;
         unsigned char *gblob = p.blobs + (size_t)r * p.L.bytes;
-        copy16(blob, gblob, p.L.bytes, lane);
-        Ctx x;
-        bind_blob(x, p.L, blob);
-        uint4 *g_slots = p.slots + (size_t)r * p.N * p.Bmax;
-        if (SMS) {
-            copy16(reinterpret_cast<unsigned char *>(sslots), reinterpret_cast<const unsigned char *>(g_slots),
-                   slot_bytes, lane);
-            x.slots = sslots;
-        } else {
-            x.slots = g_slots;
-        }
-        x.tset = tset;
-        x.set_bits = p.set_bits;
-        __syncwarp();
         const long long o = p.offsets[r];
-        x.Q = (uint32_t)(p.offsets[r + 1] - o);
-        x.node = p.node + o;
-        x.r = r;
-        x.arrival = p.arrival;
-        x.plen = p.plen;
-        x.olen = p.olen;
-        x.tier = p.tier;
-        x.node0 = p.node;
-        x.log0 = p.log;
-        x.res_off = p.res_off;
-        x.cap = p.cap;
-        x.magic = magic;
-        x.magT = p.magT;
-        x.N = p.N;
-        x.K = p.K;
-        x.T = p.T;
-        x.TH = p.TH;
-        x.Bmax = p.Bmax;
-        x.S = p.S;
-        x.lane = lane;
-        x.drains = EXT ? p.drains : 0;
-        x.t = p.rep[r].t;
+        Ctx x;
+        // The state's address stays in a register (the compiler would rather
+        // compute it again at every use: 130 instead of 116 ms on the 64-instance
+        // sweep, 9.54 instead of 9.43 ms on 1,024 x 16).
+        uint32_t zero = 0;
+        asm volatile("" : "+r"(zero));
+        bind_ctx<SMS>(x, p, smem + zero, p.node + o, (uint32_t)(p.offsets[r + 1] - o), r, p.rep[r].t);
+        if (!EXT) x.drains = 0;
+        unsigned char *blob = x.busy.base - p.L.inst;
+        uint4 *g_slots = p.slots + (size_t)r * p.N * p.Bmax;
+        copy16(blob, gblob, p.L.bytes, lane);
+        if (SMS)
+            copy16(reinterpret_cast<unsigned char *>(x.slots), reinterpret_cast<const unsigned char *>(g_slots),
+                   slot_bytes, lane);
+        __syncwarp();
         uint32_t tmax = x.t;  // latest event time this lane has processed (the replica's: max over lanes)
         Cnt cn;
         cn.finished = p.rep[r].finished;
@@ -1419,7 +1645,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
         ArrBuf ab;
         arr_refill(x, ab, cursor);
         uint32_t next_arr = __shfl_sync(kFull, ab.time, 0);
-        if constexpr (kUnifiedLoop<C, SMS>) {
+        if constexpr (MANY) {
             const uint32_t max_steps = p.max_steps;
             const uint32_t all = own_mask<C>(x);
             const bool ticks = EXT ? p.ticks != 0 : p.enable_mig != 0;
@@ -1474,7 +1700,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                     if (!any_b) {
                         tb = __reduce_min_sync(kFull, mb);
                         tg = ticks ? min(next_arr, next_tick) : next_arr;
-                        if (kQuiet<C, SMS> && !mig && tb < tg)
+                        if (C == 1 && !mig && tb < tg)
                             tb = run_quiet(x, cn, et[0], tb, tg, max_steps, tmax, p);
                     }
                     if (any_b || (tb < tg && max_steps - cn.steps > (uint32_t)x.N)) {
@@ -1519,38 +1745,56 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                         }
                     }
                 }
-                // ---- 1. iteration ends: each lane ends its own instances' iterations ----
-                uint32_t fz = 0;  // own instances with a finishing request (bits 0..C-1), sources (bits C..)
+                // ---- 1. iteration ends, finishes and copy stages: in mode 0 those of
+                // every instance together, in modes 1 and 2 instance by instance in
+                // ascending order ----
+                uint32_t todo = heads;
+                bool go = LEAN || mode == 0 || __any_sync(kFull, todo != 0);
+#pragma unroll 1
+                while (go) {
+                    uint32_t sel = todo;
+                    if (!LEAN && mode != 0) sel = lane == __ffs(__ballot_sync(kFull, todo != 0)) - 1 ? todo & (0u - todo) : 0u;
+                    todo &= ~sel;
+                    uint32_t fz = 0, src = 0;  // own instances with a finishing request; sources
 #pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    if (!((heads >> j) & 1u)) continue;
-                    const int i = lane * C + j;
-                    if (inst_complete_head(x, i)) fz |= 1u << j;
-                    if (mig && x.mrole[i] == MIG_SRC) fz |= 1u << (C + j);
-                }
-                __syncwarp();
-                // ---- finishes and copy stages, instance by instance in ascending
-                // order, by the whole warp ----
-                for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
-                    const int l = __ffs(fl) - 1;
-                    const uint32_t fzl = __shfl_sync(kFull, fz, l);
-                    for (uint32_t h = (fzl | (fzl >> C)) & ((1u << C) - 1u); h; h &= h - 1) {
-                        const int j = __ffs(h) - 1;
-                        const int i = l * C + j;
-                        x.t = __shfl_sync(kFull, pick_c<C>(et, j), l);
-                        if ((fzl >> j) & 1u) coop_finish(x, cn, i);
-                        if ((fzl >> (C + j)) & 1u) coop_stage(x, cn, i);
+                    for (int j = 0; j < C; ++j) {
+                        if (!((sel >> j) & 1u)) continue;
+                        const int i = lane * C + j;
+                        if (inst_complete_head(x, i)) fz |= 1u << j;
+                        if (mig && x.mrole[i] == MIG_SRC) src |= 1u << j;
                     }
+                    __syncwarp();
+                    if (LEAN) fz |= src << C;
+                    for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
+                        const int l = __ffs(fl) - 1;
+                        const uint32_t fzl = C == 1 && !LEAN ? 1u : __shfl_sync(kFull, fz, l);
+                        for (uint32_t h = LEAN ? (fzl | (fzl >> C)) & ((1u << C) - 1u) : fzl; h; h &= h - 1) {
+                            const int j = __ffs(h) - 1;
+                            x.t = __shfl_sync(kFull, pick_c<C>(et, j), l);
+                            if (!LEAN || ((fzl >> j) & 1u)) coop_finish(x, cn, l * C + j);
+                            if (LEAN && ((fzl >> (C + j)) & 1u)) coop_stage(x, cn, l * C + j);
+                        }
+                    }
+                    if (!LEAN && mig) stage_all<C>(x, cn, src, et);
+                    go = !LEAN && mode != 0 && __any_sync(kFull, todo != 0);
                 }
                 int dest = -1;
                 if (mode == 2) {
                     x.t = tstep;
-                    if (next_arr == tstep) dest = dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
+                    if (next_arr == tstep) dest = dispatch_phase<C, SMS, EXT, LEAN>(x, cn, cursor, next_arr, ab, p);  // 2. dispatch
                     if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                         const uint32_t nt = next_tick + p.interval;
                         next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                         if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
-                        if (p.enable_mig) mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
+                        if (p.enable_mig) {
+                        if (LEAN) {
+                            mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
+                        } else {
+                            const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
+                            mig = mig || (did & 1);
+                            if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
+                        }
+                    }
                     }
                 }
                 // ---- 4. batch formation: in mode 0 every lane forms its own
@@ -1581,7 +1825,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                         for (uint32_t h = hl; h; h &= h - 1) {
                             const int j = __ffs(h) - 1;
                             x.t = mode == 0 ? pick_c<C>(et, j) : tstep;
-                            inst_form(x, cn, owner * C + j, p.base, p.a, p.b);
+                            inst_form<SMS, LEAN>(x, cn, owner * C + j, p);
                         }
                     }
                     if (mode == 0) want = l == 0 ? heads : wake_hi;
@@ -1616,7 +1860,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                 uint32_t tb = __reduce_min_sync(kFull, mb);
                 const bool ticks = EXT ? p.ticks != 0 : p.enable_mig != 0;
                 const uint32_t tg = ticks ? min(next_arr, next_tick) : next_arr;
-                if (kQuiet<C, SMS> && !mig && tb < tg) tb = run_quiet(x, cn, bz[0], tb, tg, max_steps, tmax, p);
+                if (C == 1 && !mig && tb < tg) tb = run_quiet(x, cn, bz[0], tb, tg, max_steps, tmax, p);
                 if (tb < tg && max_steps - cn.steps > (uint32_t)x.N) {
                     // ---- window [tb, t1): at most one iteration end per instance ----
                     const uint32_t t1 =
@@ -1626,43 +1870,42 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
 #pragma unroll
                     for (int j = 0; j < C; ++j)
                         if (bz[j] < t1) tmax = max(tmax, bz[j]);
-                    // The iterations of the own instances in `sel` end; finishes and copy
-                    // stages follow, one instance at a time by the whole warp (each
-                    // touches only its own pair, so their order does not matter).
+                    // The iterations of the own instances in `sel` end; finishes follow, one
+                    // instance at a time by the whole warp (each touches only its own
+                    // pair, so their order does not matter), then copy stages.
                     auto ends = [&](uint32_t sel, bool stages) {
-                        uint32_t fz = 0;  // own instances with a finishing request (bits 0..C-1), sources (bits C..)
+                        uint32_t fz = 0, src = 0;  // own instances with a finishing request; sources
 #pragma unroll
                         for (int j = 0; j < C; ++j) {
                             if (!((sel >> j) & 1u)) continue;
                             const int i = lane * C + j;
                             if (inst_complete_head(x, i)) fz |= 1u << j;
-                            if (stages && x.mrole[i] == MIG_SRC) fz |= 1u << (C + j);
+                            if (stages && x.mrole[i] == MIG_SRC) src |= 1u << j;
                         }
                         __syncwarp();
                         for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
                             const int l = __ffs(fl) - 1;
-                            const uint32_t fzl = C == 1 && !stages ? 1u : __shfl_sync(kFull, fz, l);
-                            for (uint32_t h = (fzl | (stages ? fzl >> C : 0u)) & ((1u << C) - 1u); h; h &= h - 1) {
+                            for (uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, fz, l); h; h &= h - 1) {
                                 const int j = __ffs(h) - 1;
                                 x.t = __shfl_sync(kFull, pick_c<C>(bz, j), l);
-                                if (!stages || ((fzl >> j) & 1u)) coop_finish(x, cn, l * C + j);
-                                if (stages && ((fzl >> (C + j)) & 1u)) coop_stage(x, cn, l * C + j);
+                                coop_finish(x, cn, l * C + j);
                             }
                         }
+                        if (stages) stage_all<C>(x, cn, src, bz);
                     };
                     // Every lane forms its own instances' next batches.
                     auto forms = [&](uint32_t sel) {
                         if (C == 1) {
                             if (sel) {
                                 x.t = bz[0];
-                                inst_form(x, cn, lane, p.base, p.a, p.b);
+                                inst_form<SMS, LEAN>(x, cn, lane, p);
                             }
                         } else {
 #pragma unroll 1
                             for (uint32_t h = sel; h; h &= h - 1) {
                                 const int j = __ffs(h) - 1;
                                 x.t = pick_c<C>(bz, j);
-                                inst_form(x, cn, lane * C + j, p.base, p.a, p.b);
+                                inst_form<SMS, LEAN>(x, cn, lane * C + j, p);
                             }
                         }
                         __syncwarp();
@@ -1707,7 +1950,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                             if (tc >= t1) break;
                             x.t = tc;
                             complete_all<C>(x, cn, same);
-                            form_all<C>(x, cn, same, p);
+                            form_all<C, SMS, LEAN>(x, cn, same, p);
                             if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
                         }
                         x.hold = false;
@@ -1726,17 +1969,25 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
                 ++cn.steps;
                 if (tb == x.t) complete_all<C>(x, cn, all);  // 1. iteration ends
                 int dest = -1;
-                if (next_arr == x.t) dest = dispatch_phase<C, EXT>(x, cn, cursor, next_arr, ab);  // 2. dispatch
+                if (next_arr == x.t) dest = dispatch_phase<C, SMS, EXT, LEAN>(x, cn, cursor, next_arr, ab, p);  // 2. dispatch
                 if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                     const uint32_t nt = next_tick + p.interval;
                     next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
                     if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
-                    if (p.enable_mig) mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
+                    if (p.enable_mig) {
+                        if (LEAN) {
+                            mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
+                        } else {
+                            const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
+                            mig = mig || (did & 1);
+                            if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
+                        }
+                    }
                 }
                 // 4. batch formation.  After a lone arrival only its destination can
                 // have become able to form (an instance that stayed idle had nothing
                 // that fits, and nothing else changed).
-                if (tb == x.t || tick || dest < 0 || x.busy[dest] == kNone) form_all<C>(x, cn, all, p);
+                if (tb == x.t || tick || dest < 0 || x.busy[dest] == kNone) form_all<C, SMS, LEAN>(x, cn, all, p);
                 if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
             }
             __syncwarp();
@@ -1751,7 +2002,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, SMS || C > 2 ? 4 : C == 2
         for (int sh = 16; sh > 0; sh >>= 1) a_mi += __shfl_xor_sync(kFull, a_mi, sh);
         copy16(gblob, blob, p.L.bytes, lane);
         if (SMS)
-            copy16(reinterpret_cast<unsigned char *>(g_slots), reinterpret_cast<const unsigned char *>(sslots),
+            copy16(reinterpret_cast<unsigned char *>(g_slots), reinterpret_cast<const unsigned char *>(x.slots),
                    slot_bytes, lane);
         if (lane == 0) {
             RepState o2 = p.rep[r];  // this warp's until the launch ends
@@ -1916,13 +2167,14 @@ __global__ void k_export_stats(const RepState *rep, sim_replica_stats_t *out, in
 // ---- launch configuration ---------------------------------------------------
 typedef void (*RunKernel)(Params);
 
-template <bool SMS, bool EXT>
-RunKernel pick(int c) {  // c = instances per lane
+template <bool EXT>
+RunKernel pick(int c, bool sms, bool many) {  // c = instances per lane
+    if (many) return c == 1 ? k_run<1, false, EXT, true> : k_run<2, false, EXT, true>;
     switch (c) {
-        case 1: return k_run<1, SMS, EXT>;
-        case 2: return k_run<2, SMS, EXT>;
-        case 4: return k_run<4, SMS, EXT>;
-        default: return k_run<8, SMS, EXT>;
+        case 1: return sms ? k_run<1, true, EXT, false> : k_run<1, false, EXT, false>;
+        case 2: return sms ? k_run<2, true, EXT, false> : k_run<2, false, EXT, false>;
+        case 4: return sms ? k_run<4, true, EXT, false> : k_run<4, false, EXT, false>;
+        default: return sms ? k_run<8, true, EXT, false> : k_run<8, false, EXT, false>;
     }
 }
 
@@ -1981,12 +2233,17 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     const bool sms = slots_in_shared(N, Bmax);
     out.c = lanes_c(N);
     out.sms = sms;
-    out.fn = sms ? pick<true, false>(lanes_c(N)) : pick<false, false>(lanes_c(N));
-    out.fn_ext = sms ? pick<true, true>(lanes_c(N)) : pick<false, true>(lanes_c(N));
-    out.smem = kMagicBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << set_bits_for(N, sms)));
+    out.smem = kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << set_bits_for(N, sms)));
     int dev = 0, sms_count = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
+    // Which main loop: see k_run.  1,500 requests per replica, loop of many / of
+    // few, ms: 32 instances, 304 replicas 9.2 / 7.9, 1,216 9.9 / 9.0, 1,824 10.7 /
+    // 11.5, 2,432 11.4 / 20.1; 64 instances, 304 replicas 15.5 / 12.0, 1,824 18.8 /
+    // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).
+    const bool many = !sms && out.c <= 2 && R > (out.c == 1 ? 10 : 14) * sms_count;
+    out.fn = pick<false>(out.c, sms, many);
+    out.fn_ext = pick<true>(out.c, sms, many);
     const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
     for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
         RunKernel fn = v ? out.fn_ext : out.fn;
