@@ -302,9 +302,10 @@ int sim_metrics(sim_t *sim, sim_request_result_t *per_request, sim_replica_stats
  * requests that have finished, so it may be called between sim_run calls.
  * out is host or device per on_device, [R * max_tiers * 3] records.  Host
  * output synchronises the stream (and allocates a device staging buffer of
- * the same size on first use); device output is asynchronous.  The first
- * call also allocates the percentile selection scratch, 3,120 bytes per
- * (replica, tier, measure).  Returns SIM_ERR_STATE before sim_load_trace. */
+ * the same size on first use); device output is asynchronous.  When a replica
+ * has more requests than a block's shared memory holds (about 15,000 with 4
+ * tiers), the first call also allocates the percentile selection scratch,
+ * 3,120 bytes per (replica, tier, measure).  Returns SIM_ERR_STATE before sim_load_trace. */
 int sim_latency_stats(sim_t *sim, sim_latency_stats_t *out, int on_device);
 
 /* Releases everything the object owns (synchronises the stream first).

@@ -11,6 +11,7 @@ namespace {
 
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr uint32_t kFull = 0xFFFFFFFFu;
+constexpr size_t kMaxShared = 227u * 1024u;  // per block
 
 // Histogram bucket of a 32-bit value: v for v < 8, else eight equal buckets per
 // power of two: with e = floor(log2 v), 8 + 8 (e - 3) + (v >> (e - 3)) - 8.
@@ -125,62 +126,105 @@ __device__ __forceinline__ uint32_t *pct_field(sim_latency_stats_t *o, int q) {
 // Bit width of bucket b: values of bucket b are [lat_floor(b), lat_floor(b) + 2^w).
 __device__ __forceinline__ uint32_t lat_width_bits(uint32_t b) { return b < 8u ? 0u : (b - 8u) / 8u; }
 
-// Counts and the start of the nearest-rank P50 / P90 / P99 selection: one warp
-// per (replica, tier, measure).  The value of rank ceil(p n / 100) lies in the
-// bucket where the merged histogram's running count reaches that rank; the
-// selection state of percentile q is {floor of that bucket, its width in
-// bits, the rank among the values of the bucket}.  A bucket one value wide
-// gives the value at once; the others are narrowed by the selection passes.
+// The start of the nearest-rank P50 / P90 / P99 selection of one (replica,
+// tier, measure), by one warp whose lane l holds the counts c of buckets
+// [8 l, 8 l + 8) (240 = 30 lanes x 8).  The value of rank ceil(p n / 100)
+// lies in the bucket where the running count reaches that rank; the selection
+// state of percentile q is {floor of that bucket, its width in bits, the rank
+// among the values of the bucket}.  A bucket one value wide gives the value at
+// once; the others are narrowed by the selection passes.  Lane 0 writes the
+// states, the percentiles so far and the count.
+__device__ __forceinline__ void select_start(const uint32_t (&c)[8], sim_latency_stats_t *o, uint4 *sel) {
+    const int lane = threadIdx.x & 31;
+    uint32_t own = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) own += c[j];
+    uint32_t incl = own;
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, sh);
+        if (lane >= sh) incl += y;
+    }
+    const uint32_t n = __shfl_sync(kFull, incl, 31);
+    const uint32_t excl = incl - own;
+    const uint32_t pct[3] = {50u, 90u, 99u};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const uint32_t rank = n ? max(1u, (uint32_t)(((unsigned long long)pct[q] * n + 99u) / 100u)) : 0u;
+        uint4 st = make_uint4(0u, 0u, 0u, 0u);  // {low end, width bits, rank in the bucket, -}
+        const bool mine = n && excl < rank && rank <= incl;
+        if (mine) {
+            uint32_t cum = excl;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (st.z == 0u && cum + c[j] >= rank) {
+                    const uint32_t bj = (uint32_t)(lane * 8 + j);
+                    st = make_uint4(lat_floor(bj), lat_width_bits(bj), rank - cum, 0u);
+                }
+                cum += c[j];
+            }
+        }
+        const uint32_t who = __ballot_sync(kFull, mine);
+        const int src = who ? __ffs(who) - 1 : 0;
+        st.x = __shfl_sync(kFull, st.x, src);
+        st.y = __shfl_sync(kFull, st.y, src);
+        st.z = __shfl_sync(kFull, st.z, src);
+        if (lane == 0) {
+            if (!n) st = make_uint4(0u, 0u, 0u, 0u);
+            sel[q] = st;
+            *pct_field(o, q) = st.x;  // final when the bucket is one value wide
+        }
+    }
+    if (lane == 0) o->count = n;
+}
+
+// Narrows selection state st by one pass, by one warp whose lane l holds the
+// counts c of bins [8 l, 8 l + 8): the bin where the running count reaches the
+// rank, with the rank taken relative to it.  (Counts that disagree with the
+// rank close the state where it is.)
+__device__ __forceinline__ uint4 select_narrow(const uint32_t (&c)[8], const uint4 &st) {
+    const int lane = threadIdx.x & 31;
+    uint32_t own = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) own += c[j];
+    uint32_t incl = own;
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, sh);
+        if (lane >= sh) incl += y;
+    }
+    const uint32_t excl = incl - own;
+    const bool mine = excl < st.z && st.z <= incl;
+    uint32_t dig = 0, below = 0;
+    if (mine) {
+        uint32_t cum = excl;
+        bool got = false;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (!got && cum + c[j] >= st.z) { got = true; dig = (uint32_t)(lane * 8 + j); below = cum; }
+            cum += c[j];
+        }
+    }
+    const uint32_t who = __ballot_sync(kFull, mine);
+    if (!who) return make_uint4(st.x, 0u, st.z, 0u);
+    dig = __shfl_sync(kFull, dig, __ffs(who) - 1);
+    below = __shfl_sync(kFull, below, __ffs(who) - 1);
+    const uint32_t sh = st.y > 8u ? st.y - 8u : 0u;
+    return make_uint4(st.x + (dig << sh), sh, st.z - below, 0u);
+}
+
+// Counts and selection start of every (replica, tier, measure), one warp each.
 __global__ void k_latency_pct(long long ngroups, sim_latency_stats_t *out, uint4 *sel) {
     const int lane = threadIdx.x & 31;
     const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < ngroups; g += warps) {
-        sim_latency_stats_t *o = out + g;
-        // lane l holds buckets [8 l, 8 l + 8) (240 = 30 lanes x 8)
-        uint32_t c[8], own = 0;
+        uint32_t c[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int bj = lane * 8 + j;
-            c[j] = bj < SIM_HIST_BUCKETS ? o->hist[bj] : 0u;
-            own += c[j];
+            c[j] = bj < SIM_HIST_BUCKETS ? out[g].hist[bj] : 0u;
         }
-        uint32_t incl = own;
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, incl, sh);
-            if (lane >= sh) incl += y;
-        }
-        const uint32_t n = __shfl_sync(kFull, incl, 31);
-        const uint32_t excl = incl - own;
-        const uint32_t pct[3] = {50u, 90u, 99u};
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const uint32_t rank = n ? max(1u, (uint32_t)(((unsigned long long)pct[q] * n + 99u) / 100u)) : 0u;
-            uint4 st = make_uint4(0u, 0u, 0u, 0u);  // {low end, width bits, rank in the bucket, -}
-            const bool mine = n && excl < rank && rank <= incl;
-            if (mine) {
-                uint32_t cum = excl;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (st.z == 0u && cum + c[j] >= rank) {
-                        const uint32_t bj = (uint32_t)(lane * 8 + j);
-                        st = make_uint4(lat_floor(bj), lat_width_bits(bj), rank - cum, 0u);
-                    }
-                    cum += c[j];
-                }
-            }
-            const uint32_t who = __ballot_sync(kFull, mine);
-            const int src = who ? __ffs(who) - 1 : 0;
-            st.x = __shfl_sync(kFull, st.x, src);
-            st.y = __shfl_sync(kFull, st.y, src);
-            st.z = __shfl_sync(kFull, st.z, src);
-            if (lane == 0) {
-                if (!n) st = make_uint4(0u, 0u, 0u, 0u);
-                sel[g * 3 + q] = st;
-                *pct_field(o, q) = st.x;  // final when the bucket is one value wide
-            }
-        }
-        if (lane == 0) o->count = n;
+        select_start(c, out + g, sel + g * 3);
     }
 }
 
@@ -235,9 +279,8 @@ __global__ void k_latency_refine(const int *chunk_rep, const long long *chunk_b0
 }
 
 // Closes a selection pass: one warp per (group, percentile) still open reads
-// its bins, finds the bin where the running count reaches the rank, narrows
-// the range to that bin (rank taken relative to it) and clears the bins for
-// the next pass.  A range one value wide is the exact percentile.
+// its bins, narrows the range and clears the bins for the next pass.  A range
+// one value wide is the exact percentile.
 __global__ void k_latency_step(long long nstates, uint4 *sel, uint32_t *bins, sim_latency_stats_t *out) {
     const int lane = threadIdx.x & 31;
     const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -245,49 +288,217 @@ __global__ void k_latency_step(long long nstates, uint4 *sel, uint32_t *bins, si
         const uint4 st = sel[i];
         if (st.y == 0u) continue;
         uint32_t *bn = bins + (size_t)i * kSelBins;
-        uint32_t c[8], own = 0;  // lane l holds bins [8 l, 8 l + 8)
+        uint32_t c[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             c[j] = bn[lane * 8 + j];
-            own += c[j];
+            bn[lane * 8 + j] = 0u;
         }
-        uint32_t incl = own;
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, incl, sh);
-            if (lane >= sh) incl += y;
-        }
-        const uint32_t excl = incl - own;
-        const bool mine = excl < st.z && st.z <= incl;
-        uint32_t dig = 0, below = 0;
-        if (mine) {
-            uint32_t cum = excl;
-            bool got = false;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                if (!got && cum + c[j] >= st.z) { got = true; dig = (uint32_t)(lane * 8 + j); below = cum; }
-                cum += c[j];
-            }
-        }
-        const uint32_t who = __ballot_sync(kFull, mine);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) bn[lane * 8 + j] = 0u;
-        if (!who) {  // counts and rank disagree: stop here (the result keeps the range's low end)
-            if (lane == 0) sel[i].y = 0u;
-            continue;
-        }
-        dig = __shfl_sync(kFull, dig, __ffs(who) - 1);
-        below = __shfl_sync(kFull, below, __ffs(who) - 1);
+        const uint4 nx = select_narrow(c, st);
         if (lane == 0) {
-            const uint32_t sh = st.y > 8u ? st.y - 8u : 0u;
-            const uint4 nx = make_uint4(st.x + (dig << sh), sh, st.z - below, 0u);
             sel[i] = nx;
-            if (sh == 0u) *pct_field(out + i / 3, (int)(i % 3)) = nx.x;
+            if (nx.y == 0u) *pct_field(out + i / 3, (int)(i % 3)) = nx.x;
         }
     }
 }
 
+// All statistics of a replica by one block, its requests read once: the three
+// values and the tier of every request stay in shared memory for the selection
+// passes, whose bins (16-bit counts, two per word) are there too.  Dynamic
+// shared memory (replica_bytes): val [3][qcap], sums [warps][G], maxima
+// [warps][G], states [S], the histogram [G][SIM_HIST_BUCKETS] or, after it
+// has been written out, the bins [S][kSelBins / 2], tiers [qcap] (0x80: the
+// request has a TBT; kSkip: not finished).  Sums and maxima: per warp, one
+// reduction for each tier that the warp's 32 requests have, the sums in two
+// 16-bit halves (32 x 65,535 fits), so nothing is contended.
+// 1,024 replicas x 5,000 requests, K = 4 (130 MB): 192 us, of which about 80 in
+// the selection passes, 60 in the reductions and 50 in the read and the
+// histogram; the streaming passes take 294 us.  (Sums of up to 4 tiers in
+// registers 216 us; one look-up of the open percentiles per bucket instead of
+// nine range checks 203 us.)
+constexpr uint32_t kSkip = 0x7Fu;
+__global__ void __launch_bounds__(1024) k_latency_replica(int R, const long long *offsets, int KT,
+                                                          const uint32_t *arrival, const uint16_t *olen,
+                                                          const uint8_t *tier, const sim_request_result_t *res,
+                                                          sim_latency_stats_t *out, int qcap) {
+    extern __shared__ __align__(16) unsigned char lsm[];
+    const int G = KT * 3, S = G * 3, T = (int)blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
+    uint4 *st = reinterpret_cast<uint4 *>(lsm);                                                   // [S]
+    unsigned long long *wsum = reinterpret_cast<unsigned long long *>(st + S);                    // [nwarps][G]
+    uint32_t *wmax = reinterpret_cast<uint32_t *>(wsum + (size_t)nwarps * G);                     // [nwarps][G]
+    uint32_t *hist = wmax + (size_t)nwarps * G;                                                   // [G][240]
+    uint32_t *bins = hist;                                                                        // [S][128]
+    uint32_t *val = hist + (size_t)S * (kSelBins / 2);                                            // [3][qcap]
+    uint8_t *tr = reinterpret_cast<uint8_t *>(val + 3 * (size_t)qcap);                            // [qcap]
+    for (int r = blockIdx.x; r < R; r += gridDim.x) {
+        const long long b0 = offsets[r];
+        const int n = (int)(offsets[r + 1] - b0);
+        for (int q = threadIdx.x; q < G * SIM_HIST_BUCKETS; q += T) hist[q] = 0;
+        for (int q = threadIdx.x; q < nwarps * G; q += T) {
+            wsum[q] = 0;
+            wmax[q] = 0;
+        }
+        __syncthreads();
+        const uint4 *rs = reinterpret_cast<const uint4 *>(res + b0);
+        const uint32_t *ar = arrival + b0;
+        const uint16_t *ol = olen + b0;
+        const uint8_t *tp = tier + b0;
+        constexpr int U = 4;  // requests per thread per pass: their loads are issued together
+        for (int q0 = warp * 32; q0 < n; q0 += U * T) {  // uniform in a warp
+            uint4 rv[U];
+            uint32_t a[U], o[U], k[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + u * T + lane;
+                const bool in = q < n;
+                rv[u] = in ? rs[q] : make_uint4(0, 0, kNone, 0);
+                a[u] = in ? ar[q] : 0u;
+                o[u] = in ? (uint32_t)ol[q] : 0u;
+                k[u] = in ? (uint32_t)tp[q] : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (q0 + u * T >= n) break;
+                const int q = q0 + u * T + lane;
+                const uint32_t first = rv[u].y, fin = rv[u].z;
+                const bool ok = fin != kNone && k[u] < (uint32_t)KT;
+                const bool has_tbt = o[u] >= 2u;
+                uint32_t v[3];
+                v[0] = first - a[u];
+                v[1] = has_tbt ? (fin - first) / (o[u] - 1u) : 0u;
+                v[2] = fin - a[u];
+                if (q < n) tr[q] = (uint8_t)(ok ? k[u] | (has_tbt ? 0x80u : 0u) : kSkip);
+                if (ok) {
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        val[m * qcap + q] = v[m];
+                        if (m == 1 && !has_tbt) continue;  // a one-token request has no TBT
+                        atomicAdd(&hist[((int)k[u] * 3 + m) * SIM_HIST_BUCKETS + lat_bucket(v[m])], 1u);
+                    }
+                }
+                for (uint32_t todo = __ballot_sync(kFull, ok); todo;) {
+                    const uint32_t kk = __shfl_sync(kFull, k[u], __ffs(todo) - 1);
+                    const bool mine = ok && k[u] == kk;
+                    todo &= ~__ballot_sync(kFull, mine);
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {  // a request without TBT adds 0 there
+                        const uint32_t x = mine ? v[m] : 0u;
+                        const uint32_t slo = __reduce_add_sync(kFull, x & 0xFFFFu);
+                        const uint32_t shi = __reduce_add_sync(kFull, x >> 16);
+                        const uint32_t mx = __reduce_max_sync(kFull, x);
+                        if (lane == m) {
+                            const int at = warp * G + (int)kk * 3 + m;
+                            wsum[at] += (unsigned long long)slo + ((unsigned long long)shi << 16);
+                            wmax[at] = max(wmax[at], mx);
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // sums, maxima, histogram and selection start: one warp per group
+        sim_latency_stats_t *orow = out + (size_t)r * G;
+        bool open = false;
+        for (int g = warp; g < G; g += nwarps) {
+            unsigned long long sv = lane < nwarps ? wsum[lane * G + g] : 0ull;
+            uint32_t mv = lane < nwarps ? wmax[lane * G + g] : 0u;
+#pragma unroll
+            for (int sh = 16; sh > 0; sh >>= 1) sv += __shfl_xor_sync(kFull, sv, sh);
+            mv = __reduce_max_sync(kFull, mv);
+            sim_latency_stats_t *o = orow + g;
+            if (lane == 0) {
+                o->sum_us = sv;
+                o->max_us = mv;
+                o->pad = 0u;
+            }
+            for (int b = lane; b < SIM_HIST_BUCKETS; b += 32) o->hist[b] = hist[g * SIM_HIST_BUCKETS + b];
+            uint32_t c[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int bj = lane * 8 + j;
+                c[j] = bj < SIM_HIST_BUCKETS ? hist[g * SIM_HIST_BUCKETS + bj] : 0u;
+            }
+            select_start(c, o, st + g * 3);
+            __syncwarp();
+            open = open || st[g * 3].y != 0u || st[g * 3 + 1].y != 0u || st[g * 3 + 2].y != 0u;
+        }
+        // a bucket spans at most 2^28 values: four passes of 8 bits reach a single value
+        for (int pass = 0; pass < 4; ++pass) {
+            if (!__syncthreads_or(open ? 1 : 0)) break;  // uniform: every thread took part
+            if (pass == 0) {  // the histogram's space becomes the bins
+                for (int q = threadIdx.x; q < S * (kSelBins / 2); q += T) bins[q] = 0u;
+                __syncthreads();
+            }
+            for (int q = threadIdx.x; q < n; q += T) {
+                const uint32_t t = tr[q];
+                if (t == kSkip) continue;
+                const uint4 *s3 = st + (t & 0x1Fu) * 9u;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    if (m == 1 && !(t & 0x80u)) continue;
+                    const uint32_t v = val[m * qcap + q];
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) {
+                        const uint2 w = *reinterpret_cast<const uint2 *>(s3 + m * 3 + p);
+                        if (w.y == 0u || v - w.x >= (1u << w.y)) continue;
+                        const uint32_t bin = (v - w.x) >> (w.y > 8u ? w.y - 8u : 0u);
+                        atomicAdd(&bins[((t & 0x1Fu) * 9u + (uint32_t)(m * 3 + p)) * (kSelBins / 2) + (bin >> 1)],
+                                  1u << ((bin & 1u) * 16u));
+                    }
+                }
+            }
+            __syncthreads();
+            open = false;
+            for (int i = warp; i < S; i += nwarps) {
+                const uint4 s0 = st[i];
+                if (s0.y == 0u) continue;
+                uint4 *bn = reinterpret_cast<uint4 *>(bins + (size_t)i * (kSelBins / 2)) + lane;
+                const uint4 w = *bn;
+                *bn = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t c[8] = {w.x & 0xFFFFu, w.x >> 16, w.y & 0xFFFFu, w.y >> 16,
+                                       w.z & 0xFFFFu, w.z >> 16, w.w & 0xFFFFu, w.w >> 16};
+                const uint4 nx = select_narrow(c, s0);
+                __syncwarp();
+                if (lane == 0) {
+                    st[i] = nx;
+                    if (nx.y == 0u) *pct_field(orow + i / 3, i % 3) = nx.x;
+                }
+                open = open || nx.y != 0u;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+inline size_t replica_bytes(int qcap, int KT, int threads) {
+    const size_t G = (size_t)KT * 3, S = G * 3;
+    return S * 16 + (size_t)(threads / 32) * G * 12 + S * (kSelBins / 2) * 4 + (size_t)qcap * 13;
+}
+
 }  // namespace
+
+cudaError_t launch_replicas(int R, long long qmax, const long long *offsets, int KT, const uint32_t *arrival,
+                            const uint16_t *olen, const uint8_t *tier, const sim_request_result_t *res,
+                            sim_latency_stats_t *out, int sms, cudaStream_t stream, bool *done) {
+    *done = false;
+    if (qmax > 65535 / 4) return cudaSuccess;  // 16-bit bins, and shared memory
+    const int qcap = ((int)qmax + 15) & ~15;
+    const int threads = qmax <= 512 ? 128 : qmax <= 1024 ? 256 : qmax <= 8192 ? 512 : 1024;
+    const size_t smem = replica_bytes(qcap, KT, threads);
+    if (smem > kMaxShared) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024)
+        e = cudaFuncSetAttribute(k_latency_replica, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_latency_replica, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) return cudaSuccess;
+    const int grid = (int)std::min<long long>(R, (long long)sms * per_sm);
+    k_latency_replica<<<grid, threads, smem, stream>>>(R, offsets, KT, arrival, olen, tier, res, out, qcap);
+    *done = true;
+    return cudaGetLastError();
+}
 
 cudaError_t launch(const int *chunk_rep, const long long *chunk_b0, int nchunks, const long long *offsets, int KT,
                    const uint32_t *arrival, const uint16_t *olen, const uint8_t *tier,

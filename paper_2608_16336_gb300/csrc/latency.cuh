@@ -22,6 +22,14 @@ constexpr int kSelBins = 256;
 inline size_t select_state_bytes(long long ngroups) { return (size_t)ngroups * 3u * 16u; }
 inline size_t select_bin_bytes(long long ngroups) { return (size_t)ngroups * 3u * kSelBins * 4u; }
 
+// All statistics of R replicas with at most qmax requests each, one block per
+// replica, every request read once (no scratch).  *done is false, with nothing
+// queued, when a replica's values do not fit in shared memory; launch() below
+// takes any size.  out needs no clearing.
+cudaError_t launch_replicas(int R, long long qmax, const long long *offsets, int KT, const uint32_t *arrival,
+                            const uint16_t *olen, const uint8_t *tier, const sim_request_result_t *res,
+                            sim_latency_stats_t *out, int sms, cudaStream_t stream, bool *done);
+
 // Queues on `stream`: clear out ([ngroups] records, ngroups = R * KT * 3),
 // histogram, sum and maximum of every (replica, tier, measure) group, the
 // counts, the bucket of every percentile's rank, then the selection passes

@@ -2685,40 +2685,52 @@ int sim_latency_stats(sim_t *s, sim_latency_stats_t *out, int on_device) {
         }
         d = s->d_lat;
     }
-    if (s->lat_nchunks < 0) {  // chunk table of the loaded trace
-        std::vector<int> rep;
-        std::vector<long long> b0;
-        for (int r = 0; r < R; ++r)
-            for (long long b = s->h_off[r]; b < s->h_off[r + 1]; b += mtlat::kChunk) {
-                rep.push_back(r);
-                b0.push_back(b);
+    // Replicas whose values fit in a block's shared memory (about 15,000 requests
+    // with 4 tiers) take one kernel, larger ones the streaming passes.  One
+    // kernel / streaming, us: 1 replica x 64 requests 22 / 56, 1 x 14,000 75 / 95,
+    // 1,024 x 5,000 192 / 294, 1,024 x 14,000 473 / 528, 3,840 x 1,000 with 10
+    // tiers 441 / 792, 700 x 4,000 with 16 tiers 382 / 413.
+    long long qmax = 0;
+    for (int r = 0; r < R; ++r) qmax = std::max<long long>(qmax, s->h_off[r + 1] - s->h_off[r]);
+    bool done = false;
+    cudaError_t e = mtlat::launch_replicas(R, qmax, s->d_off, KT, s->d_arrival, s->d_olen, s->d_tier, s->d_res, d,
+                                           s->sms, s->stream, &done);
+    if (e != cudaSuccess) return cuda_fail(s, e, "sim_latency_stats");
+    if (!done) {
+        if (s->lat_nchunks < 0) {  // chunk table of the loaded trace
+            std::vector<int> rep;
+            std::vector<long long> b0;
+            for (int r = 0; r < R; ++r)
+                for (long long b = s->h_off[r]; b < s->h_off[r + 1]; b += mtlat::kChunk) {
+                    rep.push_back(r);
+                    b0.push_back(b);
+                }
+            const int nc = (int)rep.size();
+            dfree(s, s->d_lat_rep);
+            dfree(s, s->d_lat_b0);
+            s->d_lat_rep = nullptr;
+            s->d_lat_b0 = nullptr;
+            if (nc > 0) {
+                s->d_lat_rep = (int *)dalloc(s, (size_t)nc * 4);
+                s->d_lat_b0 = (long long *)dalloc(s, (size_t)nc * 8);
+                if (!s->d_lat_rep || !s->d_lat_b0) return fail(s, SIM_ERR_OOM, "device allocation of the chunk table failed");
+                e = cudaMemcpyAsync(s->d_lat_rep, rep.data(), (size_t)nc * 4, cudaMemcpyHostToDevice, s->stream);
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(s->d_lat_b0, b0.data(), (size_t)nc * 8, cudaMemcpyHostToDevice, s->stream);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // the host vectors go out of scope
+                if (e != cudaSuccess) return cuda_fail(s, e, "sim_latency_stats chunk table");
             }
-        const int nc = (int)rep.size();
-        dfree(s, s->d_lat_rep);
-        dfree(s, s->d_lat_b0);
-        s->d_lat_rep = nullptr;
-        s->d_lat_b0 = nullptr;
-        if (nc > 0) {
-            s->d_lat_rep = (int *)dalloc(s, (size_t)nc * 4);
-            s->d_lat_b0 = (long long *)dalloc(s, (size_t)nc * 8);
-            if (!s->d_lat_rep || !s->d_lat_b0) return fail(s, SIM_ERR_OOM, "device allocation of the chunk table failed");
-            cudaError_t e = cudaMemcpyAsync(s->d_lat_rep, rep.data(), (size_t)nc * 4, cudaMemcpyHostToDevice, s->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(s->d_lat_b0, b0.data(), (size_t)nc * 8, cudaMemcpyHostToDevice, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // the host vectors go out of scope
-            if (e != cudaSuccess) return cuda_fail(s, e, "sim_latency_stats chunk table");
+            s->lat_nchunks = nc;
         }
-        s->lat_nchunks = nc;
+        if (!s->d_lat_sel) {
+            s->d_lat_sel = (uint4 *)dalloc(s, mtlat::select_state_bytes((long long)n));
+            s->d_lat_bins = (uint32_t *)dalloc(s, mtlat::select_bin_bytes((long long)n));
+            if (!s->d_lat_sel || !s->d_lat_bins)
+                return fail(s, SIM_ERR_OOM, "device allocation of the percentile selection scratch failed");
+        }
+        e = mtlat::launch(s->d_lat_rep, s->d_lat_b0, s->lat_nchunks, s->d_off, KT, s->d_arrival, s->d_olen, s->d_tier,
+                          s->d_res, d, (long long)n, s->d_lat_sel, s->d_lat_bins, s->sms, s->stream);
     }
-    if (!s->d_lat_sel) {
-        s->d_lat_sel = (uint4 *)dalloc(s, mtlat::select_state_bytes((long long)n));
-        s->d_lat_bins = (uint32_t *)dalloc(s, mtlat::select_bin_bytes((long long)n));
-        if (!s->d_lat_sel || !s->d_lat_bins)
-            return fail(s, SIM_ERR_OOM, "device allocation of the percentile selection scratch failed");
-    }
-    cudaError_t e = mtlat::launch(s->d_lat_rep, s->d_lat_b0, s->lat_nchunks, s->d_off, KT, s->d_arrival, s->d_olen,
-                                  s->d_tier, s->d_res, d, (long long)n, s->d_lat_sel, s->d_lat_bins, s->sms,
-                                  s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "sim_latency_stats");
     if (!on_device) {
         e = cudaMemcpyAsync(out, d, n * sizeof(sim_latency_stats_t), cudaMemcpyDeviceToHost, s->stream);

@@ -1,0 +1,50 @@
+"""Latency statistics at the edges of the one-kernel path (replicas of 0 to
+16,383 requests, the block sizes it changes at, ragged warps, the tier counts
+whose shared memory differs, all values alike) and just past it, bit-exact
+against sorted values."""
+import numpy as np
+import pytest
+
+from paper_2608_16336_gb300 import workloads as W
+from tests.test_latency_gpu import compare, gpu_stats
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def _workload(sizes, k, alike, seed):
+    rng = np.random.default_rng(seed)
+    traces = []
+    for q in sizes:
+        a = np.cumsum(rng.integers(0, 120, q)).astype(np.uint32)
+        p, o = rng.integers(1, 200, q), rng.integers(1, 9, q)
+        traces.append((a, p.astype(np.uint16), o.astype(np.uint16), rng.integers(0, k, q).astype(np.uint8)))
+    b = 0 if alike else 5
+    return W.custom(2, 4096, [k], [[64 >> i for i in range(k)]], [0] * len(sizes), traces, iter_base_us=300,
+                    iter_us_per_prefill_token=b, iter_us_per_decode_seq=b)
+
+
+@pytest.mark.parametrize("sizes", [(0, 1, 2, 31, 32, 33, 512), (511, 513, 0, 1024), (1025, 3, 8192), (8193, 129)])
+@pytest.mark.parametrize("k", [1, 4, 5, 16])
+def test_sizes(sizes, k):
+    w = _workload(sizes, k, False, 7 * k + len(sizes))
+    compare(w, gpu_stats(w), range(len(sizes)))
+
+
+@pytest.mark.parametrize("q", [16383, 16384])
+@pytest.mark.parametrize("alike", [False, True])
+def test_largest(q, alike):
+    w = _workload((q,), 1, alike, q)
+    compare(w, gpu_stats(w), [0])
+
+
+def test_unfinished_requests_left_out():
+    w = _workload((700, 40), 3, False, 3)
+    compare(w, gpu_stats(w, max_steps=150), range(2), max_steps=150)
