@@ -247,6 +247,7 @@ struct Cnt {
     uint32_t finished, steps, iterations;
     uint64_t member_iterations;
     int status;
+    bool held;  // this lane has held back a log record in the open window
 };
 
 // The block's dynamic shared memory: a copy of the parameters (for the
@@ -428,12 +429,14 @@ __device__ __forceinline__ void log_end(const Ctx &x, Cnt &cn, int kind, uint32_
         x.mslot[s] = make_uint4(x.t, r, (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24),
                                 (uint32_t)kind);
         x.mpend[s] = (uint8_t)ph;
+        cn.held = true;
     } else {
         log_ev(x, cn, kind, r, s, d, blocks);
     }
 }
-// Closes a window with migrations: writes the records held back, and returns
-// whether some instance is still in a migration.  Collective.
+// Writes the records held back in a window that some lane has, and returns
+// whether some instance is still in a migration (one ends only with such a
+// record).  Collective.
 template <int C>
 __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
     uint32_t left = 0;
@@ -468,6 +471,7 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
             if (k < (uint32_t)x.cap) *x.log(k) = x.mslot[s];
         }
     }
+    cn.held = false;
     __syncwarp();
     return mig;
 }
@@ -583,24 +587,24 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
     const bool f0 = v0 && sl_fin(a0) == nf, f1 = v1 && sl_fin(a1) == nf;
     if (f0) { x.res(a0.x)->finish_us = x.t; x.res(a0.x)->final_instance = (uint16_t)i; }
     if (f1) { x.res(a1.x)->finish_us = x.t; x.res(a1.x)->final_instance = (uint16_t)i; }
-    const int freed = __reduce_add_sync(kFull, (f0 ? sl_blocks(x, i, a0) : 0) + (f1 ? sl_blocks(x, i, a1) : 0));
     const uint32_t m0 = __ballot_sync(kFull, f0), m1 = __ballot_sync(kFull, f1);
     // each finishing request is booked by the lane that holds it, in turn
 #pragma unroll 1
     for (uint64_t m = ((uint64_t)m1 << 32) | m0; m; m &= m - 1) {
         const int l = __ffsll((long long)m) - 1;
         if (x.lane == (l & 31)) {
-            const uint32_t rid = l & 32 ? a1.x : a0.x, w = l & 32 ? a1.w : a0.w;
-            cnt_dec(x, i, (int)(w & 0xFFu));
-            x.hist[i * x.TH + (w >> 16)]--;
-            if (MT_RARE(x.mrole[i] == MIG_SRC && x.mreq[i] == rid)) abort_mig(x, cn, i, 1);
+            const uint4 a = l & 32 ? a1 : a0;
+            x.free_[i] += sl_blocks(x, i, a);
+            cnt_dec(x, i, (int)sl_tier(a));
+            x.hist[i * x.TH + sl_rho(a)]--;
+            if (MT_RARE(x.mrole[i] == MIG_SRC && x.mreq[i] == a.x)) abort_mig(x, cn, i, 1);
         }
         __syncwarp();
     }
     const bool k0 = v0 && !f0, k1 = v1 && !f1;
-    const uint32_t e0 = __ballot_sync(kFull, k0), e1 = __ballot_sync(kFull, k1);
+    // places of the survivors: their old ones less the finishers before them
     const uint32_t below = (1u << x.lane) - 1u;
-    const int p0 = __popc(e0 & below), p1 = __popc(e0) + __popc(e1 & below);
+    const int p0 = q0 - __popc(m0 & below), p1 = q1 - __popc(m0) - __popc(m1 & below);
     const uint32_t fm = __reduce_min_sync(kFull, min(k0 ? sl_fin(a0) : kNone, k1 ? sl_fin(a1) : kNone));
     __syncwarp();
     if (k0 && p0 != q0) p[p0] = a0;  // only the records that move are written
@@ -608,8 +612,7 @@ __device__ __forceinline__ void coop_finish(const Ctx &x, Cnt &cn, int i) {
     const uint32_t nfin = __popc(m0) + __popc(m1);
     cn.finished += nfin;
     if (x.lane == 0) {
-        x.free_[i] += freed;
-        x.nrun[i] = (uint8_t)(__popc(e0) + __popc(e1));
+        x.nrun[i] = (uint8_t)(n - (int)nfin);
         x.minfin[i] = fm;
     }
     __syncwarp();
@@ -831,13 +834,15 @@ __device__ __forceinline__ void grow_slow(const Ctx &x, Cnt &cn, int i) {
 }
 
 template <bool SMS>
-__device__ __noinline__ void grow_call(uint4 *node, uint32_t Q, int r, uint32_t t, int i, bool hold) {
+__device__ __noinline__ bool grow_call(uint4 *node, uint32_t Q, int r, uint32_t t, int i, bool hold) {
     extern __shared__ __align__(16) unsigned char smem[];
     Ctx x;
     bind_ctx<SMS>(x, *reinterpret_cast<const Params *>(smem), smem, node, Q, r, t);
     x.hold = hold;
     Cnt cn;
+    cn.held = false;
     grow_slow(x, cn, i);
+    return cn.held;
 }
 
 // Phase 4: batch formation at idle instance i at x.t (Sec. 2.2, Sec. 3.1):
@@ -862,7 +867,7 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
             if (LEAN) {
                 grow_slow(x, cn, i);
             } else {
-                grow_call<SMS>(x.node, x.Q, x.r, x.t, i, x.hold);
+                cn.held |= grow_call<SMS>(x.node, x.Q, x.r, x.t, i, x.hold);
             }
             n = x.nrun[i];  // preemptions changed the running list, the free blocks, queues and head of line
             fr = x.free_[i];
@@ -1660,6 +1665,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
         cn.iterations = 0;
         cn.member_iterations = 0;
         cn.status = SIM_REPLICA_RUNNING;
+        cn.held = false;
         uint32_t cursor = p.rep[r].cursor;
         uint32_t next_tick = p.rep[r].next_tick;
         x.hold = false;
@@ -1863,10 +1869,12 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                     // the window closes
                     in_cm = false;
                     x.hold = false;
-                    if (mig) mig = flush_held<C>(x, cn);
                     cn.steps += ucount;
                 }
-                if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
+                if (__any_sync(kFull, cn.held || cn.status < 0)) {
+                    if (mode == 0 || mode == 3) mig = flush_held<C>(x, cn);
+                    if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
+                }
             }
             __syncwarp();
         } else {
@@ -1981,10 +1989,12 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                             if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
                         }
                         x.hold = false;
-                        mig = flush_held<C>(x, cn);
                     }
                     cn.steps += ucount;
-                    if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
+                    if (__any_sync(kFull, cn.held || cn.status < 0)) {
+                        mig = flush_held<C>(x, cn);
+                        if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
+                    }
                     continue;
                 }
                 // ---- one step at the next event time (global events, or near the step limit) ----
