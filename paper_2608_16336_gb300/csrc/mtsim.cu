@@ -75,8 +75,9 @@ constexpr int kWarpsPerBlock = 2;
 constexpr int kMaxBlockTokens = 64;      // T limit of the per-instance growth histogram
 constexpr uint32_t kMagicBytes = 528;    // ceil(2^64 / d) for d = 0..64, rounded up to 16 bytes
 // Bytes (2^n) of the per-warp scratch that counts a window's distinct event
-// times (distinct_times): small where many warps share an SM's shared memory.
-constexpr int kSetBitsShared = 12, kSetBits = 11;
+// times (distinct_times): small where many warps share an SM's shared memory
+// (plan_launch).
+constexpr int kSetBitsShared = 12, kSetBits = 11, kSetBitsMany = 10;
 
 enum : int { MIG_NONE = 0, MIG_SRC = 1, MIG_DST = 2 };
 
@@ -2223,6 +2224,7 @@ struct Launch {
     int per_sm = 0, per_sm_ext = 0;  // resident blocks per SM of each variant
     int c = 1;                       // instances per lane
     bool sms = false;                // running-request records in shared memory
+    int set_bits = 0;                // scratch of distinct_times, log2 of its bytes
     size_t smem = 0;
 };
 
@@ -2257,8 +2259,6 @@ inline Layout make_layout(int N, int K, int T) {
     return L;
 }
 
-// Size of the per-warp scratch of distinct_times, log2 of its bytes.
-inline int set_bits_for(int N, bool sms) { return sms || lanes_c(N) > 2 ? kSetBitsShared : kSetBits; }
 
 // Chooses the kernel variant and grid for a problem; cudaSuccess or the error.
 // Running-request records go to shared memory while a replica's take at most this many bytes.
@@ -2270,7 +2270,6 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     const bool sms = slots_in_shared(N, Bmax);
     out.c = lanes_c(N);
     out.sms = sms;
-    out.smem = kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << set_bits_for(N, sms)));
     int dev = 0, sms_count = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
@@ -2279,6 +2278,12 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     // 11.5, 2,432 11.4 / 20.1; 64 instances, 304 replicas 15.5 / 12.0, 1,824 18.8 /
     // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).
     const bool many = !sms && out.c <= 2 && R > (out.c == 1 ? 10 : 14) * sms_count;
+    // The scratch: 4 KB holds a window of the default `base` of 4 ms directly.
+    // Where two instances per lane share an SM with 17 other warps it has 2 KB,
+    // and 1 KB, with two warps more, for sweeps of several waves (8,192 x 64:
+    // 110.2 against 112.5 ms).
+    out.set_bits = sms || out.c > 2 ? kSetBitsShared : many && out.c == 2 && R > 26 * sms_count ? kSetBitsMany : kSetBits;
+    out.smem = kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << out.set_bits));
     out.fn = pick<false>(out.c, sms, many);
     out.fn_ext = pick<true>(out.c, sms, many);
     const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
@@ -2428,7 +2433,6 @@ void fill_scalars(mt::Params &p, const sim_cluster_t &cl, const sim_policy_t &po
     p.lcm_lo = (unsigned long long)l;
     p.lcm_hi = (unsigned long long)(l >> 64);
     p.L = L;
-    p.set_bits = mt::set_bits_for(cl.num_instances, mt::slots_in_shared(cl.num_instances, cl.max_batch));
 }
 
 mt::Params make_params(const sim_t *s, long long max_steps) {
@@ -2451,6 +2455,7 @@ mt::Params make_params(const sim_t *s, long long max_steps) {
     p.log = s->d_log;
     p.work = s->d_work;
     p.order = s->d_order;
+    p.set_bits = s->launch.set_bits;
     return p;
 }
 
@@ -3020,6 +3025,7 @@ extern "C" int sim_run_static(const sim_cluster_t *cl, const sim_tier_table_t *t
     p.rep = (mt::RepState *)(base + o_rep);
     p.log = events;
     p.work = (int *)(base + o_work);
+    p.set_bits = lc.set_bits;
     int *rt = (int *)(base + o_rt), *tk = (int *)(base + o_tk), *th = (int *)(base + o_th);
 
     // Inputs the kernels read from device memory; the work counter and flags start at zero.

@@ -38,10 +38,10 @@ def test_tick(n, theta):
     assert int(st["log_events"].sum()) > 0
 
 
-@pytest.mark.parametrize("n,replicas", [(30, 1519), (30, 1521), (40, 2127), (40, 2129)])
+@pytest.mark.parametrize("n,replicas", [(30, 1519), (30, 1521), (40, 2127), (40, 2129), (40, 3951), (40, 3953)])
 def test_both_loops(n, replicas):
     """One per lane and two per lane, records in HBM, around the replica counts
-    where a 152-SM GPU changes loops; sampled replicas against the oracle."""
+    where a 152-SM GPU changes loops and scratch; sampled replicas against the oracle."""
     rng = np.random.default_rng(replicas)
     traces = [_trace(rng, n, 40, 2, r % 2 == 0) for r in range(replicas)]
     w = W.custom(n, 90, [2], [[18, 9]], [0] * replicas, traces, tokens_per_block=4, max_batch=64, iter_base_us=200,
