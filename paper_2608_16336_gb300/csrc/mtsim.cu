@@ -9,9 +9,9 @@
 //   request counts, headroom table) lives in shared memory, and so do the
 //   running-request slots when they fit; everything is written back to HBM
 //   when the warp stops (step limit or completion), so sim_run can be resumed.
-//   Instances are spread over lanes in contiguous blocks of C = ceil(N/32) per
-//   lane (C is a template parameter), so "lowest lane" order is "lowest
-//   instance" order.  Per-request state stays in HBM: the read-only trace
+//   Instance i belongs to lane i mod 32, C = ceil(N/32) instances per lane (C
+//   is a template parameter, rounded up to a power of two); where the order of
+//   instances matters, it is taken from their indices.  Per-request state stays in HBM: the read-only trace
 //   (SoA), the 16-byte result record and a 16-byte queue node that threads a
 //   waiting request into its (instance, tier) FCFS bucket.  A running request
 //   is a 16-byte slot record that is written when it joins a batch and read
@@ -332,11 +332,20 @@ __device__ __forceinline__ int fnum(const Ctx &x, int i) { return x.free_[i] - x
 
 __device__ __forceinline__ void set_key(const Ctx &x, int i) { x.key[i] = make_key(x, fnum(x, i), x.nrun[i]); }
 
+// Instance j of a lane (j < C) and back.  Consecutive lanes own consecutive
+// instances, so their records (13 words each) lie in different shared-memory
+// banks.  (With C consecutive instances per lane they were C x 13 words apart,
+// a 2- to 8-way conflict for every access of all lanes: 64 x 256 63.0 -> 59.2
+// ms, 256 x 128 41.6 -> 40.8, 97 x 33 10.6 -> 10.1; 8,192 x 64 108.8 -> 109.3.)
+__device__ __forceinline__ int inst_at(int lane, int j) { return lane + 32 * j; }
+__device__ __forceinline__ int lane_of(int i) { return i & 31; }
+__device__ __forceinline__ int num_of(int i) { return i >> 5; }
+
 template <int C>
 __device__ __forceinline__ void refresh_keys(const Ctx &x) {
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (i < x.N) set_key(x, i);
     }
     __syncwarp();
@@ -347,19 +356,19 @@ __device__ __forceinline__ uint32_t own_mask(const Ctx &x) {
     uint32_t m = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j)
-        if (x.lane * C + j < x.N) m |= 1u << j;
+        if (inst_at(x.lane, j) < x.N) m |= 1u << j;
     return m;
 }
 
 // Arg-max (want_max) or arg-min of the freeness key over the instances whose
-// bit is set in `el` (bit j = instance lane*C + j), excluding `excl`; lowest
+// bit is set in `el` (bit j = the lane's instance j), excluding `excl`; lowest
 // index on ties; -1 if none.  Collective.
 template <int C>
 __device__ __forceinline__ int arg_ext(const Ctx &x, uint32_t el, bool want_max, int excl) {
     int bv = want_max ? INT_MIN : INT_MAX, bi = -1;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (((el >> j) & 1u) && i != excl) {
             const int k = x.key[i];
             if (bi < 0 || (want_max ? k > bv : k < bv)) { bv = k; bi = i; }
@@ -444,7 +453,7 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
     bool mig = false;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (i < x.N && x.mpend[i] != 0) left |= 1u << j;
         if (i < x.N && x.mrole[i] != MIG_NONE) mig = true;
     }
@@ -454,17 +463,17 @@ __device__ __forceinline__ bool flush_held(const Ctx &x, Cnt &cn) {
         uint32_t bt = kNone;
 #pragma unroll
         for (int j = 0; j < C; ++j)
-            if ((left >> j) & 1u) bt = min(bt, x.mslot[x.lane * C + j].x);
+            if ((left >> j) & 1u) bt = min(bt, x.mslot[inst_at(x.lane, j)].x);
         const uint32_t t = __reduce_min_sync(kFull, bt);
         uint32_t bk = kNone;
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-            const int i = x.lane * C + j;
+            const int i = inst_at(x.lane, j);
             if (((left >> j) & 1u) && x.mslot[i].x == t) bk = min(bk, ((uint32_t)x.mpend[i] << 16) | (uint32_t)i);
         }
         const int s = (int)(__reduce_min_sync(kFull, bk) & 0xFFFFu);
-        if (x.lane == s / C) {
-            left &= ~(1u << (s % C));
+        if (x.lane == lane_of(s)) {
+            left &= ~(1u << num_of(s));
             x.mpend[s] = 0;
         }
         if (x.lane == 0) {
@@ -706,7 +715,7 @@ __device__ __forceinline__ void stage_all(Ctx &x, Cnt &cn, uint32_t src, const u
     for (int j = 0; j < C; ++j) {
         if (!((src >> j) & 1u)) continue;
         x.t = et[j];
-        if (stage_copy(x, cn, x.lane * C + j)) due |= 1u << j;
+        if (stage_copy(x, cn, inst_at(x.lane, j))) due |= 1u << j;
     }
     __syncwarp();
     uint32_t lanes = __ballot_sync(kFull, due != 0), h = 0;
@@ -720,7 +729,7 @@ __device__ __forceinline__ void stage_all(Ctx &x, Cnt &cn, uint32_t src, const u
         }
         const int j = __ffs(h) - 1;
         h &= h - 1;
-        return l * C + j;
+        return inst_at(l, j);
     };
     int s = next();
     if (s < 0) return;
@@ -730,8 +739,8 @@ __device__ __forceinline__ void stage_all(Ctx &x, Cnt &cn, uint32_t src, const u
         const int s2 = next();
         Slots2 v2;
         if (s2 >= 0) v2 = load_slots(x, s2);
-        if (C > 1 && x.lane == s / C) x.t = pick_c<C>(et, s % C);
-        coop_commit(x, cn, s, s / C, v);
+        if (C > 1 && x.lane == lane_of(s)) x.t = pick_c<C>(et, num_of(s));
+        coop_commit(x, cn, s, lane_of(s), v);
         if (s2 < 0) break;
         s = s2;
         v = v2;
@@ -1046,7 +1055,7 @@ __device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor,
         uint32_t live = 0;
 #pragma unroll
         for (int j = 0; j < C; ++j)
-            if (((all >> j) & 1u) && x.drain[x.lane * C + j] > x.t) live |= 1u << j;
+            if (((all >> j) & 1u) && x.drain[inst_at(x.lane, j)] > x.t) live |= 1u << j;
         if (__any_sync(kFull, live != 0)) all = live;
     }
     int dest = -1;
@@ -1063,7 +1072,7 @@ __device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor,
         int bv = INT_MIN, bi = -1;
 #pragma unroll
         for (int j = 0; j < C; ++j) {
-            const int i = x.lane * C + j;
+            const int i = inst_at(x.lane, j);
             if ((all >> j) & 1u) {
                 const int kk = make_key(x, fnum(x, i), x.nrun[i]);
                 if (bi < 0 || kk > bv) { bv = kk; bi = i; }
@@ -1100,7 +1109,7 @@ __device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Para
     int n = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (i < x.N && !(x.drains && x.drain[i] <= x.t)) {
             const int num = x.free_[i] - x.hol[i];
             const int den = max((int)x.nrun[i], 1);
@@ -1203,7 +1212,7 @@ __device__ __forceinline__ bool ranked_tick(const Ctx &x, Cnt &cn, int theta_num
     uint32_t el = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         key[j] = INT_MIN;  // below every freeness key: not eligible
         if (i < x.N && x.mrole[i] == MIG_NONE) {
             key[j] = make_key(x, fnum(x, i), x.nrun[i]);
@@ -1225,8 +1234,8 @@ __device__ __forceinline__ bool ranked_tick(const Ctx &x, Cnt &cn, int theta_num
             for (int j = 0; j < C; ++j) {
                 lt[j] += kk[u] < key[j] ? 1 : 0;
                 if (kk[u] == key[j]) {
-                    eqb[j] += m + u < x.lane * C + j ? 1 : 0;
-                    eqa[j] += m + u > x.lane * C + j ? 1 : 0;
+                    eqb[j] += m + u < inst_at(x.lane, j) ? 1 : 0;
+                    eqa[j] += m + u > inst_at(x.lane, j) ? 1 : 0;
                 }
             }
     }
@@ -1234,8 +1243,8 @@ __device__ __forceinline__ bool ranked_tick(const Ctx &x, Cnt &cn, int theta_num
     for (int j = 0; j < C; ++j)
         if ((el >> j) & 1u) {
             const int below = lt[j] - (np - nel);  // eligible ones
-            lo[below + eqb[j]] = (uint8_t)(x.lane * C + j);
-            hi[nel - 1 - below - eqa[j]] = (uint8_t)(x.lane * C + j);
+            lo[below + eqb[j]] = (uint8_t)inst_at(x.lane, j);
+            hi[nel - 1 - below - eqa[j]] = (uint8_t)inst_at(x.lane, j);
         }
     __syncwarp();
     bool started = false;
@@ -1301,7 +1310,7 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
     uint32_t el = 0, dr = 0;  // eligible (not migrating); draining
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (i < x.N && x.mrole[i] == MIG_NONE) el |= 1u << j;
         if (EXT && i < x.N && x.drains && x.drain[i] <= x.t) dr |= 1u << j;
     }
@@ -1315,9 +1324,8 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
         int s;
         const uint32_t dl = EXT ? __ballot_sync(kFull, (el & dr) != 0) : 0u;
         if (dl) {
-            const int l = __ffs(dl) - 1;
-            const uint32_t bits = C == 1 ? 1u : __shfl_sync(kFull, el & dr, l);
-            s = l * C + __ffs(bits) - 1;
+            const uint32_t bits = el & dr;
+            s = __reduce_min_sync(kFull, bits ? inst_at(x.lane, __ffs(bits) - 1) : INT_MAX);
         } else {
             s = arg_ext<C>(x, el, false, -1);
         }
@@ -1339,8 +1347,8 @@ __device__ __forceinline__ bool migration_tick(const Ctx &x, Cnt &cn, int theta_
             moved = started = true;
         }
         if (moved && x.lane == 0) x.tot[TOT_LOG] = at + 1u;
-        if (x.lane == s / C) el &= ~(1u << (s % C));
-        if (moved && x.lane == d / C) el &= ~(1u << (d % C));
+        if (x.lane == lane_of(s)) el &= ~(1u << num_of(s));
+        if (moved && x.lane == lane_of(d)) el &= ~(1u << num_of(d));
         __syncwarp();
     }
     return started;
@@ -1374,11 +1382,11 @@ __device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, ui
     if (!MT_RARE(t1 - tb > 1u << x.set_bits)) {
 #pragma unroll
         for (int j = 0; j < C; ++j)
-            if (et[j] < t1) set[et[j] - tb] = (uint8_t)(x.lane * C + j);
+            if (et[j] < t1) set[et[j] - tb] = (uint8_t)inst_at(x.lane, j);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < C; ++j)
-            if (et[j] < t1) fresh += set[et[j] - tb] == (uint8_t)(x.lane * C + j) ? 1u : 0u;
+            if (et[j] < t1) fresh += set[et[j] - tb] == (uint8_t)inst_at(x.lane, j) ? 1u : 0u;
     } else {
         uint32_t todo = 0, at[C], win[C];
 #pragma unroll
@@ -1390,12 +1398,12 @@ __device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, ui
         while (__any_sync(kFull, todo != 0)) {
 #pragma unroll
             for (int j = 0; j < C; ++j)
-                if ((todo >> j) & 1u) set[at[j]] = (uint8_t)(x.lane * C + j);
+                if ((todo >> j) & 1u) set[at[j]] = (uint8_t)inst_at(x.lane, j);
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < C; ++j) {
                 win[j] = ((todo >> j) & 1u) ? set[at[j]] : 0u;
-                if (((todo >> j) & 1u) && win[j] == (uint32_t)(x.lane * C + j)) {
+                if (((todo >> j) & 1u) && win[j] == (uint32_t)inst_at(x.lane, j)) {
                     ++fresh;
                     todo &= ~(1u << j);
                 }
@@ -1404,8 +1412,8 @@ __device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, ui
             for (int j = 0; j < C; ++j)
 #pragma unroll
                 for (int k = 0; k < C; ++k) {  // instance win[j] is number k of its lane
-                    const uint32_t tw = __shfl_sync(kFull, et[k], (int)(win[j] / C));
-                    if (win[j] % C == (uint32_t)k && tw == et[j]) todo &= ~(1u << j);
+                    const uint32_t tw = __shfl_sync(kFull, et[k], lane_of((int)win[j]));
+                    if (num_of((int)win[j]) == k && tw == et[j]) todo &= ~(1u << j);
                 }
         }
     }
@@ -1419,29 +1427,24 @@ __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *
         *reinterpret_cast<uint4 *>(dst + o) = *reinterpret_cast<const uint4 *>(src + o);
 }
 
-// Phase 1 at x.t for the instances in `mask` (bit j = instance lane*C + j)
+// Phase 1 at x.t for the instances in `mask` (bit j = the lane's instance j)
 // whose iteration ends now, ascending index.  Collective.
 template <int C>
 __device__ __forceinline__ void complete_all(const Ctx &x, Cnt &cn, uint32_t mask) {
     uint32_t hits = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j)
-        if (((mask >> j) & 1u) && x.busy[x.lane * C + j] == x.t) hits |= 1u << j;
-    uint32_t lanes = __ballot_sync(kFull, hits != 0);
-    while (lanes) {
-        const int l = __ffs(lanes) - 1;
-        lanes &= lanes - 1;
-        uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, hits, l);
-        while (h) {
-            const int i = l * C + __ffs(h) - 1;
-            h &= h - 1;
+        if (((mask >> j) & 1u) && x.busy[inst_at(x.lane, j)] == x.t) hits |= 1u << j;
+#pragma unroll 1
+    for (int j = 0; j < C; ++j)
+        for (uint32_t lanes = __ballot_sync(kFull, (hits >> j) & 1u); lanes; lanes &= lanes - 1) {
+            const int i = inst_at(__ffs(lanes) - 1, j);
             int fp = 0;
             if (x.lane == 0) fp = inst_complete_head(x, i);
             const bool src = x.mrole[i] == MIG_SRC;
             if (__shfl_sync(kFull, fp, 0)) coop_finish(x, cn, i);
             if (src) coop_stage(x, cn, i);
         }
-    }
 }
 
 // Phase 4 at x.t for the idle instances in `mask` that have work, ascending
@@ -1451,22 +1454,18 @@ __device__ __forceinline__ void form_all(Ctx &x, Cnt &cn, uint32_t mask, const P
     uint32_t want = 0;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (((mask >> j) & 1u) && x.busy[i] == kNone && (x.nrun[i] | x.wmask[i]) != 0) want |= 1u << j;
     }
-    uint32_t lanes = __ballot_sync(kFull, want != 0);
-    while (lanes) {
-        const int l = __ffs(lanes) - 1;
-        lanes &= lanes - 1;
-        const uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, want, l);
-        if (x.lane == 0)
-            for (uint32_t hh = h; hh; hh &= hh - 1) inst_form<SMS, LEAN>(x, cn, l * C + __ffs(hh) - 1, p);
-    }
+#pragma unroll 1
+    for (int j = 0; j < C; ++j)
+        for (uint32_t lanes = __ballot_sync(kFull, (want >> j) & 1u); lanes; lanes &= lanes - 1)
+            if (x.lane == 0) inst_form<SMS, LEAN>(x, cn, inst_at(__ffs(lanes) - 1, j), p);
     __syncwarp();
 }
 
 // The events of a window [tb, t1) that can be taken in the next round, bit j =
-// own instance lane*C + j, at time et[j].  A window is short enough that every
+// the lane's instance j, at time et[j].  A window is short enough that every
 // instance ends at most one iteration, and instances interact only as the two
 // ends of a migration: the source's event (finish, copy stage, commit or
 // abort) reads and changes the destination, the destination's event changes
@@ -1488,7 +1487,7 @@ __device__ __forceinline__ Window<C> classify(const Ctx &x, uint32_t t1, uint32_
     Window<C> w{0, 0, 0, 0, false};
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = x.lane * C + j;
+        const int i = inst_at(x.lane, j);
         if (i >= x.N) continue;
         const int role = x.mrole[i];
         if (et[j] < t1) {
@@ -1533,7 +1532,7 @@ __device__ __forceinline__ uint32_t list_own(const Ctx &x, uint32_t sel, const u
     uint2 *list = reinterpret_cast<uint2 *>(x.tset);
 #pragma unroll
     for (int j = 0; j < C; ++j)
-        if ((sel >> j) & 1u) list[pos++] = make_uint2(et[j], (uint32_t)(x.lane * C + j));
+        if ((sel >> j) & 1u) list[pos++] = make_uint2(et[j], (uint32_t)inst_at(x.lane, j));
     __syncwarp();
     return total;
 }
@@ -1709,13 +1708,13 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                     uint32_t cb = kNone;
 #pragma unroll
                     for (int j = 0; j < C; ++j)
-                        if ((cm >> j) & 1u) cb = min(cb, x.busy[lane * C + j]);
+                        if ((cm >> j) & 1u) cb = min(cb, x.busy[inst_at(lane, j)]);
                     tstep = __reduce_min_sync(kFull, cb);
                     mode = tstep < t1 ? 1 : 3;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
                         et[j] = tstep;
-                        if (mode == 1 && ((cm >> j) & 1u) && x.busy[lane * C + j] == tstep) heads |= 1u << j;
+                        if (mode == 1 && ((cm >> j) & 1u) && x.busy[inst_at(lane, j)] == tstep) heads |= 1u << j;
                     }
                 } else {
                     if (!any_b) {
@@ -1725,7 +1724,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                     uint32_t mb = kNone;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
-                        const int i = lane * C + j;
+                        const int i = inst_at(lane, j);
                         et[j] = i < x.N ? x.busy[i] : kNone;
                         mb = min(mb, et[j]);
                     }
@@ -1786,28 +1785,30 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
 #pragma unroll 1
                 while (go) {
                     uint32_t sel = todo;
-                    if (!LEAN && mode != 0) sel = lane == __ffs(__ballot_sync(kFull, todo != 0)) - 1 ? todo & (0u - todo) : 0u;
+                    if (!LEAN && mode != 0) {  // the lowest instance left
+                        const int i = __reduce_min_sync(kFull, todo ? inst_at(lane, __ffs(todo) - 1) : INT_MAX);
+                        sel = lane == lane_of(i) ? 1u << num_of(i) : 0u;
+                    }
                     todo &= ~sel;
                     uint32_t fz = 0, src = 0;  // own instances with a finishing request; sources
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
                         if (!((sel >> j) & 1u)) continue;
-                        const int i = lane * C + j;
+                        const int i = inst_at(lane, j);
                         if (inst_complete_head(x, i)) fz |= 1u << j;
                         if (mig && x.mrole[i] == MIG_SRC) src |= 1u << j;
                     }
                     __syncwarp();
                     if (LEAN) fz |= src << C;
-                    for (uint32_t fl = __ballot_sync(kFull, fz != 0); fl; fl &= fl - 1) {
-                        const int l = __ffs(fl) - 1;
-                        const uint32_t fzl = C == 1 && !LEAN ? 1u : __shfl_sync(kFull, fz, l);
-                        for (uint32_t h = LEAN ? (fzl | (fzl >> C)) & ((1u << C) - 1u) : fzl; h; h &= h - 1) {
-                            const int j = __ffs(h) - 1;
+#pragma unroll 1
+                    for (int j = 0; j < C; ++j)
+                        for (uint32_t fl = __ballot_sync(kFull, (fz >> j) & (LEAN ? 1u | 1u << C : 1u)); fl; fl &= fl - 1) {
+                            const int l = __ffs(fl) - 1, i = inst_at(l, j);
+                            const uint32_t fzl = LEAN ? __shfl_sync(kFull, fz >> j, l) : 1u;
                             x.t = __shfl_sync(kFull, pick_c<C>(et, j), l);
-                            if (!LEAN || ((fzl >> j) & 1u)) coop_finish(x, cn, l * C + j);
-                            if (LEAN && ((fzl >> (C + j)) & 1u)) coop_stage(x, cn, l * C + j);
+                            if (!LEAN || (fzl & 1u)) coop_finish(x, cn, i);
+                            if (LEAN && (fzl & (1u << C))) coop_stage(x, cn, i);
                         }
-                    }
                     if (!LEAN && mig) stage_all<C>(x, cn, src, et);
                     go = !LEAN && mode != 0 && __any_sync(kFull, todo != 0);
                 }
@@ -1844,25 +1845,29 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                     const uint32_t mask = mode == 1 ? cm : all;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
-                        const int i = lane * C + j;
+                        const int i = inst_at(lane, j);
                         if (((mask >> j) & 1u) && x.busy[i] == kNone && (x.nrun[i] | x.wmask[i]) != 0) want |= 1u << j;
                     }
                 }
                 // (mode 0 with destinations to wake: three rounds, the lower wakes, the
                 // instances whose iterations ended, the higher wakes)
-                for (uint32_t fl = mode != 0 ? __ballot_sync(kFull, want != 0) : any_wake ? 7u : 1u; fl; fl &= fl - 1) {
-                    const int l = __ffs(fl) - 1;
-                    const uint32_t hl = mode == 0 ? want : (C == 1 ? 1u : __shfl_sync(kFull, want, l));
-                    const int owner = mode == 0 ? lane : l;
-                    if (mode == 0 || lane == 0) {
-                        for (uint32_t h = hl; h; h &= h - 1) {
-                            const int j = __ffs(h) - 1;
-                            x.t = mode == 0 ? pick_c<C>(et, j) : tstep;
-                            inst_form<SMS, LEAN>(x, cn, owner * C + j, p);
+#pragma unroll 1
+                for (int j0 = 0; j0 < (mode == 0 ? 1 : C); ++j0) {
+                    for (uint32_t fl = mode != 0 ? __ballot_sync(kFull, (want >> j0) & 1u) : any_wake ? 7u : 1u; fl;
+                         fl &= fl - 1) {
+                        const int l = __ffs(fl) - 1;
+                        const uint32_t hl = mode == 0 ? want : 1u << j0;
+                        const int owner = mode == 0 ? lane : l;
+                        if (mode == 0 || lane == 0) {
+                            for (uint32_t h = hl; h; h &= h - 1) {
+                                const int j = __ffs(h) - 1;
+                                x.t = mode == 0 ? pick_c<C>(et, j) : tstep;
+                                inst_form<SMS, LEAN>(x, cn, inst_at(owner, j), p);
+                            }
                         }
+                        if (mode == 0) want = l == 0 ? heads : wake_hi;
+                        __syncwarp();
                     }
-                    if (mode == 0) want = l == 0 ? heads : wake_hi;
-                    __syncwarp();
                 }
                 // ---- step accounting ----
                 if (mode == 0 || mode == 3) {
@@ -1888,7 +1893,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                 uint32_t mb = kNone;
 #pragma unroll
                 for (int j = 0; j < C; ++j) {
-                    const int i = lane * C + j;
+                    const int i = inst_at(lane, j);
                     bz[j] = i < x.N ? x.busy[i] : kNone;
                     mb = min(mb, bz[j]);
                 }
@@ -1913,7 +1918,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
 #pragma unroll
                         for (int j = 0; j < C; ++j) {
                             if (!((sel >> j) & 1u)) continue;
-                            const int i = lane * C + j;
+                            const int i = inst_at(lane, j);
                             if (inst_complete_head(x, i)) fz |= 1u << j;
                             if (stages && x.mrole[i] == MIG_SRC) src |= 1u << j;
                         }
@@ -1923,7 +1928,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                             for (uint32_t h = C == 1 ? 1u : __shfl_sync(kFull, fz, l); h; h &= h - 1) {
                                 const int j = __ffs(h) - 1;
                                 x.t = __shfl_sync(kFull, pick_c<C>(bz, j), l);
-                                coop_finish(x, cn, l * C + j);
+                                coop_finish(x, cn, inst_at(l, j));
                             }
                         }
                         if (stages) stage_all<C>(x, cn, src, bz);
@@ -1972,7 +1977,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                             if (any & 1u) {
 #pragma unroll
                                 for (int j = 0; j < C; ++j)
-                                    bz[j] = lane * C + j < x.N ? x.busy[lane * C + j] : kNone;
+                                    bz[j] = inst_at(lane, j) < x.N ? x.busy[inst_at(lane, j)] : kNone;
                             }
                         } while (any & 1u);
                         // pairs whose two iterations end at the same time: whole steps
@@ -1981,7 +1986,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                             uint32_t cb = kNone;
 #pragma unroll
                             for (int j = 0; j < C; ++j)
-                                if ((same >> j) & 1u) cb = min(cb, x.busy[lane * C + j]);
+                                if ((same >> j) & 1u) cb = min(cb, x.busy[inst_at(lane, j)]);
                             const uint32_t tc = __reduce_min_sync(kFull, cb);
                             if (tc >= t1) break;
                             x.t = tc;
