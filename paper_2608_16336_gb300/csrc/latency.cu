@@ -305,17 +305,18 @@ __global__ void k_latency_step(long long nstates, uint4 *sel, uint32_t *bins, si
 // All statistics of a replica by one block, its requests read once: the three
 // values and the tier of every request stay in shared memory for the selection
 // passes, whose bins (16-bit counts, two per word) are there too.  Dynamic
-// shared memory (replica_bytes): val [3][qcap], sums [warps][G], maxima
-// [warps][G], states [S], the histogram [G][SIM_HIST_BUCKETS] or, after it
-// has been written out, the bins [S][kSelBins / 2], tiers [qcap] (0x80: the
-// request has a TBT; kSkip: not finished).  Sums and maxima: per warp, one
-// reduction for each tier that the warp's 32 requests have, the sums in two
-// 16-bit halves (32 x 65,535 fits), so nothing is contended.
-// 1,024 replicas x 5,000 requests, K = 4 (130 MB): 192 us, of which about 80 in
+// shared memory (replica_bytes): states [S], sums [warps][G], maxima
+// [warps][G], the histogram [G][SIM_HIST_BUCKETS] or, after it has been
+// written out, the bins [S][kSelBins / 2], values [3][qcap], tiers [qcap]
+// (0x80: the request has a TBT; kSkip: not finished).  Sums and maxima: per warp, one
+// reduction for each tier that the warp's 32 requests have (sums in two 16-bit
+// halves when the plain sum could overflow), so nothing is contended.
+// 1,024 replicas x 5,000 requests, K = 4 (130 MB): 189 us, of which about 80 in
 // the selection passes, 60 in the reductions and 50 in the read and the
-// histogram; the streaming passes take 294 us.  (Sums of up to 4 tiers in
-// registers 216 us; one look-up of the open percentiles per bucket instead of
-// nine range checks 203 us.)
+// histogram; the streaming passes take 294 us.  (Half sums for every value, also
+// where one cannot overflow, 193 us; sums of up to 4 tiers in registers 216 us;
+// one look-up of the open percentiles per bucket instead of nine range checks
+// 203 us.)
 constexpr uint32_t kSkip = 0x7Fu;
 __global__ void __launch_bounds__(1024) k_latency_replica(int R, const long long *offsets, int KT,
                                                           const uint32_t *arrival, const uint16_t *olen,
@@ -384,12 +385,18 @@ __global__ void __launch_bounds__(1024) k_latency_replica(int R, const long long
 #pragma unroll
                     for (int m = 0; m < 3; ++m) {  // a request without TBT adds 0 there
                         const uint32_t x = mine ? v[m] : 0u;
-                        const uint32_t slo = __reduce_add_sync(kFull, x & 0xFFFFu);
-                        const uint32_t shi = __reduce_add_sync(kFull, x >> 16);
                         const uint32_t mx = __reduce_max_sync(kFull, x);
+                        unsigned long long sum;
+                        if (mx < 1u << 27) {
+                            sum = __reduce_add_sync(kFull, x);
+                        } else {
+                            const uint32_t slo = __reduce_add_sync(kFull, x & 0xFFFFu);
+                            const uint32_t shi = __reduce_add_sync(kFull, x >> 16);
+                            sum = (unsigned long long)slo + ((unsigned long long)shi << 16);
+                        }
                         if (lane == m) {
                             const int at = warp * G + (int)kk * 3 + m;
-                            wsum[at] += (unsigned long long)slo + ((unsigned long long)shi << 16);
+                            wsum[at] += sum;
                             wmax[at] = max(wmax[at], mx);
                         }
                     }

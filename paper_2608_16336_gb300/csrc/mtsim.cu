@@ -18,10 +18,10 @@
 //   only on events; batch advance is lazy (see the slot record below), so an
 //   iteration end and a batch formation without events cost O(1).
 //   Between global events (arrivals, migration ticks) the instances that are
-//   in no migration do not interact, so each lane advances its own instances
-//   through a window in which each ends at most one iteration; migrations and
-//   global events are stepped by the whole warp in the oracle's order.  The
-//   next 32 arrivals are held in registers, one per lane.
+//   in no migration do not interact, and the two ends of a migration only with
+//   each other, so the lanes advance them through a window in which each ends
+//   at most one iteration; global events are stepped by the whole warp in the
+//   oracle's order.  The next 32 arrivals are held in registers, one per lane.
 //
 // Exactness
 //   Everything is integer.  Freeness F = (M - U) / max(B, 1) (Sec. 3.2 Eq. 1-2)
@@ -144,7 +144,8 @@ struct Layout {
 // A replica's rarely changing counters, kept with its instance state so that
 // they hold no registers: log records, migrations, preemptions, migration
 // starts and aborts, scale-out and scale-in signals.  Formations on several
-// lanes may add to TOT_PRE and TOT_ABORT at once; lane 0 alone adds to the others.
+// lanes may add to TOT_PRE, TOT_ABORT and TOT_MIG (atomics); lane 0 alone adds to
+// the others.
 enum : int { TOT_LOG = 0, TOT_MIG, TOT_PRE, TOT_START, TOT_ABORT, TOT_OUT, TOT_IN, TOT_COUNT };
 
 // Per-replica scalars persisted between sim_run calls.
