@@ -2213,6 +2213,7 @@ typedef void (*RunKernel)(Params);
 
 template <bool EXT>
 RunKernel pick(int c, bool sms, bool many) {  // c = instances per lane
+    if (many && sms) return k_run<1, true, EXT, true>;
     if (many) return c == 1 ? k_run<1, false, EXT, true> : k_run<2, false, EXT, true>;
     switch (c) {
         case 1: return sms ? k_run<1, true, EXT, false> : k_run<1, false, EXT, false>;
@@ -2279,27 +2280,59 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     int dev = 0, sms_count = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
-    // Which main loop: see k_run.  1,500 requests per replica, loop of many / of
-    // few, ms: 32 instances, 304 replicas 9.2 / 7.9, 1,216 9.9 / 9.0, 1,824 10.7 /
+    const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    auto smem_of = [&](int bits) {
+        return kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << bits));
+    };
+    auto resident = [&](RunKernel fn, int bits, int &per_sm) {
+        cudaError_t err = cudaSuccess;
+        if (smem_of(bits) > 48 * 1024)
+            err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(bits));
+        if (err == cudaSuccess)
+            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarpsPerBlock, smem_of(bits));
+        return err;
+    };
+    // Which main loop (see k_run): that of many replicas above 10 (C = 1) or 14
+    // (C = 2) per SM.  1,500 requests per replica, records in HBM, loop of many /
+    // of few, ms: 32 instances, 304 replicas 9.2 / 7.9, 1,216 9.9 / 9.0, 1,824 10.7 /
     // 11.5, 2,432 11.4 / 20.1; 64 instances, 304 replicas 15.5 / 12.0, 1,824 18.8 /
-    // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).
-    const bool many = !sms && out.c <= 2 && R > (out.c == 1 ? 10 : 14) * sms_count;
+    // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).  With
+    // records in shared memory only where at least 5 blocks fit: 8,192 replicas x 8
+    // x 400 requests 15.9 / 21.6, 8,192 x 16 x 500 26.0 / 28.3 (5 blocks), 6,000 x
+    // 24 x 400 27.7 / 24.4 (3 blocks).
+    bool many = (sms ? out.c == 1 : out.c <= 2) && R > (sms ? 10 : out.c == 1 ? 10 : 14) * sms_count;
+    if (many && sms && e == cudaSuccess) {
+        int n = 0;
+        e = resident(pick<false>(out.c, sms, true), kSetBitsMany, n);
+        many = n >= 5;
+    }
+    out.fn = pick<false>(out.c, sms, many);
+    out.fn_ext = pick<true>(out.c, sms, many);
     // The scratch: 4 KB holds a window of the default `base` of 4 ms directly.
     // Where two instances per lane share an SM with 17 other warps it has 2 KB,
     // and 1 KB, with two warps more, for sweeps of several waves (8,192 x 64:
-    // 110.2 against 112.5 ms).
-    out.set_bits = sms || out.c > 2 ? kSetBitsShared : many && out.c == 2 && R > 26 * sms_count ? kSetBitsMany : kSetBits;
-    out.smem = kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << out.set_bits));
-    out.fn = pick<false>(out.c, sms, many);
-    out.fn_ext = pick<true>(out.c, sms, many);
-    const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    // 110.2 against 112.5 ms).  Elsewhere it shrinks where that makes every replica
+    // resident (1,400 x 16 x 500: 4.9 instead of 7.1 ms); more warps of several
+    // waves alone gain nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).
+    if (many && sms) {
+        out.set_bits = kSetBitsMany;
+    } else if (many && out.c == 2) {
+        out.set_bits = R > 26 * sms_count ? kSetBitsMany : kSetBits;
+    } else {
+        out.set_bits = kSetBitsShared;
+        for (int bits = kSetBitsShared; bits >= kSetBitsMany && e == cudaSuccess; --bits) {
+            int n = 0;
+            e = resident(out.fn, bits, n);
+            if ((long long)n * sms_count >= want) {
+                out.set_bits = bits;
+                break;
+            }
+        }
+    }
+    out.smem = smem_of(out.set_bits);
     for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
-        RunKernel fn = v ? out.fn_ext : out.fn;
         int per_sm = 0;
-        if (out.smem > 48 * 1024)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)out.smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarpsPerBlock, out.smem);
+        e = resident(v ? out.fn_ext : out.fn, out.set_bits, per_sm);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         (v ? out.grid_ext : out.grid) = (int)std::min<long long>(want, (long long)sms_count * per_sm);

@@ -38,9 +38,10 @@ def test_tick(n, theta):
     assert int(st["log_events"].sum()) > 0
 
 
-@pytest.mark.parametrize("n,replicas", [(30, 1519), (30, 1521), (40, 2127), (40, 2129), (40, 3951), (40, 3953)])
+@pytest.mark.parametrize("n,replicas", [(30, 1519), (30, 1521), (40, 2127), (40, 2129), (40, 3951), (40, 3953), (8, 1519),
+                                        (8, 1521), (16, 1300)])
 def test_both_loops(n, replicas):
-    """One per lane and two per lane, records in HBM, around the replica counts
+    """One per lane and two per lane, records in HBM or shared, around the replica counts
     where a 152-SM GPU changes loops and scratch; sampled replicas against the oracle."""
     rng = np.random.default_rng(replicas)
     traces = [_trace(rng, n, 40, 2, r % 2 == 0) for r in range(replicas)]
