@@ -1488,26 +1488,19 @@ __device__ __forceinline__ Window<C> classify(const Ctx &x, uint32_t t1, uint32_
     Window<C> w{0, 0, 0, 0, false};
 #pragma unroll
     for (int j = 0; j < C; ++j) {
-        const int i = inst_at(x.lane, j);
-        if (i >= x.N) continue;
-        const int role = x.mrole[i];
-        if (et[j] < t1) {
-            if (role == MIG_NONE) {
-                w.first |= 1u << j;
-            } else {
-                const uint32_t pb = x.busy[x.mpeer[i]];
-                if (pb > et[j]) w.first |= 1u << j;
-                else if (pb < et[j]) w.later = true;
-                else w.same |= 1u << j;
-            }
-        } else if (role == MIG_DST && et[j] == kNone) {
-            const int s = x.mpeer[i];
-            const uint32_t pb = x.busy[s];
-            if (pb < t1) {
-                (i < s ? w.wake_lo : w.wake_hi) |= 1u << j;
-                et[j] = pb;
-            }
-        }
+        // without branches, the peer's busy time read in any case: a divergent branch
+        // costs more than the read (256 x 128 40.8 -> 39.1 ms, 1,024 x 16 9.12 -> 8.74)
+        const int i = inst_at(x.lane, j), ii = i < x.N ? i : 0;
+        const int role = x.mrole[ii], peer = x.mpeer[ii];
+        const uint32_t pb = x.busy[peer], t = et[j];
+        const bool in = i < x.N && t < t1, pair = role != MIG_NONE;
+        const bool wake = i < x.N && t == kNone && role == MIG_DST && pb < t1;
+        w.first |= (in && (!pair || pb > t) ? 1u : 0u) << j;
+        w.same |= (in && pair && pb == t ? 1u : 0u) << j;
+        w.later = w.later || (in && pair && pb < t);
+        w.wake_lo |= (wake && i < peer ? 1u : 0u) << j;
+        w.wake_hi |= (wake && i > peer ? 1u : 0u) << j;
+        et[j] = wake ? pb : t;
     }
     return w;
 }
