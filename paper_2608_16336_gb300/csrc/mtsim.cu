@@ -320,13 +320,17 @@ __device__ __forceinline__ uint32_t mod_t(const Ctx &x, uint32_t v) {  // v mod 
 
 // floor(v / d) for v < 2^32 and 1 <= d <= 64: the high half of v * ceil(2^64 / d).
 __device__ __forceinline__ uint32_t div_small(const Ctx &x, uint32_t v, int d) {
-    return d == 1 ? v : (uint32_t)__umul64hi((unsigned long long)v, x.magic[d]);
+    const uint32_t q = (uint32_t)__umul64hi((unsigned long long)v, x.magic[d]);
+    return d == 1 ? v : q;
 }
 
 __device__ __forceinline__ int make_key(const Ctx &x, int num, int nrun) {
-    const int d = nrun > 0 ? nrun : 1;
-    if (num >= 0) return (int)div_small(x, (uint32_t)num << kKeyShift, d);
-    return -(int)div_small(x, ((uint32_t)(-num) << kKeyShift) + (uint32_t)(d - 1), d);
+    // one division of the magnitude, rounded down or (negative) up, without
+    // branches (64 x 256 58.8 -> 56.9 ms, 1,024 x 16 8.75 -> 8.60)
+    const int d = max(nrun, 1);
+    const uint32_t mag = ((uint32_t)abs(num) << kKeyShift) + (num < 0 ? (uint32_t)(d - 1) : 0u);
+    const int q = (int)div_small(x, mag, d);
+    return num < 0 ? -q : q;
 }
 
 __device__ __forceinline__ int fnum(const Ctx &x, int i) { return x.free_[i] - x.hol[i] - x.hr[i]; }
@@ -870,7 +874,7 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
     const uint32_t nf = x.nf[i];
     uint32_t wm = x.wmask[i];
     int need = x.hol[i];
-    if (n > 0) {
+    {
         const int deficit = x.hist[i * x.TH + (ph == 0 ? 0u : (uint32_t)x.T - ph)];
         if (!MT_RARE(deficit > fr)) {
             fr -= deficit;  // every request that needs a block gets it
@@ -890,9 +894,7 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
     const int n_decode = n;
     int prefill = 0;
 #pragma unroll 1
-    while (n < x.Bmax) {
-        if (!wm) break;
-        if (need > fr) break;
+    while ((n < x.Bmax) & (wm != 0u) & (need <= fr)) {
         const int k = __ffs(wm) - 1;
         const int b = i * x.K + k;
         const uint32_t info = x.hinfo[b];
@@ -1553,7 +1555,7 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
     // whether the end of the running iteration is quiet, and the blocks its successor takes
     auto look = [&]() {
         grow = hist[ph == 0 ? 0u : (uint32_t)x.T - ph];
-        quiet = nf != minfin && grow <= fr && !(waits && need <= fr - grow) && busy < 0xFFFFFFFEu - dur;
+        quiet = (nf != minfin) & (grow <= fr) & !(waits & (need <= fr - grow)) & (busy < 0xFFFFFFFEu - dur);
     };
     look();
     while (tb < tg && max_steps - cn.steps > (uint32_t)x.N) {
