@@ -441,10 +441,12 @@ def time_latency_stats(torch, mtsim, sim, w, stream, reps: int = 10) -> dict:
     nbytes = Q * (16 + 4 + 2 + 1) + out.numel()
     peak, kind = measured_peak_hbm()
     gbs = nbytes / (ms / 1e3) / 1e9
-    return {"kernel": "sim_latency_stats: k_latency_hist, k_latency_pct and up to four k_latency_refine + "
-                      "k_latency_step selection passes (output clear included)",
+    return {"kernel": "sim_latency_stats: k_latency_replica, or for replicas of more than about 15,000 requests "
+                      "k_latency_hist, k_latency_pct and up to four k_latency_refine + k_latency_step selection "
+                      "passes (output clear included)",
             "work": "per-tier TTFT/TBT/E2E histograms and exact nearest-rank P50/P90/P99 of every request; "
-                    "algorithmic bytes = one read of the inputs, which each selection pass still open reads again",
+                    "algorithmic bytes = one read of the inputs (the selection passes of large replicas read "
+                    "them again)",
             "bound": "hbm", "ms": ms, "algorithmic_bytes_per_launch": nbytes, "achieved": gbs, "peak": peak,
             "peak_kind": kind, "unit": "GB/s", "frac": gbs / peak}
 
