@@ -324,7 +324,17 @@ __device__ __forceinline__ uint32_t div_small(const Ctx &x, uint32_t v, int d) {
     return d == 1 ? v : q;
 }
 
+// SELECT: without branches.  Where instruction fetch bounds (two instances per
+// lane, many replicas) the other form is faster: 8,192 x 64 108.8 against 112.0
+// ms, in its steady state (4,096 x 10,000 requests) 151 against 157 ms.
+template <bool SELECT = true>
 __device__ __forceinline__ int make_key(const Ctx &x, int num, int nrun) {
+    if constexpr (!SELECT) {
+        const int d = nrun > 0 ? nrun : 1;
+        if (num >= 0) return (int)(d == 1 ? (uint32_t)num << kKeyShift : div_small(x, (uint32_t)num << kKeyShift, d));
+        const uint32_t v = ((uint32_t)(-num) << kKeyShift) + (uint32_t)(d - 1);
+        return -(int)(d == 1 ? v : div_small(x, v, d));
+    }
     // one division of the magnitude, rounded down or (negative) up, without
     // branches (64 x 256 58.8 -> 56.9 ms, 1,024 x 16 8.75 -> 8.60)
     const int d = max(nrun, 1);
@@ -335,7 +345,10 @@ __device__ __forceinline__ int make_key(const Ctx &x, int num, int nrun) {
 
 __device__ __forceinline__ int fnum(const Ctx &x, int i) { return x.free_[i] - x.hol[i] - x.hr[i]; }
 
-__device__ __forceinline__ void set_key(const Ctx &x, int i) { x.key[i] = make_key(x, fnum(x, i), x.nrun[i]); }
+template <bool SELECT>
+__device__ __forceinline__ void set_key(const Ctx &x, int i) {
+    x.key[i] = make_key<SELECT>(x, fnum(x, i), x.nrun[i]);
+}
 
 // Instance j of a lane (j < C) and back.  Consecutive lanes own consecutive
 // instances, so their records (13 words each) lie in different shared-memory
@@ -351,7 +364,7 @@ __device__ __forceinline__ void refresh_keys(const Ctx &x) {
 #pragma unroll
     for (int j = 0; j < C; ++j) {
         const int i = inst_at(x.lane, j);
-        if (i < x.N) set_key(x, i);
+        if (i < x.N) set_key<C != 2>(x, i);
     }
     __syncwarp();
 }
@@ -874,7 +887,7 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
     const uint32_t nf = x.nf[i];
     uint32_t wm = x.wmask[i];
     int need = x.hol[i];
-    {
+    if (!LEAN || n > 0) {  // (nothing is counted where nothing runs)
         const int deficit = x.hist[i * x.TH + (ph == 0 ? 0u : (uint32_t)x.T - ph)];
         if (!MT_RARE(deficit > fr)) {
             fr -= deficit;  // every request that needs a block gets it
@@ -894,7 +907,9 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
     const int n_decode = n;
     int prefill = 0;
 #pragma unroll 1
-    while ((n < x.Bmax) & (wm != 0u) & (need <= fr)) {
+    while (LEAN ? n < x.Bmax : (n < x.Bmax) & (wm != 0u) & (need <= fr)) {
+        if (LEAN && !wm) break;
+        if (LEAN && need > fr) break;
         const int k = __ffs(wm) - 1;
         const int b = i * x.K + k;
         const uint32_t info = x.hinfo[b];
@@ -969,7 +984,7 @@ __device__ __forceinline__ void dispatch_to(const Ctx &x, Cnt &cn, int best, uin
         if (c0 == 0) x.hr[best] = hr += hk;                    // tier k now present (Eq. 4)
         if ((old & ((2u << k) - 1u)) == 0) x.hol[best] = hol = blocks_for(x, P);  // becomes head of line
         x.res(r)->dispatch_instance = (uint16_t)best;
-        if (store_key) x.key[best] = make_key(x, fr - hol - hr, nr);
+        if (store_key) x.key[best] = make_key<false>(x, fr - hol - hr, nr);
     }
 }
 
@@ -1077,7 +1092,7 @@ __device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor,
         for (int j = 0; j < C; ++j) {
             const int i = inst_at(x.lane, j);
             if ((all >> j) & 1u) {
-                const int kk = make_key(x, fnum(x, i), x.nrun[i]);
+                const int kk = make_key<!LEAN>(x, fnum(x, i), x.nrun[i]);
                 if (bi < 0 || kk > bv) { bv = kk; bi = i; }
             }
         }
@@ -1218,7 +1233,7 @@ __device__ __forceinline__ bool ranked_tick(const Ctx &x, Cnt &cn, int theta_num
         const int i = inst_at(x.lane, j);
         key[j] = INT_MIN;  // below every freeness key: not eligible
         if (i < x.N && x.mrole[i] == MIG_NONE) {
-            key[j] = make_key(x, fnum(x, i), x.nrun[i]);
+            key[j] = make_key<C != 2>(x, fnum(x, i), x.nrun[i]);
             el |= 1u << j;
         }
         if (i < np) sk[i] = key[j];
