@@ -47,6 +47,7 @@
 //   out-of-bounds access.
 #include "mtsim.h"
 #include "latency.cuh"
+#include "plan.cuh"
 
 #include <cuda_runtime.h>
 
@@ -71,13 +72,7 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr int kKeyShift = 12;            // keys are floor(num * 4096 / den)
 constexpr int kMaxKeyRange = 1 << 19;    // |num| < 2^19 keeps num * 4096 below 2^31
 constexpr int kMagicShift = 40;          // floor(n / T) = (n * ceil(2^40 / T)) >> 40 for n < 2^20, T <= 65535
-constexpr int kWarpsPerBlock = 2;
 constexpr int kMaxBlockTokens = 64;      // T limit of the per-instance growth histogram
-constexpr uint32_t kMagicBytes = 528;    // ceil(2^64 / d) for d = 0..64, rounded up to 16 bytes
-// Bytes (2^n) of the per-warp scratch that counts a window's distinct event
-// times (distinct_times): small where many warps share an SM's shared memory
-// (plan_launch).
-constexpr int kSetBitsShared = 12, kSetBits = 11, kSetBitsMany = 10;
 
 enum : int { MIG_NONE = 0, MIG_SRC = 1, MIG_DST = 2 };
 
@@ -118,7 +113,7 @@ struct InstRec {
     uint8_t nrun, pc, phase;      // running requests; iteration-ended flag; nf mod T
     uint8_t mrole, mpeer, mpend;  // migration role and peer; phase of a log record held back in mslot, or 0
 };
-static_assert(sizeof(InstRec) == 52, "InstRec is 13 words");
+static_assert(sizeof(InstRec) == 52 && sizeof(InstRec) == kInstBytes, "InstRec is 13 words");
 
 // x.busy[i] and the like: field F of instance i's record.
 template <typename T, int OFF>
@@ -130,23 +125,13 @@ struct Field {
 };
 #define MT_FIELD(T, f) Field<T, (int)offsetof(InstRec, f)> f
 
-struct Layout {
-    uint32_t inst;                                                       // [N] x InstRec
-    uint32_t cnt;                                                        // [N*K] x 2 B
-    uint32_t head, tail, hinfo;                                          // [N*K] x 4 B
-    uint32_t h;                                                          // [K] x 4 B
-    uint32_t hist;                                                       // [N*TH] x 1 B
-    uint32_t mslot;                                                      // [N] x 16 B
-    uint32_t tot;                                                        // [TOT_COUNT] x 4 B
-    uint32_t bytes;
-};
-
 // A replica's rarely changing counters, kept with its instance state so that
 // they hold no registers: log records, migrations, preemptions, migration
 // starts and aborts, scale-out and scale-in signals.  Formations on several
 // lanes may add to TOT_PRE, TOT_ABORT and TOT_MIG (atomics); lane 0 alone adds to
 // the others.
 enum : int { TOT_LOG = 0, TOT_MIG, TOT_PRE, TOT_START, TOT_ABORT, TOT_OUT, TOT_IN, TOT_COUNT };
+static_assert(TOT_COUNT == kTotCount, "counters of the layout");
 
 // Per-replica scalars persisted between sim_run calls.
 struct RepState {
@@ -214,7 +199,7 @@ struct Ctx {
     uint8_t *hist;
     uint4 *mslot;                     // record of the request a migration source is copying out
     uint4 *slots;
-    uint32_t *tset;                   // scratch of distinct_times
+    uint32_t *tset;                   // scratch: event times, a tick's ranking, a window's formations (scratch_need)
     const unsigned long long *magic;  // [65]: ceil(2^64 / d) for d >= 2
     uint32_t *tot;                    // TOT_* counters
     uint4 *node;                      // the replica's queue nodes
@@ -252,11 +237,7 @@ struct Cnt {
     bool held;  // this lane has held back a log record in the open window
 };
 
-// The block's dynamic shared memory: a copy of the parameters (for the
-// out-of-line functions below, which cannot reach the kernel's own), the
-// table of ceil(2^64 / d), then each warp's replica state.
-constexpr uint32_t kParamBytes = (sizeof(Params) + 15u) & ~15u;
-constexpr uint32_t kHeadBytes = kParamBytes + kMagicBytes;
+static_assert(((sizeof(Params) + 15u) & ~15u) == kParamBytes, "parameter copy of the block's shared memory");
 
 __device__ __forceinline__ void bind_blob(Ctx &x, const Layout &L, unsigned char *blob) {
     unsigned char *ib = blob + L.inst;
@@ -2245,110 +2226,38 @@ struct Launch {
     size_t smem = 0;
 };
 
-inline int lanes_c(int N) { return N <= 32 ? 1 : N <= 64 ? 2 : N <= 128 ? 4 : 8; }
-
-// Bytes per instance of the growth histogram: T rounded up to an odd number
-// of words, so lanes reading one entry of consecutive instances hit distinct
-// banks (1,024-replica workload +0.8 %; the same odd stride for the bucket
-// arrays, as one {head, tail, info, count} record per tier, was 3 % slower
-// on the 16,384-replica workload).
-inline int hist_stride(int T) { return (((T + 3) >> 2) | 1) << 2; }
-
-inline Layout make_layout(int N, int K, int T) {
-    Layout L;
-    uint32_t o = 0;
-    auto take = [&](uint32_t bytes, uint32_t align) {
-        o = (o + align - 1) / align * align;
-        const uint32_t at = o;
-        o += bytes;
-        return at;
-    };
-    L.inst = take((uint32_t)sizeof(InstRec) * N, 16);
-    L.head = take(4u * N * K, 16);
-    L.tail = take(4u * N * K, 16);
-    L.hinfo = take(4u * N * K, 16);
-    L.h = take(4u * K, 16);
-    L.cnt = take(2u * N * K, 16);
-    L.hist = take((uint32_t)N * hist_stride(T), 16);
-    L.mslot = take(16u * N, 16);
-    L.tot = take(4u * TOT_COUNT, 16);
-    L.bytes = (o + 15u) & ~15u;
-    return L;
-}
-
-
 // Chooses the kernel variant and grid for a problem; cudaSuccess or the error.
-// Running-request records go to shared memory while a replica's take at most this many bytes.
-constexpr uint32_t kSmemSlotLimit = 24u * 1024u;
-inline bool slots_in_shared(int N, int Bmax) { return (uint32_t)N * (uint32_t)Bmax * 16u <= kSmemSlotLimit; }
-
 inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &out) {
-    const uint32_t slot_bytes = (uint32_t)N * (uint32_t)Bmax * 16u;
-    const bool sms = slots_in_shared(N, Bmax);
-    out.c = lanes_c(N);
-    out.sms = sms;
     int dev = 0, sms_count = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    auto smem_of = [&](int bits) {
-        return kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + (sms ? slot_bytes : 0u) + (1u << bits));
-    };
-    auto resident = [&](RunKernel fn, int bits, int &per_sm) {
-        cudaError_t err = cudaSuccess;
-        if (smem_of(bits) > 48 * 1024)
-            err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(bits));
-        if (err == cudaSuccess)
-            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarpsPerBlock, smem_of(bits));
-        return err;
-    };
-    // Which main loop (see k_run): that of many replicas above 10 (C = 1) or 14
-    // (C = 2) per SM.  1,500 requests per replica, records in HBM, loop of many /
-    // of few, ms: 32 instances, 304 replicas 9.2 / 7.9, 1,216 9.9 / 9.0, 1,824 10.7 /
-    // 11.5, 2,432 11.4 / 20.1; 64 instances, 304 replicas 15.5 / 12.0, 1,824 18.8 /
-    // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).  With
-    // records in shared memory only where at least 5 blocks fit: 8,192 replicas x 8
-    // x 400 requests 15.9 / 21.6, 8,192 x 16 x 500 26.0 / 28.3 (5 blocks), 6,000 x
-    // 24 x 400 27.7 / 24.4 (3 blocks).
-    bool many = (sms ? out.c == 1 : out.c <= 2) && R > (sms ? 10 : out.c == 1 ? 10 : 14) * sms_count;
-    if (many && sms && e == cudaSuccess) {
-        int n = 0;
-        e = resident(pick<false>(out.c, sms, true), kSetBitsMany, n);
-        many = n >= 5;
-    }
-    out.fn = pick<false>(out.c, sms, many);
-    out.fn_ext = pick<true>(out.c, sms, many);
-    // The scratch: 4 KB holds a window of the default `base` of 4 ms directly.
-    // Where two instances per lane share an SM with 17 other warps it has 2 KB,
-    // and 1 KB, with two warps more, for sweeps of several waves (8,192 x 64:
-    // 110.2 against 112.5 ms).  Elsewhere it shrinks where that makes every replica
-    // resident (1,400 x 16 x 500: 4.9 instead of 7.1 ms); more warps of several
-    // waves alone gain nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).
-    if (many && sms) {
-        out.set_bits = kSetBitsMany;
-    } else if (many && out.c == 2) {
-        out.set_bits = R > 26 * sms_count ? kSetBitsMany : kSetBits;
-    } else {
-        out.set_bits = kSetBitsShared;
-        for (int bits = kSetBitsShared; bits >= kSetBitsMany && e == cudaSuccess; --bits) {
-            int n = 0;
-            e = resident(out.fn, bits, n);
-            if ((long long)n * sms_count >= want) {
-                out.set_bits = bits;
-                break;
-            }
-        }
-    }
-    out.smem = smem_of(out.set_bits);
-    for (int v = 0; v < 2 && e == cudaSuccess; ++v) {
+    if (e != cudaSuccess) return e;
+    auto resident = [&](RunKernel fn, size_t smem) -> int {
         int per_sm = 0;
-        e = resident(v ? out.fn_ext : out.fn, out.set_bits, per_sm);
-        if (e != cudaSuccess) return e;
+        if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarpsPerBlock, smem);
+        return e == cudaSuccess ? per_sm : -1;
+    };
+    Plan plan;
+    if (choose_plan(R, N, Bmax, L, sms_count,
+                    [&](const Plan &q) { return resident(pick<false>(q.c, q.sms, q.many), q.smem); }, plan) < 0)
+        return e;
+    out.c = plan.c;
+    out.sms = plan.sms;
+    out.set_bits = plan.set_bits;
+    out.smem = plan.smem;
+    out.fn = pick<false>(plan.c, plan.sms, plan.many);
+    out.fn_ext = pick<true>(plan.c, plan.sms, plan.many);
+    const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    for (int v = 0; v < 2; ++v) {
+        const int per_sm = resident(v ? out.fn_ext : out.fn, out.smem);
+        if (per_sm < 0) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         (v ? out.grid_ext : out.grid) = (int)std::min<long long>(want, (long long)sms_count * per_sm);
         (v ? out.per_sm_ext : out.per_sm) = per_sm;
     }
-    return e;
+    return cudaSuccess;
 }
 
 inline unsigned long long magic40(unsigned d) { return ((1ull << kMagicShift) + d - 1ull) / d; }

@@ -1,0 +1,76 @@
+"""The choice of kernel variant and scratch size (csrc/plan.cuh), compiled for
+the host and run over the accepted shapes with an occupancy made up from the
+shared memory and a register limit: the per-warp scratch always holds what the
+kernel writes there, a tick's ranking (a key and two byte indices per instance,
+padded to four instances) and, in the loop of few replicas with several
+instances per lane, the list of a window's formations (8 bytes per instance)."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2608_16336_gb300 import _build
+
+SRC = r"""
+#include <initializer_list>
+#include "plan.cuh"
+using namespace mt;
+struct Res { int err, c, sms, many, set_bits; long long smem; };
+// an SM of 228 KB of which every block takes 1 KB more, and reg_blocks blocks by registers
+extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_blocks) {
+    Plan p;
+    const int e = choose_plan(R, N, Bmax, make_layout(N, K, T), sms, [&](const Plan &q) {
+        const int n = q.smem > 232448 ? 0 : (int)(233472 / (q.smem + 1024));
+        return n < reg_blocks ? n : reg_blocks;
+    }, p);
+    return Res{e, p.c, p.sms, p.many, p.set_bits, (long long)p.smem};
+}
+// shapes and replica counts whose scratch is too small; the last one in *at
+extern "C" int too_small(int N, int sms, int *at) {
+    int bad = 0;
+    for (int K = 1; K <= 16; ++K)
+        for (int T : {1, 16, 64})
+            for (int B : {1, 5, 6, 64})
+                for (int reg_blocks : {4, 5, 6, 8, 10})
+                    for (int k = 1; k <= 10; ++k)
+                        for (int odd = 0; odd < 2; ++odd) {
+                            const int R = 2 * sms * k + odd;
+                            const Res p = plan(R, N, K, T, B, sms, reg_blocks);
+                            const int np = (N + 3) / 4 * 4, rank = 4 * np + 2 * np;
+                            const int list = !p.many && p.c > 1 ? 8 * N : 0;
+                            if ((1 << p.set_bits) < rank || (1 << p.set_bits) < list) {
+                                ++bad;
+                                at[0] = R; at[1] = N; at[2] = K; at[3] = T; at[4] = B;
+                            }
+                        }
+    return bad;
+}
+"""
+
+
+class Res(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int) for n in ("err", "c", "sms", "many", "set_bits")] + [("smem", ctypes.c_longlong)]
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text(SRC)
+    so = str(d / "plan.so")
+    subprocess.run([cxx, "-std=c++17", "-O2", "-Wall", "-Werror", "-shared", "-fPIC", "-x", "c++", "-I",
+                    os.path.join(_build.CSRC), str(d / "plan.cpp"), "-o", so], check=True)
+    L = ctypes.CDLL(so)
+    L.plan.restype = Res
+    return L
+
+
+@pytest.mark.parametrize("sms", [152, 148, 1])
+def test_scratch_holds_its_uses(lib, sms):
+    at = (ctypes.c_int * 5)()
+    for n in range(1, 257):
+        assert lib.too_small(n, sms, at) == 0, "R, N, K, T, Bmax = %s" % list(at)

@@ -1,0 +1,52 @@
+"""Replica counts at which a smaller per-warp scratch makes every replica
+resident on 152 SMs, or would if it held less than the shape needs, with four
+and eight instances per lane: ticks that rank all instances and windows in which
+most of them form a batch, bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+from paper_2608_16336_gb300 import mtsim
+from paper_2608_16336_gb300 import workloads as W
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def _workload(n, k, replicas):
+    """Constant iteration times and arrivals a microsecond or two apart: hundreds
+    of instances end and form batches in the same window."""
+    rng = np.random.default_rng(n + k)
+    q = 3 * n
+    traces = [(np.cumsum(rng.integers(0, 3, q)).astype(np.uint32), rng.integers(1, 60, q).astype(np.uint16),
+               rng.integers(1, 40, q).astype(np.uint16), rng.integers(0, k, q).astype(np.uint8))
+              for _ in range(replicas)]
+    return W.custom(n, 100, [k], [[max(1, 20 >> i) for i in range(k)]], [0] * replicas, traces, tokens_per_block=16,
+                    max_batch=64, iter_base_us=200, iter_us_per_prefill_token=0, iter_us_per_decode_seq=0,
+                    migrate_blocks_per_iter=8, migrate_interval_us=350, theta_num=1, theta_den=1000)
+
+
+def shared_bytes(w):
+    sim = mtsim.Simulator(w, event_log_capacity=0)
+    try:
+        return sim.launch_info()["shared_bytes"]
+    finally:
+        sim.close()
+
+
+@pytest.mark.parametrize("n,k,replicas,shrunk", [(250, 4, 700, False), (196, 7, 700, False), (196, 14, 400, False),
+                                                 (244, 4, 700, True), (256, 1, 1100, True), (123, 15, 700, True)])
+def test_scratch_at_its_least(n, k, replicas, shrunk):
+    import torch
+    w = _workload(n, k, replicas)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert (shared_bytes(w) < shared_bytes(_workload(n, k, 2))) == shrunk
+    _, st, _ = parity.check_parity(w, replicas=[0, 1, replicas // 2, replicas - 1], event_log_capacity=1 << 12)
+    assert int(st["log_events"].sum()) > 0
