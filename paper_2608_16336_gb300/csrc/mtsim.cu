@@ -2228,9 +2228,10 @@ struct Launch {
 
 // Chooses the kernel variant and grid for a problem; cudaSuccess or the error.
 inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &out) {
-    int dev = 0, sms_count = 0;
+    int dev = 0, sms_count = 0, max_smem = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms_count, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     auto resident = [&](RunKernel fn, size_t smem) -> int {
         int per_sm = 0;
@@ -2240,9 +2241,10 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
         return e == cudaSuccess ? per_sm : -1;
     };
     Plan plan;
-    if (choose_plan(R, N, Bmax, L, sms_count,
-                    [&](const Plan &q) { return resident(pick<false>(q.c, q.sms, q.many), q.smem); }, plan) < 0)
-        return e;
+    const int fits = choose_plan(R, N, Bmax, L, sms_count, (size_t)max_smem, [&](const Plan &q) {
+        return resident(pick<false>(q.c, q.sms, q.many), q.smem);
+    }, plan);
+    if (fits < 1) return fits < 0 ? e : cudaErrorInvalidConfiguration;
     out.c = plan.c;
     out.sms = plan.sms;
     out.set_bits = plan.set_bits;

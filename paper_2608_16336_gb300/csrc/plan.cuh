@@ -90,21 +90,28 @@ struct Plan {
     size_t smem = 0;   // dynamic shared memory of a block
 };
 
-// Chooses the kernel variant and the scratch for R replicas on sms_count SMs.
-// resident(plan) gives the blocks of the plan's kernel variant that fit on an
-// SM with its dynamic shared memory, or a negative value on an error, which
-// choose_plan returns.  0: success.
+// Chooses the kernel variant and the scratch for R replicas on sms_count SMs
+// whose blocks can have max_smem bytes of dynamic shared memory.  resident(plan)
+// gives the blocks of the plan's kernel variant that fit on an SM with its
+// dynamic shared memory (at most max_smem), or a negative value on an error,
+// which choose_plan returns.  Otherwise it returns the resident blocks of the
+// plan chosen; 0: the state does not fit.
 template <class Resident>
-int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, Resident resident, Plan &out) {
-    const bool sms = slots_in_shared(N, Bmax);
-    const uint32_t slot_bytes = sms ? (uint32_t)N * (uint32_t)Bmax * 16u : 0u;
+int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t max_smem, Resident resident, Plan &out) {
     const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    auto smem_of = [&](bool sms, int bits) {
+        return kHeadBytes +
+               (size_t)kWarpsPerBlock * (L.bytes + (sms ? (uint32_t)N * (uint32_t)Bmax * 16u : 0u) + (1u << bits));
+    };
+    // the records stay in HBM where the state leaves no room for them (254 or more
+    // instances with 16 tiers and about 50 tokens per block)
+    const bool sms = slots_in_shared(N, Bmax) && smem_of(true, scratch_need(N)) <= max_smem;
     out.c = lanes_c(N);
     out.sms = sms;
     auto with_bits = [&](int bits) {
         out.set_bits = bits;
-        out.smem = kHeadBytes + (size_t)kWarpsPerBlock * (L.bytes + slot_bytes + (1u << bits));
-        return resident(out);
+        out.smem = smem_of(sms, bits);
+        return out.smem <= max_smem ? resident(out) : 0;
     };
     // Which main loop (see k_run): that of many replicas above 10 (C = 1) or 14
     // (C = 2) per SM.  1,500 requests per replica, records in HBM, loop of many /
@@ -128,12 +135,13 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, Resident
     // waves alone gain nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).  It
     // never goes below what the shape's other uses take.
     int bits = kSetBitsShared;
+    while (bits > scratch_need(N) && smem_of(sms, bits) > max_smem) --bits;
     if (out.many && sms) {
         bits = kSetBitsMany;
     } else if (out.many && out.c == 2) {
         bits = R > 26 * sms_count ? kSetBitsMany : kSetBits;
     } else {
-        for (int b = kSetBitsShared; b >= scratch_need(N); --b) {
+        for (int b = bits; b >= scratch_need(N); --b) {
             const int n = with_bits(b);
             if (n < 0) return n;
             if ((long long)n * sms_count >= want) {
@@ -142,8 +150,7 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, Resident
             }
         }
     }
-    const int n = with_bits(bits > scratch_need(N) ? bits : scratch_need(N));
-    return n < 0 ? n : 0;
+    return with_bits(bits > scratch_need(N) ? bits : scratch_need(N));
 }
 
 }  // namespace mt

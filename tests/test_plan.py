@@ -1,9 +1,10 @@
 """The choice of kernel variant and scratch size (csrc/plan.cuh), compiled for
 the host and run over the accepted shapes with an occupancy made up from the
-shared memory and a register limit: the per-warp scratch always holds what the
-kernel writes there, a tick's ranking (a key and two byte indices per instance,
-padded to four instances) and, in the loop of few replicas with several
-instances per lane, the list of a window's formations (8 bytes per instance)."""
+shared memory and a register limit: every shape fits in a block's shared
+memory, and the per-warp scratch always holds what the kernel writes there, a
+tick's ranking (a key and two byte indices per instance, padded to four
+instances) and, in the loop of few replicas with several instances per lane,
+the list of a window's formations (8 bytes per instance)."""
 import ctypes
 import os
 import shutil
@@ -17,15 +18,16 @@ SRC = r"""
 #include <initializer_list>
 #include "plan.cuh"
 using namespace mt;
-struct Res { int err, c, sms, many, set_bits; long long smem; };
-// an SM of 228 KB of which every block takes 1 KB more, and reg_blocks blocks by registers
+struct Res { int fits, c, sms, many, set_bits; long long smem; };
+// an SM of 228 KB of which every block takes 1 KB more, and reg_blocks blocks by
+// registers; more than 227 KB for a block is an error, as it is for the driver
 extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_blocks) {
     Plan p;
-    const int e = choose_plan(R, N, Bmax, make_layout(N, K, T), sms, [&](const Plan &q) {
-        const int n = q.smem > 232448 ? 0 : (int)(233472 / (q.smem + 1024));
+    const int f = choose_plan(R, N, Bmax, make_layout(N, K, T), sms, 232448, [&](const Plan &q) {
+        const int n = q.smem > 232448 ? -1 : (int)(233472 / (q.smem + 1024));
         return n < reg_blocks ? n : reg_blocks;
     }, p);
-    return Res{e, p.c, p.sms, p.many, p.set_bits, (long long)p.smem};
+    return Res{f, p.c, p.sms, p.many, p.set_bits, (long long)p.smem};
 }
 // shapes and replica counts whose scratch is too small; the last one in *at
 extern "C" int too_small(int N, int sms, int *at) {
@@ -47,11 +49,26 @@ extern "C" int too_small(int N, int sms, int *at) {
                         }
     return bad;
 }
+// shapes without a plan that fits in a block's shared memory
+extern "C" int refused(int N, int *at) {
+    int bad = 0;
+    for (int K = 1; K <= 16; ++K)
+        for (int T = 1; T <= 64; ++T)
+            for (int B = 1; B <= 64; ++B)
+                for (int R : {1, 700, 8192}) {
+                    const Res p = plan(R, N, K, T, B, 152, 4);
+                    if (p.fits < 1 || p.smem > 232448) {
+                        ++bad;
+                        at[0] = R; at[1] = N; at[2] = K; at[3] = T; at[4] = B;
+                    }
+                }
+    return bad;
+}
 """
 
 
 class Res(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_int) for n in ("err", "c", "sms", "many", "set_bits")] + [("smem", ctypes.c_longlong)]
+    _fields_ = [(n, ctypes.c_int) for n in ("fits", "c", "sms", "many", "set_bits")] + [("smem", ctypes.c_longlong)]
 
 
 @pytest.fixture(scope="module")
@@ -74,3 +91,9 @@ def test_scratch_holds_its_uses(lib, sms):
     at = (ctypes.c_int * 5)()
     for n in range(1, 257):
         assert lib.too_small(n, sms, at) == 0, "R, N, K, T, Bmax = %s" % list(at)
+
+
+def test_every_accepted_shape_has_a_plan(lib):
+    at = (ctypes.c_int * 5)()
+    for n in range(1, 257):
+        assert lib.refused(n, at) == 0, "R, N, K, T, Bmax = %s" % list(at)

@@ -20,7 +20,7 @@ def _cuda():
     torch.cuda.set_device(0)
 
 
-def _workload(n, k, replicas):
+def _workload(n, k, replicas, block_tokens=16, batch=64):
     """Constant iteration times and arrivals a microsecond or two apart: hundreds
     of instances end and form batches in the same window."""
     rng = np.random.default_rng(n + k)
@@ -28,8 +28,8 @@ def _workload(n, k, replicas):
     traces = [(np.cumsum(rng.integers(0, 3, q)).astype(np.uint32), rng.integers(1, 60, q).astype(np.uint16),
                rng.integers(1, 40, q).astype(np.uint16), rng.integers(0, k, q).astype(np.uint8))
               for _ in range(replicas)]
-    return W.custom(n, 100, [k], [[max(1, 20 >> i) for i in range(k)]], [0] * replicas, traces, tokens_per_block=16,
-                    max_batch=64, iter_base_us=200, iter_us_per_prefill_token=0, iter_us_per_decode_seq=0,
+    return W.custom(n, 100, [k], [[max(1, 20 >> i) for i in range(k)]], [0] * replicas, traces, tokens_per_block=block_tokens,
+                    max_batch=batch, iter_base_us=200, iter_us_per_prefill_token=0, iter_us_per_decode_seq=0,
                     migrate_blocks_per_iter=8, migrate_interval_us=350, theta_num=1, theta_den=1000)
 
 
@@ -50,3 +50,15 @@ def test_scratch_at_its_least(n, k, replicas, shrunk):
         assert (shared_bytes(w) < shared_bytes(_workload(n, k, 2))) == shrunk
     _, st, _ = parity.check_parity(w, replicas=[0, 1, replicas // 2, replicas - 1], event_log_capacity=1 << 12)
     assert int(st["log_events"].sum()) > 0
+
+
+@pytest.mark.parametrize("n,block_tokens,records_in_shared", [(256, 52, 1), (249, 64, 1), (254, 60, 0), (256, 64, 0)])
+def test_largest_state_beside_the_records(n, block_tokens, records_in_shared):
+    """16 tiers and a batch of 6: the records and a 4 KB scratch do not fit together."""
+    w = _workload(n, 16, 3, block_tokens, 6)
+    sim = mtsim.Simulator(w, event_log_capacity=0)
+    try:
+        assert sim.launch_info()["slots_in_shared"] == records_in_shared
+    finally:
+        sim.close()
+    parity.check_parity(w, event_log_capacity=1 << 14)
