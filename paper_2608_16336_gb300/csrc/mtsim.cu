@@ -2235,7 +2235,9 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     if (e != cudaSuccess) return e;
     auto resident = [&](RunKernel fn, size_t smem) -> int {
         int per_sm = 0;
-        if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // The limit belongs to the kernel, not to a launch: it is always set to the
+        // device's, so that no plan lowers it for an object that launches later.
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * kWarpsPerBlock, smem);
         return e == cudaSuccess ? per_sm : -1;

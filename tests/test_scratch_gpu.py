@@ -1,7 +1,9 @@
-"""Replica counts at which a smaller per-warp scratch makes every replica
+"""Shared memory of the simulation kernel.  Replica counts at which a smaller per-warp scratch makes every replica
 resident on 152 SMs, or would if it held less than the shape needs, with four
 and eight instances per lane: ticks that rank all instances and windows in which
-most of them form a batch, bit-exact against the oracle."""
+most of them form a batch; states that leave little room; live objects whose
+kernels are the same and whose shared memory differs.  Bit-exact against the
+oracle."""
 import numpy as np
 import pytest
 
@@ -62,3 +64,25 @@ def test_largest_state_beside_the_records(n, block_tokens, records_in_shared):
     finally:
         sim.close()
     parity.check_parity(w, event_log_capacity=1 << 14)
+
+
+@pytest.mark.parametrize("first,second", [((128, 8, 64), (128, 8, 1000)), ((128, 8, 1000), (128, 8, 64)),
+                                          ((256, 16, 2), (256, 1, 3)), ((64, 16, 2), (40, 9, 2))])
+def test_live_objects(first, second):
+    """Neither object's launch depends on what the other planned, in either order."""
+    ws = [_workload(*first), _workload(*second)]
+    sims = [mtsim.Simulator(w, event_log_capacity=1 << 12) for w in ws]
+    try:
+        assert sims[0].launch_info()["shared_bytes"] != sims[1].launch_info()["shared_bytes"]
+        for s in sims:
+            s.load()
+        for w, s in zip(ws, sims):
+            assert s.run() == 0
+            res, st, ev = s.metrics()
+            events = [s.events_of(ev, st, r) for r in range(w.num_replicas)]
+            ref = parity.run_oracle(w, [0, w.num_replicas - 1], event_log_capacity=1 << 12)
+            for r in (0, w.num_replicas - 1):
+                parity.compare_replica(w, r, res, st, events, ref[r])
+    finally:
+        for s in sims:
+            s.close()
