@@ -478,6 +478,17 @@ __global__ void __launch_bounds__(1024) k_latency_replica(int R, const long long
     }
 }
 
+// Lets kernel f have the device's dynamic shared memory per block.  The limit
+// belongs to the kernel: were it set to each launch's size, a launch from
+// another host thread could find it lowered.
+template <class F>
+cudaError_t allow_shared(F f) {
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e == cudaSuccess ? cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most) : e;
+}
+
 inline size_t replica_bytes(int qcap, int KT, int threads) {
     const size_t G = (size_t)KT * 3, S = G * 3;
     return S * 16 + (size_t)(threads / 32) * G * 12 + S * (kSelBins / 2) * 4 + (size_t)qcap * 13;
@@ -497,9 +508,7 @@ cudaError_t launch_replicas(int R, long long qmax, const long long *offsets, int
                                  : (qmax <= 512 ? 128 : qmax <= 1024 ? 256 : qmax <= 8192 ? 512 : 1024);
     const size_t smem = replica_bytes(qcap, KT, threads);
     if (smem > kMaxShared) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)
-        e = cudaFuncSetAttribute(k_latency_replica, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k_latency_replica);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_latency_replica, threads, smem);
     if (e != cudaSuccess) return e;
@@ -523,10 +532,8 @@ cudaError_t launch(const int *chunk_rep, const long long *chunk_b0, int nchunks,
         // accumulators take 12 bytes per thread and group)
         const int threads = KT <= 4 ? 256 : 128;
         const size_t smem = (size_t)KT * 3 * (12u * (size_t)threads + 4u * SIM_HIST_BUCKETS);  // <= 119,808 bytes
-        if (smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(k_latency_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        e = allow_shared(k_latency_hist);
+        if (e != cudaSuccess) return e;
         k_latency_hist<<<grid, threads, smem, stream>>>(chunk_rep, chunk_b0, nchunks, offsets, KT, arrival, olen, tier,
                                                         res, out);
         e = cudaGetLastError();

@@ -2,9 +2,12 @@
 16,383 requests, the block sizes it changes at, ragged warps, the tier counts
 whose shared memory differs, all values alike) and just past it, bit-exact
 against sorted values."""
+import threading
+
 import numpy as np
 import pytest
 
+from paper_2608_16336_gb300 import mtsim
 from paper_2608_16336_gb300 import workloads as W
 from tests.test_latency_gpu import compare, gpu_stats
 
@@ -48,3 +51,34 @@ def test_largest(q, alike):
 def test_unfinished_requests_left_out():
     w = _workload((700, 40), 3, False, 3)
     compare(w, gpu_stats(w, max_steps=150), range(2), max_steps=150)
+
+
+@pytest.mark.parametrize("sizes", [((40,), (400,)), ((17000,), (17001, 5))])  # one kernel; streaming passes
+def test_two_host_threads(sizes):
+    """Objects in use by two host threads whose launches take different shared memory."""
+    ws = [_workload(s, k, False, 11 + k) for s, k in zip(sizes, (9, 16))]
+    sims = [mtsim.Simulator(w, event_log_capacity=0) for w in ws]
+    errors, got = [], [None, None]
+
+    def work(i):
+        try:
+            for _ in range(3000):
+                got[i] = sims[i].latency_stats()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    try:
+        for s in sims:
+            s.load()
+            s.run()
+        threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not errors, errors[0]
+        for w, g in zip(ws, got):
+            compare(w, g, range(w.num_replicas))
+    finally:
+        for s in sims:
+            s.close()
