@@ -154,7 +154,8 @@ struct Params {
     int drains;                   // a drain schedule is loaded
     unsigned long long lcm_lo, lcm_hi;  // lcm(1, ..., Bmax) as two 64-bit halves
     Layout L;
-    int set_bits;                 // per-warp scratch of distinct_times, log2 of its bytes
+    int set_bits;                 // scratch of distinct_times (several instances per lane), log2 of its bytes
+    uint32_t scratch;             // per-warp scratch, bytes
     const long long *offsets;
     const uint32_t *drain_src;    // [R][N] drain start times, or NULL
     const uint32_t *arrival;
@@ -260,7 +261,7 @@ __device__ __forceinline__ void bind_ctx(Ctx &x, const Params &p, unsigned char 
                                          uint32_t t) {
     const uint32_t slot_bytes = SMS ? (uint32_t)p.N * (uint32_t)p.Bmax * 16u : 0u;
     unsigned char *blob =
-        smem + kHeadBytes + (size_t)(threadIdx.x >> 5) * (p.L.bytes + slot_bytes + (1u << p.set_bits));
+        smem + kHeadBytes + (size_t)(threadIdx.x >> 5) * (p.L.bytes + slot_bytes + p.scratch);
     bind_blob(x, p.L, blob);
     x.slots = SMS ? reinterpret_cast<uint4 *>(blob + p.L.bytes) : p.slots + (size_t)r * p.N * p.Bmax;
     x.tset = reinterpret_cast<uint32_t *>(blob + p.L.bytes + slot_bytes);
@@ -1368,14 +1369,22 @@ __device__ __noinline__ int tick_call(uint4 *node, uint32_t Q, int r, uint32_t t
 }
 
 // The number of distinct times et[j] < t1 over the warp, for a window
-// [tb, t1).  Collective.  Every instance writes its index into a byte that its
-// time selects and reads it back: one index per byte wins and counts, nothing
-// needs clearing.  When the scratch has a byte for every microsecond of the
-// window the others have the winner's time; in a longer window the byte is
-// hashed, the winner's time is compared, and the instances that met another
-// time try again without the winners (at least one per byte leaves each round).
+// [tb, t1), in two parts: distinct_times when it opens, distinct_count when it
+// closes.  Collective.  One instance per lane: the lanes that share a time form a
+// group (match), which nothing waits for until the window closes.  (A count in
+// shared memory, as below, cost 4 KB or 1 KB per warp and 160 instructions more:
+// 1,024 x 16 at 0.85 load with 20,000 requests 82.6 -> 78.4 ms, 1,024 x 24, four
+// blocks per SM instead of three, 19.3 -> 10.7 ms, one 4-instance cluster 42.2 ->
+// 40.1 ms, 3,840 x 32 16.9 -> 16.4 ms.)  Several: every instance writes its index
+// into a byte that its time selects and reads it back: one index per byte wins
+// and counts, nothing needs clearing.  When the scratch has a byte for every
+// microsecond of the window the others have the winner's time; in a longer window
+// the byte is hashed, the winner's time is compared, and the instances that met
+// another time try again without the winners (at least one per byte leaves each
+// round).
 template <int C>
 __device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, uint32_t t1, const uint32_t (&et)[C]) {
+    if constexpr (C == 1) return __match_any_sync(kFull, et[0] < t1 ? et[0] : kNone);
     uint8_t *set = reinterpret_cast<uint8_t *>(x.tset);
     uint32_t fresh = 0;
     if (!MT_RARE(t1 - tb > 1u << x.set_bits)) {
@@ -1416,8 +1425,13 @@ __device__ __forceinline__ uint32_t distinct_times(const Ctx &x, uint32_t tb, ui
                 }
         }
     }
-    if (C == 1) return __popc(__ballot_sync(kFull, fresh != 0));
     return __reduce_add_sync(kFull, fresh);
+}
+
+// The count; in: the lane's instance had an event in the window (C = 1).
+template <int C>
+__device__ __forceinline__ uint32_t distinct_count(const Ctx &x, uint32_t u, bool in) {
+    return C == 1 ? (uint32_t)__popc(__ballot_sync(kFull, in && __ffs(u) - 1 == x.lane)) : u;
 }
 
 __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *src, uint32_t bytes, int lane) {
@@ -1559,7 +1573,7 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
         const bool ends = busy < t1;
         if (__any_sync(kFull, ends && !quiet)) break;
         const uint32_t et[1] = {busy};
-        cn.steps += distinct_times<1>(x, tb, t1, et);
+        const uint32_t group = distinct_times<1>(x, tb, t1, et);
         if (ends) {
             ++done;
             tmax = max(tmax, busy);
@@ -1569,6 +1583,7 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
             busy += dur;
             look();
         }
+        cn.steps += distinct_count<1>(x, group, ends);
         tb = __reduce_min_sync(kFull, busy);
     }
     if (done) {
@@ -1688,6 +1703,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
             bool any_b = false, in_cm = false;  // second events / mode-1 steps of the window remain
             uint32_t t1 = 0, cm = 0;            // window end; own instances stepped in mode 1
             uint32_t ucount = 0;                // distinct event times of the window
+            bool in_window = false;             // the own instance has an event in it (C = 1)
             for (;;) {
                 int mode;
                 uint32_t et[C];      // event time of each own instance in this pass
@@ -1733,6 +1749,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                             t1 = (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
                             // distinct event times of the window, and the latest
                             ucount = distinct_times<C>(x, tb, t1, et);
+                            in_window = et[0] < t1;
 #pragma unroll
                             for (int j = 0; j < C; ++j)
                                 if (et[j] < t1) tmax = max(tmax, et[j]);
@@ -1867,7 +1884,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                     // the window closes
                     in_cm = false;
                     x.hold = false;
-                    cn.steps += ucount;
+                    cn.steps += distinct_count<C>(x, ucount, in_window);
                 }
                 if (__any_sync(kFull, cn.held || cn.status < 0)) {
                     if (mode == 0 || mode == 3) mig = flush_held<C>(x, cn);
@@ -1899,6 +1916,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                         (uint32_t)min((unsigned long long)tg, (unsigned long long)tb + (uint32_t)p.base);
                     // distinct event times of the window, and the latest
                     const uint32_t ucount = distinct_times<C>(x, tb, t1, bz);
+                    const bool in_window = bz[0] < t1;
 #pragma unroll
                     for (int j = 0; j < C; ++j)
                         if (bz[j] < t1) tmax = max(tmax, bz[j]);
@@ -1988,7 +2006,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 :
                         }
                         x.hold = false;
                     }
-                    cn.steps += ucount;
+                    cn.steps += distinct_count<C>(x, ucount, in_window);
                     if (__any_sync(kFull, cn.held || cn.status < 0)) {
                         mig = flush_held<C>(x, cn);
                         if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
@@ -2223,6 +2241,7 @@ struct Launch {
     int c = 1;                       // instances per lane
     bool sms = false;                // running-request records in shared memory
     int set_bits = 0;                // scratch of distinct_times, log2 of its bytes
+    uint32_t scratch = 0;            // scratch of a warp, bytes
     size_t smem = 0;
 };
 
@@ -2250,6 +2269,7 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
     out.c = plan.c;
     out.sms = plan.sms;
     out.set_bits = plan.set_bits;
+    out.scratch = plan.scratch;
     out.smem = plan.smem;
     out.fn = pick<false>(plan.c, plan.sms, plan.many);
     out.fn_ext = pick<true>(plan.c, plan.sms, plan.many);
@@ -2418,6 +2438,7 @@ mt::Params make_params(const sim_t *s, long long max_steps) {
     p.work = s->d_work;
     p.order = s->d_order;
     p.set_bits = s->launch.set_bits;
+    p.scratch = s->launch.scratch;
     return p;
 }
 
@@ -2988,6 +3009,7 @@ extern "C" int sim_run_static(const sim_cluster_t *cl, const sim_tier_table_t *t
     p.log = events;
     p.work = (int *)(base + o_work);
     p.set_bits = lc.set_bits;
+    p.scratch = lc.scratch;
     int *rt = (int *)(base + o_rt), *tk = (int *)(base + o_tk), *th = (int *)(base + o_th);
 
     // Inputs the kernels read from device memory; the work counter and flags start at zero.

@@ -20,9 +20,10 @@ constexpr uint32_t kMagicBytes = 528;  // ceil(2^64 / d) for d = 0..64, rounded 
 // they are in shared memory, and the scratch.
 constexpr uint32_t kHeadBytes = kParamBytes + kMagicBytes;
 
-// Bytes (2^n) of the per-warp scratch: what a window's distinct event times are
-// counted in, and also the tick's ranking and the list of a window's formations
-// (scratch_need).  Small where many warps share an SM's shared memory (choose_plan).
+// The per-warp scratch of variants with several instances per lane, log2 of its
+// bytes: a window's distinct event times are counted in it, a tick's ranking and
+// the list of a window's formations are kept there (scratch_need).  Small where
+// many warps share an SM's shared memory (choose_plan).
 constexpr int kSetBitsShared = 12, kSetBits = 11, kSetBitsMany = 10;
 
 struct Layout {
@@ -71,22 +72,21 @@ inline Layout make_layout(int N, int K, int T) {
 constexpr uint32_t kSmemSlotLimit = 24u * 1024u;
 inline bool slots_in_shared(int N, int Bmax) { return (uint32_t)N * (uint32_t)Bmax * 16u <= kSmemSlotLimit; }
 
-// The least scratch, log2 of its bytes: the ranking of a tick (ranked_tick)
-// takes a key and two indices per instance, 6 bytes for N rounded up to a
-// multiple of 4, and the list of a window's formations (list_own) 8 bytes per
-// instance where a lane owns several.
-inline int scratch_need(int N) {
+// The least scratch in bytes: the ranking of a tick (ranked_tick) takes a key
+// and two indices per instance, 6 bytes for N rounded up to a multiple of 4, and
+// the list of a window's formations (list_own) 8 bytes per instance where a
+// lane owns several.
+inline uint32_t scratch_need(int N) {
     const uint32_t rank = 6u * (((uint32_t)N + 3u) & ~3u), list = lanes_c(N) > 1 ? 8u * (uint32_t)N : 0u;
-    int bits = kSetBitsMany;
-    while ((1u << bits) < rank || (1u << bits) < list) ++bits;
-    return bits;
+    return ((rank > list ? rank : list) + 15u) & ~15u;
 }
 
 struct Plan {
     int c = 1;         // instances per lane
     bool sms = false;  // running-request records in shared memory
     bool many = false; // the loop of many replicas
-    int set_bits = 0;  // scratch, log2 of its bytes
+    int set_bits = 0;  // the part of the scratch that counts event times, log2 of its bytes
+    uint32_t scratch = 0;  // scratch of a warp, bytes
     size_t smem = 0;   // dynamic shared memory of a block
 };
 
@@ -99,17 +99,22 @@ struct Plan {
 template <class Resident>
 int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t max_smem, Resident resident, Plan &out) {
     const long long want = ((long long)R + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    // scratch of a given number of bits (0: event times are not counted in it)
+    auto scratch_of = [&](int bits) { return bits > 0 ? 1u << bits : scratch_need(N); };
     auto smem_of = [&](bool sms, int bits) {
         return kHeadBytes +
-               (size_t)kWarpsPerBlock * (L.bytes + (sms ? (uint32_t)N * (uint32_t)Bmax * 16u : 0u) + (1u << bits));
+               (size_t)kWarpsPerBlock * (L.bytes + (sms ? (uint32_t)N * (uint32_t)Bmax * 16u : 0u) + scratch_of(bits));
     };
+    int least = lanes_c(N) > 1 ? kSetBitsMany : 0;
+    while (scratch_of(least) < scratch_need(N)) ++least;
     // the records stay in HBM where the state leaves no room for them (254 or more
     // instances with 16 tiers and about 50 tokens per block)
-    const bool sms = slots_in_shared(N, Bmax) && smem_of(true, scratch_need(N)) <= max_smem;
+    const bool sms = slots_in_shared(N, Bmax) && smem_of(true, least) <= max_smem;
     out.c = lanes_c(N);
     out.sms = sms;
     auto with_bits = [&](int bits) {
         out.set_bits = bits;
+        out.scratch = scratch_of(bits);
         out.smem = smem_of(sms, bits);
         return out.smem <= max_smem ? resident(out) : 0;
     };
@@ -123,34 +128,27 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
     // 24 x 400 27.7 / 24.4 (3 blocks).
     out.many = (sms ? out.c == 1 : out.c <= 2) && R > (sms ? 10 : out.c == 1 ? 10 : 14) * sms_count;
     if (out.many && sms) {
-        const int n = with_bits(kSetBitsMany);
+        const int n = with_bits(0);
         if (n < 0) return n;
         out.many = n >= 5;
     }
-    // The scratch: 4 KB holds a window of the default `base` of 4 ms directly.
-    // Where two instances per lane share an SM with 17 other warps it has 2 KB,
-    // and 1 KB, with two warps more, for sweeps of several waves (8,192 x 64:
-    // 110.2 against 112.5 ms).  Elsewhere it shrinks where that makes every replica
-    // resident (1,400 x 16 x 500: 4.9 instead of 7.1 ms); more warps of several
-    // waves alone gain nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).  It
-    // never goes below what the shape's other uses take.
+    // The scratch with several instances per lane: 4 KB holds a window of the
+    // default `base` of 4 ms directly.  Where two instances per lane share an SM
+    // with 17 other warps it has 2 KB, and 1 KB, with two warps more, for sweeps of
+    // several waves (8,192 x 64: 110.2 against 112.5 ms).  Elsewhere it shrinks where
+    // that makes every replica resident; more warps of several waves alone gain
+    // nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).  It never goes below
+    // what the shape's other uses take.
+    if (out.c == 1) return with_bits(0);
+    if (out.many) return with_bits(R > 26 * sms_count ? kSetBitsMany : kSetBits);
     int bits = kSetBitsShared;
-    while (bits > scratch_need(N) && smem_of(sms, bits) > max_smem) --bits;
-    if (out.many && sms) {
-        bits = kSetBitsMany;
-    } else if (out.many && out.c == 2) {
-        bits = R > 26 * sms_count ? kSetBitsMany : kSetBits;
-    } else {
-        for (int b = bits; b >= scratch_need(N); --b) {
-            const int n = with_bits(b);
-            if (n < 0) return n;
-            if ((long long)n * sms_count >= want) {
-                bits = b;
-                break;
-            }
-        }
+    while (bits > least && smem_of(sms, bits) > max_smem) --bits;
+    for (int b = bits; b >= least; --b) {
+        const int n = with_bits(b);
+        if (n < 0) return n;
+        if ((long long)n * sms_count >= want) return n;
     }
-    return with_bits(bits > scratch_need(N) ? bits : scratch_need(N));
+    return with_bits(bits);
 }
 
 }  // namespace mt

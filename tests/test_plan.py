@@ -18,7 +18,7 @@ SRC = r"""
 #include <initializer_list>
 #include "plan.cuh"
 using namespace mt;
-struct Res { int fits, c, sms, many, set_bits; long long smem; };
+struct Res { int fits, c, sms, many, set_bits, scratch; long long smem; };
 // an SM of 228 KB of which every block takes 1 KB more, and reg_blocks blocks by
 // registers; more than 227 KB for a block is an error, as it is for the driver
 extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_blocks) {
@@ -27,7 +27,7 @@ extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_block
         const int n = q.smem > 232448 ? -1 : (int)(233472 / (q.smem + 1024));
         return n < reg_blocks ? n : reg_blocks;
     }, p);
-    return Res{f, p.c, p.sms, p.many, p.set_bits, (long long)p.smem};
+    return Res{f, p.c, p.sms, p.many, p.set_bits, (int)p.scratch, (long long)p.smem};
 }
 // shapes and replica counts whose scratch is too small; the last one in *at
 extern "C" int too_small(int N, int sms, int *at) {
@@ -42,7 +42,8 @@ extern "C" int too_small(int N, int sms, int *at) {
                             const Res p = plan(R, N, K, T, B, sms, reg_blocks);
                             const int np = (N + 3) / 4 * 4, rank = 4 * np + 2 * np;
                             const int list = !p.many && p.c > 1 ? 8 * N : 0;
-                            if ((1 << p.set_bits) < rank || (1 << p.set_bits) < list) {
+                            const int scratch = (int)p.scratch;
+                            if (scratch < rank || scratch < list || (p.c > 1 && scratch < 1 << p.set_bits)) {
                                 ++bad;
                                 at[0] = R; at[1] = N; at[2] = K; at[3] = T; at[4] = B;
                             }
@@ -68,7 +69,7 @@ extern "C" int refused(int N, int *at) {
 
 
 class Res(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_int) for n in ("fits", "c", "sms", "many", "set_bits")] + [("smem", ctypes.c_longlong)]
+    _fields_ = [(n, ctypes.c_int) for n in ("fits", "c", "sms", "many", "set_bits", "scratch")] + [("smem", ctypes.c_longlong)]
 
 
 @pytest.fixture(scope="module")
@@ -97,3 +98,10 @@ def test_every_accepted_shape_has_a_plan(lib):
     at = (ctypes.c_int * 5)()
     for n in range(1, 257):
         assert lib.refused(n, at) == 0, "R, N, K, T, Bmax = %s" % list(at)
+
+
+def test_one_instance_per_lane_keeps_its_residency(lib):
+    """24 instances with 4 tiers and a batch of 64: four blocks per SM as long as the
+    scratch holds the ranking alone, so that 1,024 replicas are all resident."""
+    p = lib.plan(1024, 24, 4, 16, 64, 152, 6)
+    assert (p.c, p.sms, p.many, p.fits) == (1, 1, 0, 4)
