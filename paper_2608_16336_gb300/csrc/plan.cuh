@@ -118,37 +118,65 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
         out.smem = smem_of(sms, bits);
         return out.smem <= max_smem ? resident(out) : 0;
     };
-    // Which main loop (see k_run): that of many replicas above 10 (C = 1) or 14
-    // (C = 2) per SM.  1,500 requests per replica, records in HBM, loop of many /
-    // of few, ms: 32 instances, 304 replicas 9.2 / 7.9, 1,216 9.9 / 9.0, 1,824 10.7 /
-    // 11.5, 2,432 11.4 / 20.1; 64 instances, 304 replicas 15.5 / 12.0, 1,824 18.8 /
-    // 15.7, 2,432 20.1 / 28.0 (14 warps of the loop of few fit on an SM).  With
-    // records in shared memory only where at least 5 blocks fit: 8,192 replicas x 8
-    // x 400 requests 15.9 / 21.6, 8,192 x 16 x 500 26.0 / 28.3 (5 blocks), 6,000 x
-    // 24 x 400 27.7 / 24.4 (3 blocks).
-    out.many = (sms ? out.c == 1 : out.c <= 2) && R > (sms ? 10 : out.c == 1 ? 10 : 14) * sms_count;
-    if (out.many && sms) {
-        const int n = with_bits(0);
-        if (n < 0) return n;
-        out.many = n >= 5;
+    auto waves = [&](int n) { return n > 0 ? (want + (long long)n * sms_count - 1) / ((long long)n * sms_count) : 1ll << 40; };
+    // The plan of one main loop, which out keeps: its scratch and its resident
+    // blocks.  With several instances per lane 4 KB of scratch hold a window of the
+    // default `base` of 4 ms directly.  The loop of few takes less where that makes
+    // every replica resident (more warps of several waves alone gain nothing: 2,048 x
+    // 100 x 500 26.3 against 23.9 ms).  The loop of many has 2 KB, and for sweeps of
+    // several waves 1 KB where more blocks then fit (8,192 x 64 with 4 tiers, ten
+    // blocks instead of nine: 110.2 against 112.5 ms; with 6 tiers eight blocks either
+    // way).  Never less than the shape's other uses take.
+    auto plan_loop = [&](bool many) {
+        out.many = many;
+        if (out.c == 1) return with_bits(0);
+        if (many) {
+            const int n = with_bits(kSetBits);
+            if (n < 0 || R <= 26 * sms_count) return n;
+            const int n2 = with_bits(kSetBitsMany);
+            return n2 < 0 || n2 > n ? n2 : with_bits(kSetBits);
+        }
+        int bits = kSetBitsShared;
+        while (bits > least && smem_of(sms, bits) > max_smem) --bits;
+        for (int b = bits; b >= least; --b) {
+            const int n = with_bits(b);
+            if (n < 0 || waves(n) == 1) return n;
+        }
+        return with_bits(bits);
+    };
+    // Which main loop (see k_run), up to 64 instances.
+    if (out.c == 1 && sms) {
+        // Records in shared memory: both loops have about the same residency, and the
+        // loop of many scales better with the warps that share an SM's instruction
+        // cache, the sooner the fewer instances share a window.  Loop of few / of many,
+        // ms, at 0.85 load: 4 instances, 912 replicas 16.3 / 17.0, 1,216 19.3 / 17.2; 8,
+        // 912 13.5 / 14.5, 1,216 15.9 / 14.7; 12, 1,216 9.2 / 9.8, 1,368 10.3 / 10.3; 16,
+        // 1,216 16.5 / 17.2, 1,520 19.7 / 18.4 (800 requests 5.4 / 6.1, 8,000 41.5 / 35.7);
+        // one instance, 1,520 6.7 / 7.7.  At 0.3 to 0.4 load the lines lie about 1
+        // replica per SM higher.  Only where at least 5 blocks fit (6,000 x 24 x 400,
+        // 3 blocks: 24.4 / 27.7).
+        const int per_sm = N == 1 ? 12 : N <= 8 ? 7 : 9;
+        if (R > per_sm * sms_count) {
+            const int n = plan_loop(true);
+            if (n < 0 || n >= 5) return n;
+        }
+    } else if (out.c <= 2 && !sms) {
+        // Records in HBM: a wave of the loop of few takes less time than one of the
+        // loop of many, which holds more replicas.  Loop of few / of many, ms: 64
+        // instances, 4 tiers (12 and 18 to 20 warps per SM), 1,824 replicas 13.8 / 18.2,
+        // 2,000 23.7 / 19.2, 3,648 21.6 / 26.8, 4,000 37.9 / 37.2; 16 tiers (8 and 10
+        // warps) 2,432 18.5 / 25.1, 4,000 34.0 / 37.2; 40 instances 1,824 13.1 / 15.5, 2,000
+        // 21.5 / 16.6; 32 instances (12 and 16 warps) 1,824 9.0 / 10.0, 2,128 15.3 / 10.7,
+        // 3,648 17.6 / 19.5, 4,864 24.8 / 20.9.  Past three waves the rate of a full SM
+        // decides: 16,384 x 64 x 400 with 4, 8, 13 and 16 tiers (20, 14, 12 and 10 warps of
+        // the loop of many) 81.7 / 65.9, 83.6 / 79.2, 90.3 / 87.2, 93.1 / 100.1.
+        const int few = plan_loop(false);
+        if (few < 0) return few;
+        const int many = plan_loop(true);
+        if (many < 0) return many;
+        if (waves(few) > 3 ? many >= 6 : (out.c == 1 ? 11 : 14) * waves(many) < 10 * waves(few)) return many;
     }
-    // The scratch with several instances per lane: 4 KB holds a window of the
-    // default `base` of 4 ms directly.  Where two instances per lane share an SM
-    // with 17 other warps it has 2 KB, and 1 KB, with two warps more, for sweeps of
-    // several waves (8,192 x 64: 110.2 against 112.5 ms).  Elsewhere it shrinks where
-    // that makes every replica resident; more warps of several waves alone gain
-    // nothing there (2,048 x 100 x 500: 26.3 against 23.9 ms).  It never goes below
-    // what the shape's other uses take.
-    if (out.c == 1) return with_bits(0);
-    if (out.many) return with_bits(R > 26 * sms_count ? kSetBitsMany : kSetBits);
-    int bits = kSetBitsShared;
-    while (bits > least && smem_of(sms, bits) > max_smem) --bits;
-    for (int b = bits; b >= least; --b) {
-        const int n = with_bits(b);
-        if (n < 0) return n;
-        if ((long long)n * sms_count >= want) return n;
-    }
-    return with_bits(bits);
+    return plan_loop(false);
 }
 
 }  // namespace mt

@@ -20,12 +20,13 @@ SRC = r"""
 using namespace mt;
 struct Res { int fits, c, sms, many, set_bits, scratch; long long smem; };
 // an SM of 228 KB of which every block takes 1 KB more, and reg_blocks blocks by
-// registers; more than 227 KB for a block is an error, as it is for the driver
+// registers (0: what the kernels' registers allow); more than 227 KB for a block is an error, as it is for the driver
 extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_blocks) {
     Plan p;
     const int f = choose_plan(R, N, Bmax, make_layout(N, K, T), sms, 232448, [&](const Plan &q) {
         const int n = q.smem > 232448 ? -1 : (int)(233472 / (q.smem + 1024));
-        return n < reg_blocks ? n : reg_blocks;
+        const int regs = reg_blocks > 0 ? reg_blocks : !q.many ? (q.c <= 2 ? 6 : 4) : q.c == 2 ? 10 : 8;
+        return n < regs ? n : regs;
     }, p);
     return Res{f, p.c, p.sms, p.many, p.set_bits, (int)p.scratch, (long long)p.smem};
 }
@@ -105,3 +106,22 @@ def test_one_instance_per_lane_keeps_its_residency(lib):
     scratch holds the ranking alone, so that 1,024 replicas are all resident."""
     p = lib.plan(1024, 24, 4, 16, 64, 152, 6)
     assert (p.c, p.sms, p.many, p.fits) == (1, 1, 0, 4)
+
+
+@pytest.mark.parametrize("n,k,replicas,many", [
+    (64, 4, 1824, 0), (64, 4, 1825, 1), (64, 4, 2736, 1), (64, 4, 2737, 0), (64, 4, 3648, 0), (64, 4, 3649, 1),
+    (64, 4, 8192, 1), (64, 10, 16384, 1), (64, 16, 1520, 0), (64, 16, 2432, 0), (64, 16, 16384, 0), (40, 4, 1825, 1), (32, 4, 1824, 0), (32, 4, 1825, 1),
+    (32, 4, 2433, 0), (32, 10, 3840, 1), (1, 4, 1824, 0), (8, 4, 1064, 0), (8, 4, 1065, 1), (16, 4, 1368, 0),
+    (16, 4, 1369, 1), (24, 4, 8192, 0), (65, 4, 8192, 0)])
+def test_main_loop(lib, n, k, replicas, many):
+    """The loop whose waves take less time, on either side of the replica counts that
+    fill a wave of 152 SMs; with records in shared memory, of the lines drawn there."""
+    p = lib.plan(replicas, n, k, 16, 64, 152, 0)
+    assert p.many == many
+
+
+@pytest.mark.parametrize("k,replicas,scratch", [(4, 2736, 2048), (4, 3952, 2048), (4, 3953, 1024), (4, 16384, 1024), (3, 16384, 2048),
+                                                (5, 16384, 1024), (8, 16384, 2048)])
+def test_small_scratch_only_where_it_holds_more_blocks(lib, k, replicas, scratch):
+    p = lib.plan(replicas, 64, k, 16, 64, 152, 0)
+    assert p.many == 1 and p.scratch == scratch
