@@ -1624,9 +1624,12 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
 // 124 registers.  (10 resident blocks, with 1 KB less of scratch per warp:
 // 110.4 ms; 12 blocks would need 80 registers, which spills.)  One instance
 // per lane: 8 blocks (110 registers) 20.8 ms on 3,840 x 32 x 1,000, 10 blocks
-// 21.8 ms, 12 blocks (80 registers) 21.9 ms.
+// 21.8 ms, 12 blocks (80 registers) 21.9 ms.  Four per lane: a bound of 6 blocks
+// gives 168 registers, which 12 warps of an SM can have; unbounded it takes 181, for 8
+// warps: 1,500 x 128 x 500 21.9 -> 15.5 ms, 1,824 x 100 x 500 21.0 -> 16.1, 256 x 128 x
+// 6,000 the same (blocks_at_once).
 template <int C, bool SMS, bool EXT, bool MANY>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 2 ? 10 : 8) k_run(Params p) {
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) : C == 2 ? 10 : 8) k_run(Params p) {
     // At 96 registers there is no room for values kept across calls: the rare
     // paths stay inline (116 ms instead of 196 on the 64-instance sweep), and
     // copy stages go source by source.
@@ -2278,7 +2281,8 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
         const int per_sm = resident(v ? out.fn_ext : out.fn, out.smem);
         if (per_sm < 0) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        (v ? out.grid_ext : out.grid) = (int)std::min<long long>(want, (long long)sms_count * per_sm);
+        (v ? out.grid_ext : out.grid) =
+            (int)std::min<long long>(want, (long long)sms_count * blocks_at_once(out.c, want, sms_count, per_sm));
         (v ? out.per_sm_ext : out.per_sm) = per_sm;
     }
     return cudaSuccess;

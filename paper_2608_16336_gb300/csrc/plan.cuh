@@ -179,4 +179,18 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
     return plan_loop(false);
 }
 
+// The blocks of a launch per SM, of the per_sm that fit, for `want` blocks' worth
+// of replicas.  With four instances per lane more than four blocks are taken only
+// for fewer waves: five instead of four 13.0 / 19.2 ms on 1,400 x 100 x 500 (one wave
+// instead of two), but 23.0 / 21.6 on 2,048 x 100 x 500 and 54.0 / 48.4 on 2,048 x 100 x
+// 3,000 (two waves either way).  With one or two per lane more blocks are never
+// slower: 3,000 x 32 x 800 with six and five 11.6 / 12.1.
+inline int blocks_at_once(int c, long long want, int sms_count, int per_sm) {
+    if (c != 4 || per_sm <= 4) return per_sm;
+    auto waves = [&](long long n) { return (want + n * sms_count - 1) / (n * sms_count); };
+    int n = 4;
+    while (waves(n) > waves(per_sm)) ++n;
+    return n;
+}
+
 }  // namespace mt

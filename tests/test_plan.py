@@ -30,6 +30,7 @@ extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_block
     }, p);
     return Res{f, p.c, p.sms, p.many, p.set_bits, (int)p.scratch, (long long)p.smem};
 }
+extern "C" int at_once(int c, long long want, int sms, int per_sm) { return blocks_at_once(c, want, sms, per_sm); }
 // shapes and replica counts whose scratch is too small; the last one in *at
 extern "C" int too_small(int N, int sms, int *at) {
     int bad = 0;
@@ -125,3 +126,12 @@ def test_main_loop(lib, n, k, replicas, many):
 def test_small_scratch_only_where_it_holds_more_blocks(lib, k, replicas, scratch):
     p = lib.plan(replicas, 64, k, 16, 64, 152, 0)
     assert p.many == 1 and p.scratch == scratch
+
+
+def test_blocks_at_once(lib):
+    """Four instances per lane: more than four blocks per SM only for fewer waves."""
+    for c in (1, 2, 8):
+        assert [lib.at_once(c, ctypes.c_longlong(1024), 152, n) for n in (1, 4, 6)] == [1, 4, 6]
+    for want, per_sm, n in ((608, 5, 4), (609, 5, 5), (760, 5, 5), (912, 6, 6), (761, 5, 4), (1216, 5, 4), (1217, 5, 5),
+                            (1217, 6, 5), (1521, 6, 6), (1, 6, 4), (5000, 3, 3)):
+        assert lib.at_once(4, ctypes.c_longlong(want), 152, per_sm) == n
