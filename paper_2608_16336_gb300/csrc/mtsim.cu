@@ -2716,9 +2716,12 @@ int sim_latency_stats(sim_t *s, sim_latency_stats_t *out, int on_device) {
     }
     // Replicas whose values fit in a block's shared memory (about 15,000 requests
     // with 4 tiers) take one kernel, larger ones the streaming passes.  One
-    // kernel / streaming, us: 1 replica x 64 requests 22 / 56, 1 x 14,000 75 / 95,
-    // 1,024 x 5,000 192 / 294, 1,024 x 14,000 473 / 528, 3,840 x 1,000 with 10
-    // tiers 441 / 792, 700 x 4,000 with 16 tiers 382 / 413.
+    // kernel / streaming, us back to back: 1 replica x 64 requests 17 / 45, 1 x 14,000
+    // 57 / 74, 1,024 x 5,000 161 / 240, 1,000 x 8,000 245 / 279, 3,840 x 1,000 with 10
+    // tiers 388 / 730, 700 x 4,000 with 16 tiers 231 / 370.  Slower are only the largest
+    // replicas just past a wave (153 x 15,900 122 / 111, 153 x 10,500 with 16 tiers 193
+    // / 167) and thousands of tiny replicas beside such a one (1 tier, 8,192 x 10 +
+    // 15,000 requests 305 / 222).
     long long qmax = 0;
     for (int r = 0; r < R; ++r) qmax = std::max<long long>(qmax, s->h_off[r + 1] - s->h_off[r]);
     bool done = false;

@@ -48,6 +48,13 @@ def test_largest(q, alike):
     compare(w, gpu_stats(w), [0])
 
 
+@pytest.mark.parametrize("q,k", [(8192, 4), (8191, 1), (4000, 16)])
+def test_one_block_per_sm(q, k):
+    """More replicas than SMs, each filling an SM's shared memory (or, with one tier, half of it)."""
+    w = _workload((q,) * 160, k, False, q)
+    compare(w, gpu_stats(w), [0, 80, 159])
+
+
 def test_unfinished_requests_left_out():
     w = _workload((700, 40), 3, False, 3)
     compare(w, gpu_stats(w, max_steps=150), range(2), max_steps=150)
