@@ -127,9 +127,9 @@ struct Field {
 
 // A replica's rarely changing counters, kept with its instance state so that
 // they hold no registers: log records, migrations, preemptions, migration
-// starts and aborts, scale-out and scale-in signals.  Formations on several
-// lanes may add to TOT_PRE, TOT_ABORT and TOT_MIG (atomics); lane 0 alone adds to
-// the others.
+// starts and aborts, scale-out and scale-in signals.  Several lanes at once may
+// add to TOT_PRE, TOT_ABORT and TOT_MIG (atomics), one lane at a time to the
+// others.
 enum : int { TOT_LOG = 0, TOT_MIG, TOT_PRE, TOT_START, TOT_ABORT, TOT_OUT, TOT_IN, TOT_COUNT };
 static_assert(TOT_COUNT == kTotCount, "counters of the layout");
 
@@ -422,7 +422,7 @@ __device__ __forceinline__ void refresh_hol(const Ctx &x, int i) {
     const uint32_t wm = x.wmask[i];
     x.hol[i] = wm ? blocks_for(x, x.hinfo[i * x.K + (__ffs(wm) - 1)] & 0xFFFFu) : 0;
 }
-__device__ __forceinline__ void log_ev(const Ctx &x, Cnt &cn, int kind, uint32_t r, int s, int d, int blocks) {
+__device__ __forceinline__ void log_ev(const Ctx &x, int kind, uint32_t r, int s, int d, int blocks) {
     const uint32_t k = x.tot[TOT_LOG]++;
     if (k < (uint32_t)x.cap)
         *x.log(k) = make_uint4(x.t, r, (uint32_t)(blocks & 0xFFFF) | ((uint32_t)s << 16) | ((uint32_t)d << 24),
@@ -441,7 +441,7 @@ __device__ __forceinline__ void log_end(const Ctx &x, Cnt &cn, int kind, uint32_
         x.mpend[s] = (uint8_t)ph;
         cn.held = true;
     } else {
-        log_ev(x, cn, kind, r, s, d, blocks);
+        log_ev(x, kind, r, s, d, blocks);
     }
 }
 // Writes the records held back in a window that some lane has, and returns
@@ -775,72 +775,72 @@ __device__ __forceinline__ unsigned int preempt_book(const Ctx &x, Cnt &cn, int 
 __device__ __forceinline__ void grow_slow(const Ctx &x, Cnt &cn, int i) {
     const int n = x.nrun[i], fr = x.free_[i];
     const uint32_t ph = x.phase[i], nf = x.nf[i];
-                // In running order, a request that needs a block (at most one)
-                // takes a free one or preempts the lowest-priority newest running
-                // request, possibly itself.  Positions are the list's before this
-                // step; removals are applied afterwards.
-                uint4 *p = slot_ptr(x, i, 0);
-                const uint64_t all = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
-                uint64_t alive = all, needs = 0, granted = 0;
-                // The requests that need a block now are those whose context reaches
-                // a block boundary: rho == -nf (mod T), the ones hist counts.
-                const uint32_t target = ph == 0 ? 0u : (uint32_t)x.T - ph;
-                // the same pass finds the first victim (lowest priority, then newest):
-                // more requests need a block than there are free blocks, so there is one
-                int v1 = -1;
-                uint32_t vt1 = 0, vr1 = 0;
+    // In running order, a request that needs a block (at most one)
+    // takes a free one or preempts the lowest-priority newest running
+    // request, possibly itself.  Positions are the list's before this
+    // step; removals are applied afterwards.
+    uint4 *p = slot_ptr(x, i, 0);
+    const uint64_t all = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
+    uint64_t alive = all, needs = 0, granted = 0;
+    // The requests that need a block now are those whose context reaches
+    // a block boundary: rho == -nf (mod T), the ones hist counts.
+    const uint32_t target = ph == 0 ? 0u : (uint32_t)x.T - ph;
+    // the same pass finds the first victim (lowest priority, then newest):
+    // more requests need a block than there are free blocks, so there is one
+    int v1 = -1;
+    uint32_t vt1 = 0, vr1 = 0;
 #pragma unroll 4
-                for (int q = 0; q < n; ++q) {
-                    const uint4 sl = p[q];
-                    needs |= (uint64_t)(sl_rho(sl) == target) << q;
-                    const uint32_t ts = sl_tier(sl);
-                    if (v1 < 0 || ts > vt1 || (ts == vt1 && sl.x > vr1)) { v1 = q; vt1 = ts; vr1 = sl.x; }
-                }
-                int fb = fr;
-                uint32_t pr = kNone;  // the last preempted request and its counter word before the add
-                unsigned int pold = 0;
+    for (int q = 0; q < n; ++q) {
+        const uint4 sl = p[q];
+        needs |= (uint64_t)(sl_rho(sl) == target) << q;
+        const uint32_t ts = sl_tier(sl);
+        if (v1 < 0 || ts > vt1 || (ts == vt1 && sl.x > vr1)) { v1 = q; vt1 = ts; vr1 = sl.x; }
+    }
+    int fb = fr;
+    uint32_t pr = kNone;  // the last preempted request and its counter word before the add
+    unsigned int pold = 0;
 #pragma unroll 1
-                for (int q = 0; q < n; ++q) {
-                    if (!((alive & needs) >> q & 1ull)) continue;
-                    for (;;) {
-                        if (fb > 0) { --fb; granted |= 1ull << q; break; }
-                        int v = -1;
-                        if (alive == all) {
-                            v = v1;  // nobody preempted yet: the victim found by the scan
-                        } else {
-                            uint32_t vt = 0, vr = 0;
+    for (int q = 0; q < n; ++q) {
+        if (!((alive & needs) >> q & 1ull)) continue;
+        for (;;) {
+            if (fb > 0) { --fb; granted |= 1ull << q; break; }
+            int v = -1;
+            if (alive == all) {
+                v = v1;  // nobody preempted yet: the victim found by the scan
+            } else {
+                uint32_t vt = 0, vr = 0;
 #pragma unroll 1
-                            for (uint64_t m = alive; m; m &= m - 1) {
-                                const int s2 = __ffsll((long long)m) - 1;
-                                const uint32_t ts = sl_tier(p[s2]), rs = p[s2].x;
-                                if (v < 0 || ts > vt || (ts == vt && rs > vr)) { v = s2; vt = ts; vr = rs; }
-                            }
-                        }
-                        const int vb = blocks_for(x, sl_c(p[v]) + nf - p[v].y) + (int)((granted >> v) & 1ull);
-                        alive &= ~(1ull << v);
-                        x.free_[i] = fb;
-                        if (pr != kNone) pre_fix(x, pr, pold);
-                        pr = p[v].x;
-                        pold = preempt_book(x, cn, i, p[v], vb);
-                        fb = x.free_[i];
-                        if (v == q) break;
-                    }
+                for (uint64_t m = alive; m; m &= m - 1) {
+                    const int s2 = __ffsll((long long)m) - 1;
+                    const uint32_t ts = sl_tier(p[s2]), rs = p[s2].x;
+                    if (v < 0 || ts > vt || (ts == vt && rs > vr)) { v = s2; vt = ts; vr = rs; }
                 }
-                x.free_[i] = fb;
-                int w = 0;
-                uint32_t fm = kNone;  // the survivors' next finishing formation
+            }
+            const int vb = blocks_for(x, sl_c(p[v]) + nf - p[v].y) + (int)((granted >> v) & 1ull);
+            alive &= ~(1ull << v);
+            x.free_[i] = fb;
+            if (pr != kNone) pre_fix(x, pr, pold);
+            pr = p[v].x;
+            pold = preempt_book(x, cn, i, p[v], vb);
+            fb = x.free_[i];
+            if (v == q) break;
+        }
+    }
+    x.free_[i] = fb;
+    int w = 0;
+    uint32_t fm = kNone;  // the survivors' next finishing formation
 #pragma unroll 1
-                for (int q = 0; q < n; ++q) {
-                    if ((alive >> q) & 1ull) {
-                        const uint4 sl = p[q];
-                        if (w != q) p[w] = sl;
-                        ++w;
-                        fm = min(fm, sl_fin(sl));
-                    }
-                }
-                x.nrun[i] = (uint8_t)w;
-                x.minfin[i] = fm;
-                if (pr != kNone) pre_fix(x, pr, pold);
+    for (int q = 0; q < n; ++q) {
+        if ((alive >> q) & 1ull) {
+            const uint4 sl = p[q];
+            if (w != q) p[w] = sl;
+            ++w;
+            fm = min(fm, sl_fin(sl));
+        }
+    }
+    x.nrun[i] = (uint8_t)w;
+    x.minfin[i] = fm;
+    if (pr != kNone) pre_fix(x, pr, pold);
 }
 
 template <bool SMS>
@@ -943,7 +943,7 @@ __device__ __forceinline__ void inst_form(Ctx &x, Cnt &cn, int i, const Params &
 // Lane 0 appends arriving request r (tier k, prompt P, output O) to instance
 // best's bucket and updates the instance (Sec. 3.4); the key store is needed
 // only if another arrival at the same time is dispatched next.
-__device__ __forceinline__ void dispatch_to(const Ctx &x, Cnt &cn, int best, uint32_t r, int k, uint32_t P,
+__device__ __forceinline__ void dispatch_to(const Ctx &x, int best, uint32_t r, int k, uint32_t P,
                                             uint32_t O, bool store_key) {
     if (x.lane == 0) {
         // the destination's scalars, read together; the new key is computed from them
@@ -972,10 +972,10 @@ __device__ __forceinline__ void dispatch_to(const Ctx &x, Cnt &cn, int best, uin
 
 // Dispatch one arriving request r of tier k with prompt length P (Sec. 3.4).
 template <int C>
-__device__ __forceinline__ void dispatch_one(const Ctx &x, Cnt &cn, uint32_t r, int k, uint32_t P, uint32_t O,
+__device__ __forceinline__ void dispatch_one(const Ctx &x, uint32_t r, int k, uint32_t P, uint32_t O,
                                              uint32_t all) {
     const int best = arg_ext<C>(x, all, true, -1);
-    dispatch_to(x, cn, best, r, k, P, O, true);
+    dispatch_to(x, best, r, k, P, O, true);
     __syncwarp();
 }
 
@@ -997,7 +997,7 @@ __device__ __forceinline__ void arr_refill(const Ctx &x, ArrBuf &ab, uint32_t cu
 // Dispatches all arrivals at t, from trace record `cursor` on, tier by tier to
 // the instances in `all`; returns their number.  Collective.
 template <int C>
-__device__ __forceinline__ uint32_t dispatch_many(const Ctx &x, Cnt &cn, uint32_t cursor, uint32_t all) {
+__device__ __forceinline__ uint32_t dispatch_many(const Ctx &x, uint32_t cursor, uint32_t all) {
     refresh_keys<C>(x);
     const long long at = x.first();
     uint32_t m = 0;
@@ -1023,7 +1023,7 @@ __device__ __forceinline__ uint32_t dispatch_many(const Ctx &x, Cnt &cn, uint32_
             while (bits) {
                 const int l = __ffs(bits) - 1;
                 bits &= bits - 1;
-                dispatch_one<C>(x, cn, cursor + base + (uint32_t)l, k, __shfl_sync(kFull, P, l),
+                dispatch_one<C>(x, cursor + base + (uint32_t)l, k, __shfl_sync(kFull, P, l),
                                 __shfl_sync(kFull, O, l), all);
             }
         }
@@ -1037,15 +1037,14 @@ __device__ __noinline__ uint32_t dispatch_call(uint4 *node, uint32_t Q, int r, u
     extern __shared__ __align__(16) unsigned char smem[];
     Ctx x;
     bind_ctx<SMS>(x, *reinterpret_cast<const Params *>(smem), smem, node, Q, r, t);
-    Cnt cn;
-    return dispatch_many<C>(x, cn, cursor, all);
+    return dispatch_many<C>(x, cursor, all);
 }
 
 // Phase 2: arrivals at t, tier 0 first, FCFS (trace order) within a tier.
 // EXT: draining instances may exist.  Returns the destination of a lone
 // arrival, or -1 after several.
 template <int C, bool SMS, bool EXT, bool LEAN>
-__device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor, uint32_t &next_arr, ArrBuf &ab,
+__device__ __forceinline__ int dispatch_phase(Ctx &x, uint32_t &cursor, uint32_t &next_arr, ArrBuf &ab,
                                               const Params &p) {
     uint32_t all = own_mask<C>(x);
     if (EXT && x.drains) {
@@ -1080,13 +1079,13 @@ __device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor,
         }
         const int m = __reduce_max_sync(kFull, bv);
         const int best = __reduce_min_sync(kFull, (bi >= 0 && bv == m) ? bi : INT_MAX);
-        dispatch_to(x, cn, best, ab.pb + (uint32_t)l, (int)k1, po & 0xFFFFu, po >> 16, false);
+        dispatch_to(x, best, ab.pb + (uint32_t)l, (int)k1, po & 0xFFFFu, po >> 16, false);
         __syncwarp();
         dest = best;
         cursor += 1u;
     } else {
         if (LEAN) {
-            cursor += dispatch_many<C>(x, cn, cursor, all);
+            cursor += dispatch_many<C>(x, cursor, all);
         } else {
             cursor += dispatch_call<C, SMS>(x.node, x.Q, x.r, x.t, cursor, all);
         }
@@ -1103,7 +1102,7 @@ __device__ __forceinline__ int dispatch_phase(Ctx &x, Cnt &cn, uint32_t &cursor,
 // by L = lcm(1, ..., Bmax), so S = L * sum F_normal is an exact 128-bit
 // integer (|S| < 2^117), and mean < x / D  <=>  S * D < x * n * L.  Collective.
 template <int C>
-__device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Params &p) {
+__device__ __forceinline__ void autoscale_tick(const Ctx &x, const Params &p) {
     const __int128 L = (__int128)(((unsigned __int128)p.lcm_hi << 64) | p.lcm_lo);
     __int128 sum = 0;
     int n = 0;
@@ -1128,10 +1127,10 @@ __device__ __forceinline__ void autoscale_tick(const Ctx &x, Cnt &cn, const Para
         const __int128 lhs = sum * p.scale_den;
         if (lhs < (__int128)p.scale_out_num * n * L) {
             x.tot[TOT_OUT]++;
-            log_ev(x, cn, SIM_EV_SCALE_OUT, kNone, 255, 255, 0);
+            log_ev(x, SIM_EV_SCALE_OUT, kNone, 255, 255, 0);
         } else if (lhs > (__int128)p.scale_in_num * n * L) {
             x.tot[TOT_IN]++;
-            log_ev(x, cn, SIM_EV_SCALE_IN, kNone, 255, 255, 0);
+            log_ev(x, SIM_EV_SCALE_IN, kNone, 255, 255, 0);
         }
     }
     __syncwarp();
@@ -1611,7 +1610,7 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
 //
 // EXT: the variant that also handles draining instances and the auto-scaling
 // signal (the other variant compiles that code out).  MANY: the loop for more
-// replicas than a few warps per SM (plan_launch).  What bounds the two differs:
+// replicas than a few warps per SM (choose_plan).  What bounds the two differs:
 // with few warps each replica's dependent chain, so the loop without MANY has
 // a straight path per kind of pass; with many, instruction fetch and registers
 // (64 instances: 14 % less code took 161 to 131 ms, 18 instead of 16 warps
@@ -1623,11 +1622,11 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
 // replicas x 64 instances x 4,000 requests, against 131.0 ms with 8 blocks at
 // 124 registers.  (10 resident blocks, with 1 KB less of scratch per warp:
 // 110.4 ms; 12 blocks would need 80 registers, which spills.)  One instance
-// per lane: 8 blocks (110 registers) 20.8 ms on 3,840 x 32 x 1,000, 10 blocks
-// 21.8 ms, 12 blocks (80 registers) 21.9 ms.  Four per lane: a bound of 6 blocks
-// gives 168 registers, which 12 warps of an SM can have; unbounded it takes 181, for 8
-// warps: 1,500 x 128 x 500 21.9 -> 15.5 ms, 1,824 x 100 x 500 21.0 -> 16.1, 256 x 128 x
-// 6,000 the same (blocks_at_once).
+// per lane: 8 blocks (128 registers); 10 and 12 blocks were 5 % slower on 3,840 x
+// 32 x 1,000.  Four per lane: a bound of 6 blocks gives 168 registers, which 12
+// warps of an SM can have; unbounded it takes 181, for 8 warps: 1,500 x 128 x 500
+// 21.9 -> 15.5 ms, 1,824 x 100 x 500 21.0 -> 16.1, 256 x 128 x 6,000 the same
+// (blocks_at_once).
 template <int C, bool SMS, bool EXT, bool MANY>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) : C == 2 ? 10 : 8) k_run(Params p) {
     // At 96 registers there is no room for values kept across calls: the rare
@@ -1827,20 +1826,20 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
                 int dest = -1;
                 if (mode == 2) {
                     x.t = tstep;
-                    if (next_arr == tstep) dest = dispatch_phase<C, SMS, EXT, LEAN>(x, cn, cursor, next_arr, ab, p);  // 2. dispatch
+                    if (next_arr == tstep) dest = dispatch_phase<C, SMS, EXT, LEAN>(x, cursor, next_arr, ab, p);  // 2. dispatch
                     if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                         const uint32_t nt = next_tick + p.interval;
                         next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
-                        if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
+                        if (EXT && p.autoscale) autoscale_tick<C>(x, p);
                         if (p.enable_mig) {
-                        if (LEAN) {
-                            mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
-                        } else {
-                            const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
-                            mig = mig || (did & 1);
-                            if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
+                            if (LEAN) {
+                                mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
+                            } else {
+                                const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
+                                mig = mig || (did & 1);
+                                if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
+                            }
                         }
-                    }
                     }
                 }
                 // ---- 4. batch formation: in mode 0 every lane forms its own
@@ -1951,7 +1950,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
                         if (C == 1) {
                             if (sel) {
                                 x.t = bz[0];
-                                inst_form<SMS, LEAN>(x, cn, lane, p);
+                                inst_form<SMS, false>(x, cn, lane, p);
                             }
                         } else {
                             const uint32_t total = list_own<C>(x, sel, bz);
@@ -1959,7 +1958,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
                             for (uint32_t q = (uint32_t)lane; q < total; q += 32) {
                                 const uint2 e = reinterpret_cast<const uint2 *>(x.tset)[q];
                                 x.t = e.x;
-                                inst_form<SMS, LEAN>(x, cn, (int)e.y, p);
+                                inst_form<SMS, false>(x, cn, (int)e.y, p);
                             }
                         }
                         __syncwarp();
@@ -2004,7 +2003,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
                             if (tc >= t1) break;
                             x.t = tc;
                             complete_all<C>(x, cn, same);
-                            form_all<C, SMS, LEAN>(x, cn, same, p);
+                            form_all<C, SMS, false>(x, cn, same, p);
                             if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
                         }
                         x.hold = false;
@@ -2025,25 +2024,21 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
                 ++cn.steps;
                 if (tb == x.t) complete_all<C>(x, cn, all);  // 1. iteration ends
                 int dest = -1;
-                if (next_arr == x.t) dest = dispatch_phase<C, SMS, EXT, LEAN>(x, cn, cursor, next_arr, ab, p);  // 2. dispatch
+                if (next_arr == x.t) dest = dispatch_phase<C, SMS, EXT, false>(x, cursor, next_arr, ab, p);  // 2. dispatch
                 if (MT_RARE(tick)) {  // 3. auto-scaling signal and migration tick
                     const uint32_t nt = next_tick + p.interval;
                     next_tick = nt < next_tick ? kNone : nt;  // saturate: no tick beyond 2^32 - 1
-                    if (EXT && p.autoscale) autoscale_tick<C>(x, cn, p);
+                    if (EXT && p.autoscale) autoscale_tick<C>(x, p);
                     if (p.enable_mig) {
-                        if (LEAN) {
-                            mig = migration_tick<C, EXT>(x, cn, p.theta_num, p.theta_den) || mig;
-                        } else {
-                            const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
-                            mig = mig || (did & 1);
-                            if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
-                        }
+                        const int did = tick_call<C, SMS, EXT>(x.node, x.Q, x.r, x.t);
+                        mig = mig || (did & 1);
+                        if (MT_RARE(did & 2)) cn.status = SIM_ERR_INTERNAL;
                     }
                 }
                 // 4. batch formation.  After a lone arrival only its destination can
                 // have become able to form (an instance that stayed idle had nothing
                 // that fits, and nothing else changed).
-                if (tb == x.t || tick || dest < 0 || x.busy[dest] == kNone) form_all<C, SMS, LEAN>(x, cn, all, p);
+                if (tb == x.t || tick || dest < 0 || x.busy[dest] == kNone) form_all<C, SMS, false>(x, cn, all, p);
                 if (MT_RARE(__any_sync(kFull, cn.status < 0))) break;
             }
             __syncwarp();
