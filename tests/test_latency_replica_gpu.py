@@ -1,7 +1,8 @@
 """Latency statistics at the edges of the one-kernel path (replicas of 0 to
 16,383 requests, the block sizes it changes at, ragged warps, the tier counts
-whose shared memory differs, all values alike) and just past it, bit-exact
-against sorted values."""
+whose shared memory differs, all values alike, the largest replicas its shared
+memory holds) and past it, where the streaming passes take replicas of any size
+together, bit-exact against sorted values."""
 import threading
 
 import numpy as np
@@ -53,6 +54,33 @@ def test_one_block_per_sm(q, k):
     """More replicas than SMs, each filling an SM's shared memory (or, with one tier, half of it)."""
     w = _workload((q,) * 160, k, False, q)
     compare(w, gpu_stats(w), [0, 80, 159])
+
+
+@pytest.mark.parametrize("q,k", [(16064, 4), (16065, 4), (10608, 16), (10609, 16)])
+def test_shared_memory_limit(q, k):
+    """The largest replica that a block's 227 KB holds, and one request more."""
+    w = _workload((q, 7), k, False, q)
+    compare(w, gpu_stats(w), range(2))
+
+
+@pytest.mark.parametrize("max_steps", [None, 4000])
+@pytest.mark.parametrize("k", [1, 16])
+def test_streaming_mixed_sizes(k, max_steps):
+    """Empty and tiny replicas beside large ones, finished or stopped early, to host and device."""
+    import torch
+    w = _workload((0, 17000, 3, 4096, 0, 16500, 4097), k, False, 5 + k)
+    sim = mtsim.Simulator(w, event_log_capacity=0)
+    try:
+        sim.load()
+        sim.run() if max_steps is None else sim.run(max_steps)
+        host = sim.latency_stats()
+        d = torch.empty(host.nbytes, dtype=torch.uint8, device="cuda")
+        mtsim.sim_latency_stats(sim.handle, d.data_ptr(), 1)
+        torch.cuda.synchronize()
+    finally:
+        sim.close()
+    assert d.cpu().numpy().tobytes() == host.tobytes()
+    compare(w, host, range(w.num_replicas), **({} if max_steps is None else dict(max_steps=max_steps)))
 
 
 def test_unfinished_requests_left_out():
