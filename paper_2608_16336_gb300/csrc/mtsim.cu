@@ -1623,12 +1623,11 @@ __device__ __forceinline__ uint32_t run_quiet(const Ctx &x, Cnt &cn, uint32_t &b
 // 124 registers.  (10 resident blocks, with 1 KB less of scratch per warp:
 // 110.4 ms; 12 blocks would need 80 registers, which spills.)  One instance
 // per lane: 8 blocks (128 registers); 10 and 12 blocks were 5 % slower on 3,840 x
-// 32 x 1,000.  Four per lane: a bound of 6 blocks gives 168 registers, which 12
-// warps of an SM can have; unbounded it takes 181, for 8 warps: 1,500 x 128 x 500
-// 21.9 -> 15.5 ms, 1,824 x 100 x 500 21.0 -> 16.1, 256 x 128 x 6,000 the same
-// (blocks_at_once).
+// 32 x 1,000.  Four per lane, records in HBM: the loop of few takes 181 registers
+// (8 warps per SM); MANY is the same loop at a bound of 6 blocks (168 registers, 12
+// warps), for the replica counts that take fewer waves then (choose_plan).
 template <int C, bool SMS, bool EXT, bool MANY>
-__global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) : C == 2 ? 10 : 8) k_run(Params p) {
+__global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? 4 : C == 4 ? 6 : C == 2 ? 10 : 8) k_run(Params p) {
     // At 96 registers there is no room for values kept across calls: the rare
     // paths stay inline (116 ms instead of 196 on the 64-instance sweep), and
     // copy stages go source by source.
@@ -1686,7 +1685,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, !MANY ? (C == 4 ? 6 : 4) 
         ArrBuf ab;
         arr_refill(x, ab, cursor);
         uint32_t next_arr = __shfl_sync(kFull, ab.time, 0);
-        if constexpr (MANY) {
+        if constexpr (MANY && C <= 2) {
             const uint32_t max_steps = p.max_steps;
             const uint32_t all = own_mask<C>(x);
             const bool ticks = EXT ? p.ticks != 0 : p.enable_mig != 0;
@@ -2221,7 +2220,7 @@ typedef void (*RunKernel)(Params);
 template <bool EXT>
 RunKernel pick(int c, bool sms, bool many) {  // c = instances per lane
     if (many && sms) return k_run<1, true, EXT, true>;
-    if (many) return c == 1 ? k_run<1, false, EXT, true> : k_run<2, false, EXT, true>;
+    if (many) return c == 1 ? k_run<1, false, EXT, true> : c == 2 ? k_run<2, false, EXT, true> : k_run<4, false, EXT, true>;
     switch (c) {
         case 1: return sms ? k_run<1, true, EXT, false> : k_run<1, false, EXT, false>;
         case 2: return sms ? k_run<2, true, EXT, false> : k_run<2, false, EXT, false>;
@@ -2276,8 +2275,7 @@ inline cudaError_t plan_launch(int R, int N, int Bmax, const Layout &L, Launch &
         const int per_sm = resident(v ? out.fn_ext : out.fn, out.smem);
         if (per_sm < 0) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        (v ? out.grid_ext : out.grid) =
-            (int)std::min<long long>(want, (long long)sms_count * blocks_at_once(out.c, want, sms_count, per_sm));
+        (v ? out.grid_ext : out.grid) = (int)std::min<long long>(want, (long long)sms_count * per_sm);
         (v ? out.per_sm_ext : out.per_sm) = per_sm;
     }
     return cudaSuccess;

@@ -84,7 +84,7 @@ inline uint32_t scratch_need(int N) {
 struct Plan {
     int c = 1;         // instances per lane
     bool sms = false;  // running-request records in shared memory
-    bool many = false; // the loop of many replicas
+    bool many = false; // the variant for many replicas
     int set_bits = 0;  // the part of the scratch that counts event times, log2 of its bytes
     uint32_t scratch = 0;  // scratch of a warp, bytes
     size_t smem = 0;   // dynamic shared memory of a block
@@ -130,7 +130,7 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
     auto plan_loop = [&](bool many) {
         out.many = many;
         if (out.c == 1) return with_bits(0);
-        if (many) {
+        if (many && out.c == 2) {
             const int n = with_bits(kSetBits);
             if (n < 0 || R <= 26 * sms_count) return n;
             const int n2 = with_bits(kSetBitsMany);
@@ -144,18 +144,18 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
         }
         return with_bits(bits);
     };
-    // Which main loop (see k_run), up to 64 instances.
+    // Which main loop (see k_run).
     if (out.c == 1 && sms) {
         // Records in shared memory: both loops have about the same residency, and the
         // loop of many scales better with the warps that share an SM's instruction
         // cache, the sooner the fewer instances share a window.  Loop of few / of many,
         // ms, at 0.85 load: 4 instances, 912 replicas 16.3 / 17.0, 1,216 19.3 / 17.2; 8,
-        // 912 13.5 / 14.5, 1,216 15.9 / 14.7; 12, 1,216 9.2 / 9.8, 1,368 10.3 / 10.3; 16,
+        // 912 13.5 / 14.5, 1,216 15.9 / 14.7; 12, 1,216 9.2 / 9.8, 1,520 10.8 / 10.3; 16,
         // 1,216 16.5 / 17.2, 1,520 19.7 / 18.4 (800 requests 5.4 / 6.1, 8,000 41.5 / 35.7);
         // one instance, 1,520 6.7 / 7.7.  At 0.3 to 0.4 load the lines lie about 1
         // replica per SM higher.  Only where at least 5 blocks fit (6,000 x 24 x 400,
         // 3 blocks: 24.4 / 27.7).
-        const int per_sm = N == 1 ? 12 : N <= 8 ? 7 : 9;
+        const int per_sm = N == 1 ? 12 : N <= 8 ? 7 : 10;
         if (R > per_sm * sms_count) {
             const int n = plan_loop(true);
             if (n < 0 || n >= 5) return n;
@@ -176,21 +176,14 @@ int choose_plan(int R, int N, int Bmax, const Layout &L, int sms_count, size_t m
         if (many < 0) return many;
         if (waves(few) > 3 ? many >= 6 : (out.c == 1 ? 11 : 14) * waves(many) < 10 * waves(few)) return many;
     }
-    return plan_loop(false);
-}
-
-// The blocks of a launch per SM, of the per_sm that fit, for `want` blocks' worth
-// of replicas.  With four instances per lane more than four blocks are taken only
-// for fewer waves: five instead of four 13.0 / 19.2 ms on 1,400 x 100 x 500 (one wave
-// instead of two), but 23.0 / 21.6 on 2,048 x 100 x 500 and 54.0 / 48.4 on 2,048 x 100 x
-// 3,000 (two waves either way).  With one or two per lane more blocks are never
-// slower: 3,000 x 32 x 800 with six and five 11.6 / 12.1.
-inline int blocks_at_once(int c, long long want, int sms_count, int per_sm) {
-    if (c != 4 || per_sm <= 4) return per_sm;
-    auto waves = [&](long long n) { return (want + n * sms_count - 1) / (n * sms_count); };
-    int n = 4;
-    while (waves(n) > waves(per_sm)) ++n;
-    return n;
+    const int few = plan_loop(false);
+    if (few < 0 || out.c != 4 || sms || waves(few) == 1) return few;
+    // Four instances per lane, records in HBM: the same loop with 12 warps per SM
+    // instead of 8 where that saves a wave.  8 / 12 warps, ms: 1,500 x 128 x 500 21.9 /
+    // 15.5, 1,824 x 100 x 500 21.0 / 16.1, 4,096 x 100 44.7 / 41.2; 2,048 x 100 x 3,000,
+    // two waves either way, 48.4 / 54.0; 2 x 74 x 1,279 14.8 / 15.3.
+    const int many = plan_loop(true);
+    return many < 0 || waves(many) < waves(few) ? many : plan_loop(false);
 }
 
 }  // namespace mt

@@ -25,12 +25,11 @@ extern "C" Res plan(int R, int N, int K, int T, int Bmax, int sms, int reg_block
     Plan p;
     const int f = choose_plan(R, N, Bmax, make_layout(N, K, T), sms, 232448, [&](const Plan &q) {
         const int n = q.smem > 232448 ? -1 : (int)(233472 / (q.smem + 1024));
-        const int regs = reg_blocks > 0 ? reg_blocks : !q.many ? (q.c <= 2 ? 6 : 4) : q.c == 2 ? 10 : 8;
+        const int regs = reg_blocks > 0 ? reg_blocks : !q.many ? (q.c <= 2 ? 6 : 4) : q.c == 1 ? 8 : q.c == 2 ? 10 : 6;
         return n < regs ? n : regs;
     }, p);
     return Res{f, p.c, p.sms, p.many, p.set_bits, (int)p.scratch, (long long)p.smem};
 }
-extern "C" int at_once(int c, long long want, int sms, int per_sm) { return blocks_at_once(c, want, sms, per_sm); }
 // shapes and replica counts whose scratch is too small; the last one in *at
 extern "C" int too_small(int N, int sms, int *at) {
     int bad = 0;
@@ -112,10 +111,11 @@ def test_one_instance_per_lane_keeps_its_residency(lib):
 @pytest.mark.parametrize("n,k,replicas,many", [
     (64, 4, 1824, 0), (64, 4, 1825, 1), (64, 4, 2736, 1), (64, 4, 2737, 0), (64, 4, 3648, 0), (64, 4, 3649, 1),
     (64, 4, 8192, 1), (64, 10, 16384, 1), (64, 16, 1520, 0), (64, 16, 2432, 0), (64, 16, 16384, 0), (40, 4, 1825, 1), (32, 4, 1824, 0), (32, 4, 1825, 1),
-    (32, 4, 2433, 0), (32, 10, 3840, 1), (1, 4, 1824, 0), (8, 4, 1064, 0), (8, 4, 1065, 1), (16, 4, 1368, 0),
-    (16, 4, 1369, 1), (24, 4, 8192, 0), (65, 4, 8192, 0)])
+    (32, 4, 2433, 0), (32, 10, 3840, 1), (1, 4, 1824, 0), (8, 4, 1064, 0), (8, 4, 1065, 1), (16, 4, 1520, 0),
+    (16, 4, 1521, 1), (24, 4, 8192, 0), (100, 4, 1216, 0), (100, 4, 1217, 1), (100, 4, 1520, 1), (100, 4, 1824, 1),
+    (100, 4, 2048, 0), (100, 4, 2433, 1), (128, 10, 8192, 0), (129, 4, 8192, 0)])
 def test_main_loop(lib, n, k, replicas, many):
-    """The loop whose waves take less time, on either side of the replica counts that
+    """The variant whose waves take less time, on either side of the replica counts that
     fill a wave of 152 SMs; with records in shared memory, of the lines drawn there."""
     p = lib.plan(replicas, n, k, 16, 64, 152, 0)
     assert p.many == many
@@ -127,11 +127,3 @@ def test_small_scratch_only_where_it_holds_more_blocks(lib, k, replicas, scratch
     p = lib.plan(replicas, 64, k, 16, 64, 152, 0)
     assert p.many == 1 and p.scratch == scratch
 
-
-def test_blocks_at_once(lib):
-    """Four instances per lane: more than four blocks per SM only for fewer waves."""
-    for c in (1, 2, 8):
-        assert [lib.at_once(c, ctypes.c_longlong(1024), 152, n) for n in (1, 4, 6)] == [1, 4, 6]
-    for want, per_sm, n in ((608, 5, 4), (609, 5, 5), (760, 5, 5), (912, 6, 6), (761, 5, 4), (1216, 5, 4), (1217, 5, 5),
-                            (1217, 6, 5), (1521, 6, 6), (1, 6, 4), (5000, 3, 3)):
-        assert lib.at_once(4, ctypes.c_longlong(want), 152, per_sm) == n

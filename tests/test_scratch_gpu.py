@@ -88,8 +88,8 @@ def test_live_objects(first, second):
             s.close()
 
 
-@pytest.mark.parametrize("n,k,replicas", [(2, 2, 1064), (2, 2, 1065), (16, 4, 1369), (32, 4, 1825), (32, 4, 2433),
-                                          (40, 4, 1825), (64, 4, 2737), (64, 4, 3648), (64, 16, 2432)])
+@pytest.mark.parametrize("n,k,replicas", [(2, 2, 1064), (2, 2, 1065), (16, 4, 1521), (32, 4, 1825), (32, 4, 2433),
+                                          (40, 4, 1825), (64, 4, 2737), (64, 4, 3648), (64, 16, 2432), (100, 4, 1400), (100, 4, 2048)])
 def test_loop_edges(n, k, replicas):
     """Replica counts on either side of the choice between the two main loops on 152 SMs."""
     w = _workload(n, k, replicas)
